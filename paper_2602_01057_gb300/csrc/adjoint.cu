@@ -1,0 +1,795 @@
+// Adjoint of the parallel-ray geometries (a5): CT parallel beam and the PET
+// ring with or without time of flight, dL/dI back to the Gaussians'
+// (mu, rho, G_P, G_S).  (Cone beam and 3-D PET: adjoint_tile.cu.)
+//
+// Gaussian-stationary: a warp takes up to 32 Gaussians that lie close together in
+// space (launch_order) and, with the CTA's other warps,
+// a range of views.  Per view
+//  * lane k turns record k into its view-space form (shared memory) and reads
+//    its pixel box (k_cull's rectangle); the CTA stages the rectangle of dL/dI
+//    that holds all its boxes, in bands when it is larger than the buffer;
+//  * sub-warps of S = 2^LG lanes take the Gaussians in turn, a lane walking
+//    every S-th row of the box along the footprint's chord,
+//    two pixels at a time in packed binary32, and reduce the view-space
+//    moments across the sub-warp;
+//  * lane k chains Gaussian k's moments (view_chain) into the world-space
+//    gradient that it keeps over the CTA's views.
+// No tile lists, no per-tile atomics: one set of 16 sums per Gaussian and view
+// range, added to the accumulator at the end.
+//
+// Bound by instruction issue (the pixels of the chords, their set-up, and the
+// lanes that wait for a longer chord of the same round).  Against one Gaussian
+// per thread and tile (record gathers, box searches, a chain and 16 atomics
+// for each of the 1.9 tiles of a PET footprint), measured on a GB300: PET ring
+// of 288 x 329 x 63, 200,000 Gaussians 9.6 -> 6.9 ms; 8 raw angles, 100,000
+// 0.73 -> 0.15 ms; 24 angles x 13 time-of-flight bins 4.96 -> 3.7 ms; parallel
+// beam, 1,000 Gaussians on 16 x 64^2 0.34 -> 0.11 ms (that one had 256 CTAs of
+// serial pixels).  Sorting a warp's Gaussians by box area per view took the
+// ring from 8.0 to 6.9 ms: a round's lanes then have chords of like length.
+#include <type_traits>
+
+#include "view.cuh"
+
+namespace rgrt {
+namespace {
+
+constexpr int BS = 128;
+constexpr int NW = BS / 32;
+template <bool TOF> struct Wide { static constexpr int v = TOF ? 256 : 512; };   // widest band (columns)
+constexpr int BH = 256;         // highest band (rows)
+
+// shared floats of the staged band
+template <bool TOF> struct Cap { static constexpr int v = TOF ? 5120 : 4096; };
+
+// ---- packed pairs of binary32 -------------------------------------------
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk(float a, float b)
+{
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void up(f2 x, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x));
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c)
+{
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b)
+{
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b)
+{
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ float hadd(f2 x)
+{
+    float a, b;
+    up(x, a, b);
+    return a + b;
+}
+
+// factors of the moments' derivatives: with h = dL/dI times the kernel's
+// profile and p = h arg,  -dL/dQ = A^-3/2 FQ h  and  dL/dA = A^-3/2 (FP p -
+// h / 2)  per unit alpha
+template <int KER> struct Fac;
+template <> struct Fac<0> {
+    static constexpr float FQ = 0.5f, FP = 0.5f * M_PER_ARG;
+};
+template <> struct Fac<1> {
+    static constexpr float FQ = 1.5f / 7.0f, FP = -2.0f;
+};
+
+// the kernel's profile of a pair: e^{-m/2} inside the cut (Gaussian), sqrt(c)
+// inside the support (Epanechnikov, c = 1 + arg)
+template <int KER>
+__device__ __forceinline__ float profile(float arg)
+{
+    if (KER == 1) {
+        const float c = 1.0f + arg;
+        return c > 0.0f ? sqrt_approx(c) : 0.0f;
+    }
+    return arg >= CUT_ARG ? ex2_approx(arg) : 0.0f;
+}
+
+struct Box {
+    int ilo, ihi, jlo, jhi;
+};
+
+// a staged band: columns [cb, cb + w), rows [rb, rb + h), row stride st
+struct Band {
+    int cb, rb, w, h, st;
+};
+
+// cut of the chords: a little outside the pairs' own, so that rounding in the
+// roots loses no pixel (the chord is widened by 0.05 columns as well)
+template <int KER>
+__device__ __forceinline__ float chord_cut()
+{
+    return KER == 1 ? -1.0f - 2e-4f : CUT_ARG * (1.0f + 2e-4f);
+}
+
+// columns [lo, hi] cut down to the chord al du^2 + be du + ga >= 0 (al < 0),
+// xc = the column coordinate of du = 0, iv = columns per unit
+__device__ __forceinline__ void chord(float al, float be, float ga, float xc, float iv, int &lo, int &hi)
+{
+    const float D = fmaf(be, be, -4.0f * al * ga);
+    const float sq = sqrt_approx(fmaxf(D, 0.0f)), i2a = __fdividef(0.5f * iv, al);
+    const float a = fmaf(sq - be, i2a, xc - 0.05f), b = fmaf(-be - sq, i2a, xc + 0.05f);   // a <= b
+    lo = max(lo, (int)ceilf(fmaxf(a, -1.0f)));
+    hi = D < 0.0f ? -1 : min(hi, (int)floorf(fminf(b, 65536.0f)));
+}
+
+// Moments of one Gaussian over the lane's share of its box within the band:
+// rows jlo + r0, + dr, ..., in each the chord of the footprint (every pixel is
+// still tested), two columns at a time.  With h = dL/dI times the kernel's
+// profile and p = h arg,
+//   m[0..5] = sum h {1, du, dv, du^2, du dv, dv^2},  m[6] = sum p;
+// A is constant along parallel rays, its powers are left to finish().
+template <int KER>
+__device__ __forceinline__ void rows(const DevGeom &g, const float4 &c0, const float4 &c1, const Box &bx, int r0,
+                                     int dr, const Band &bd, const float *sg, const float *su, const float *sv,
+                                     float *m)
+{
+    const float u0 = c0.x, v0 = c0.y, kMuv2 = c0.w, kMvv = c1.x, thr = chord_cut<KER>();
+    const int ilo = max(bx.ilo - bd.cb, 0), ihi = min(bx.ihi - bd.cb, bd.w - 1);
+    const float xc = (u0 - g.u0) * g.uinv - (float)bd.cb;
+    int j = bx.jlo - bd.rb + r0;
+    if (j < 0) j += (-j + dr - 1) / dr * dr;
+    const int je = min(bx.jhi - bd.rb, bd.h - 1);
+    const f2 nu0 = pk(-u0, -u0), Muu = pk(c0.z, c0.z);
+#pragma unroll
+    for (int q = 0; q < 7; q++) m[q] = 0.0f;
+    for (; j <= je; j += dr) {
+        const float dv = sv[j] - v0, dv2 = dv * dv;
+        const float a1 = kMuv2 * dv, a0 = kMvv * dv2;
+        const f2 A1 = pk(a1, a1), A0 = pk(a0, a0);
+        int ia = ilo, ie = ihi;
+        if (g.uinv != 0.0f && c0.z < 0.0f) chord(c0.z, a1, a0 - thr, xc, g.uinv, ia, ie);
+        const float *gr = sg + j * bd.st;
+        f2 h0 = 0, h1 = 0, h2 = 0, q0 = 0;
+#pragma unroll 1
+        for (int i = ia & ~1; i <= ie; i += 2) {
+            const float2 uu = *reinterpret_cast<const float2 *>(su + i), gg = *reinterpret_cast<const float2 *>(gr + i);
+            const f2 du = add2(pk(uu.x, uu.y), nu0);
+            const f2 q = fma2(fma2(Muu, du, A1), du, A0);
+            float qx, qy;
+            up(q, qx, qy);
+            const f2 h = mul2(pk(gg.x, gg.y), pk(profile<KER>(qx), profile<KER>(qy)));
+            const f2 hd = mul2(h, du);
+            h0 = add2(h0, h);
+            h1 = add2(h1, hd);
+            h2 = fma2(hd, du, h2);
+            q0 = fma2(h, q, q0);
+        }
+        const float s0 = hadd(h0), s1 = hadd(h1);
+        m[0] += s0;
+        m[1] += s1;
+        m[2] = fmaf(s0, dv, m[2]);
+        m[3] += hadd(h2);
+        m[4] = fmaf(s1, dv, m[4]);
+        m[5] = fmaf(s0, dv2, m[5]);
+        m[6] += hadd(q0);
+    }
+}
+
+// The same with time of flight (parallel rays, one pixel at a time): a pair's
+// value times the bin's weight W_k = N(t* - t_k; 0, s^2), s^2 = 1/A +
+// sigma_T^2.  h carries G = sum_k g_k W_k in place of dL/dI, and four more
+// sums the weights' own gradients: m[7..10] = val dW/dt* (1, du, dv) and
+// val dW/ds^2.
+__device__ __forceinline__ void rows_tof(const DevGeom &g, const float4 &c0, const float4 &c1, const float4 &t4,
+                                         const Box &bx, int r0, int dr, const Band &bd, const float *sg,
+                                         const float *su, const float *sv, float *m)
+{
+    const float u0 = c0.x, v0 = c0.y;
+    const int ilo = max(bx.ilo - bd.cb, 0), ihi = min(bx.ihi - bd.cb, bd.w - 1);
+    const float xc = (u0 - g.u0) * g.uinv - (float)bd.cb;
+    int j = bx.jlo - bd.rb + r0;
+    if (j < 0) j += (-j + dr - 1) / dr * dr;
+    const int je = min(bx.jhi - bd.rb, bd.h - 1);
+    const float s2 = t4.w + g.tof_s2, is2 = 1.0f / s2, ns = Kern<0>::QSCALE * is2;
+    const float nrm = rsqrtf(2.0f * 3.14159265358979324f / is2);
+    const int plane = bd.h * bd.st;
+#pragma unroll
+    for (int q = 0; q < 11; q++) m[q] = 0.0f;
+    const f2 NS = pk(ns, ns);
+    for (; j <= je; j += dr) {
+        const float dv = sv[j] - v0;
+        const float dv2 = dv * dv, a1 = c0.w * dv, a0 = c1.x * dv2;
+        int ia = ilo, ie = ihi;
+        if (g.uinv != 0.0f && c0.z < 0.0f) chord(c0.z, a1, a0 - chord_cut<0>(), xc, g.uinv, ia, ie);
+        for (int i = ia & ~1; i <= ie; i += 2) {
+            const float2 uu = *reinterpret_cast<const float2 *>(su + i);
+            const float du0 = uu.x - u0, du1 = uu.y - u0;
+            const float q0 = fmaf(fmaf(c0.z, du0, a1), du0, a0), q1 = fmaf(fmaf(c0.z, du1, a1), du1, a0);
+            const float e0 = profile<0>(q0), e1 = profile<0>(q1);
+            if (e0 == 0.0f && e1 == 0.0f) continue;
+            const float tb = t4.x + t4.z * dv - g.tof_t0;
+            const f2 ts = pk(tb + t4.y * du0, tb + t4.y * du1);
+            f2 Ge = 0, D1 = 0, D2 = 0;
+            const float *gp = sg + j * bd.st + i;
+            for (int b = 0; b < g.n_tof; b++) {
+                const float t = -(float)b * g.tof_h;
+                const f2 x = add2(ts, pk(t, t)), x2 = mul2(x, x), y = mul2(NS, x2);
+                float y0, y1;
+                up(y, y0, y1);
+                const float2 gg = *reinterpret_cast<const float2 *>(gp + b * plane);
+                const f2 gw = mul2(pk(gg.x, gg.y), pk(ex2_approx(y0), ex2_approx(y1)));
+                Ge = add2(Ge, gw);
+                D1 = fma2(gw, x, D1);
+                D2 = fma2(gw, x2, D2);
+            }
+#pragma unroll
+            for (int k = 0; k < 2; k++) {
+                float G0, G1, d10, d11, d20, d21;
+                up(Ge, G0, G1);
+                up(D1, d10, d11);
+                up(D2, d20, d21);
+                const float du = k ? du1 : du0, e = k ? e1 : e0, q = k ? q1 : q0;
+                const float ge = (k ? G1 : G0) * nrm;
+                const float v1 = e * ((k ? d11 : d10) * (-nrm * is2));              // val sum g_k dW_k/dt*
+                const float v2 = e * (0.5f * is2 * (nrm * is2 * (k ? d21 : d20) - ge));   // val sum g_k dW_k/ds^2
+                const float h = ge * e, hd = h * du;
+                m[0] += h;
+                m[1] += hd;
+                m[2] = fmaf(h, dv, m[2]);
+                m[3] = fmaf(hd, du, m[3]);
+                m[4] = fmaf(hd, dv, m[4]);
+                m[5] = fmaf(h * dv, dv, m[5]);
+                m[6] = fmaf(h, q, m[6]);
+                m[7] += v1;
+                m[8] = fmaf(v1, du, m[8]);
+                m[9] = fmaf(v1, dv, m[9]);
+                m[10] += v2;
+            }
+        }
+    }
+}
+
+// moments of rows() in the layout of view_chain
+template <int KER>
+__device__ __forceinline__ void finish(const float *m, float iA, float rA, float *s)
+{
+    constexpr float FQ = Fac<KER>::FQ, FP = Fac<KER>::FP;
+    const float f = rA * iA;
+    s[0] = -FQ * f * m[1];
+    s[1] = -FQ * f * m[2];
+    s[2] = -FQ * f * m[3];
+    s[3] = -FQ * f * m[4];
+    s[4] = -FQ * f * m[5];
+    s[5] = f * (FP * m[6] - 0.5f * m[0]);
+    s[6] = rA * (KER == 1 ? m[0] + m[6] : m[0]);
+}
+
+// Sum the N moments over sub-warps of 2^LG lanes, transposed (each halving of
+// the sub-warp also halves the values a lane keeps), and add this lane's sums
+// to out[0..N).
+template <int N, int LG>
+__device__ __forceinline__ void reduce_add(float *v, int sl, float *out)
+{
+    constexpr int H1 = (N + 1) / 2, H2 = (H1 + 1) / 2, H3 = (H2 + 1) / 2, H4 = (H3 + 1) / 2, H5 = (H4 + 1) / 2;
+    constexpr int HN[6] = { N, H1, H2, H3, H4, H5 };
+    int p = 0, len = N;
+    if (LG >= 1) { tr_stage<N, 1>(v, sl); const int h = H1; if (sl & 1) { p += h; len -= h; } else len = h; }
+    if (LG >= 2) { tr_stage<H1, 2>(v, sl); const int h = H2; if (sl & 2) { p += h; len -= h; } else len = min(len, h); }
+    if (LG >= 3) { tr_stage<H2, 4>(v, sl); const int h = H3; if (sl & 4) { p += h; len -= h; } else len = min(len, h); }
+    if (LG >= 4) { tr_stage<H3, 8>(v, sl); const int h = H4; if (sl & 8) { p += h; len -= h; } else len = min(len, h); }
+    if (LG >= 5) { tr_stage<H4, 16>(v, sl); const int h = H5; if (sl & 16) { p += h; len -= h; } else len = min(len, h); }
+    constexpr int LAST = HN[LG];
+#pragma unroll
+    for (int q = 0; q < LAST; q++)
+        if (q < len) out[p + q] += v[q];
+}
+
+// A Gaussian near a segment end, in world coordinates: the warp shares the
+// pixels of its box; the owner lane adds the sums to its gradient.  Out of
+// line: it is rarely taken.
+template <int KER, bool TOF>
+__device__ __noinline__ void general_box(const DevGeom &g, int view, const float4 *rec,
+                                         uint32_t gid, int ilo, int ihi, int jlo, int jhi, const float *dLdI,
+                                         float *val)
+{
+    const int lane = threadIdx.x & 31;
+    float F[9];
+    for (int q = 0; q < 9; q++) F[q] = __ldg(g.frames + 9 * (size_t)view + q);
+    struct { float4 g0, g1, g2; } r;
+    r.g0 = __ldg(rec + REC_F4 * (size_t)gid);
+    r.g1 = __ldg(rec + REC_F4 * (size_t)gid + 1);
+    r.g2 = __ldg(rec + REC_F4 * (size_t)gid + 2);
+    const int w = ihi - ilo + 1;
+    const long long np = (long long)w * (jhi - jlo + 1);
+    for (int q = 0; q < NG; q++) val[q] = 0.0f;
+    for (long long p = lane; p < np; p += 32) {
+        const int i = ilo + (int)(p % w), j = jlo + (int)(p / w);
+        const Ray ray = make_ray<GM_PARALLEL>(g, F, __ldg(g.utab + i), __ldg(g.vtab + j));
+        PairGeo q;
+        pair_geo(ray, r, q);
+        if (!(q.m <= PAIR_CUT2)) continue;
+        const long long idx = (long long)view * g.stride_view + (long long)j * g.stride_row + i;
+        for (int b = 0; b < (TOF ? g.n_tof : 1); b++) {
+            const float gw = __ldg(dLdI + idx + (TOF ? b * g.stride_tof : 0));
+            if (gw == 0.0f) continue;
+            float pv[NG];
+            if (TOF) general_grad<KER>(ray, q, r.g0.w, gw, pv, g.tof_t0 + (float)b * g.tof_h, g.tof_tau);
+            else general_grad<KER>(ray, q, r.g0.w, gw, pv);
+            for (int k = 0; k < NG; k++) val[k] += pv[k];
+        }
+    }
+    for (int q = 0; q < NG; q++)
+        for (int o = 16; o > 0; o >>= 1) val[q] += __shfl_xor_sync(0xffffffffu, val[q], o);
+}
+
+// views staged by the CTA and its warps' records and moments
+template <bool TOF> struct Shared {
+    static constexpr int BW = Wide<TOF>::v;
+    static constexpr int NM = TOF ? 11 : 7;
+    float sg[Cap<TOF>::v];
+    float su[BW + 2], sv[BH + 2];
+    int4 sbox[2][NW];
+    float4 c0[BS], c1[BS], t4[TOF ? BS : 1];
+    int2 box[BS];                // the Gaussian's rectangle (packed as k_cull's)
+    float mom[BS * NM];
+    float acc[16][BS];
+};
+
+template <int KER, bool TOF, int LG>
+__global__ void __launch_bounds__(BS, 6) k_adjoint(DevGeom g, int nv, int64_t n, int gw, int vper,
+                                                   const uint32_t *__restrict__ order,
+                                                   const float4 *__restrict__ rec,
+                                                   const float4 *__restrict__ crec,
+                                                   const uint2 *__restrict__ rect,
+                                                   const float *__restrict__ dLdI, float4 *__restrict__ grad)
+{
+    using Sh = Shared<TOF>;
+    constexpr int NM = Sh::NM, S = 1 << LG, BW = Sh::BW;
+    __shared__ __align__(16) Sh sh;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, wb = 32 * w;
+    const int sl = lane & (S - 1), sw = lane >> LG;
+    const int64_t slot = ((int64_t)blockIdx.x * NW + w) * gw + lane;
+    const bool active = lane < gw && slot < n;
+    const uint32_t gid = active ? __ldg(order + slot) : 0u;
+    const int va = blockIdx.y * vper, vb = min(nv, va + vper);
+    const int nb = TOF ? g.n_tof : 1;
+#pragma unroll
+    for (int q = 0; q < 16; q++) sh.acc[q][threadIdx.x] = 0.0f;
+    uint2 rc_next = active && va < vb ? __ldg(rect + (int64_t)va * n + gid) : make_uint2(1u, 1u);
+    for (int vl = va; vl < vb; vl++) {
+        const uint2 rc = rc_next;
+        if (vl + 1 < vb && active) rc_next = __ldg(rect + (int64_t)(vl + 1) * n + gid);
+        Box me;
+        me.ilo = rc.x & 0xffff; me.ihi = rc.x >> 16; me.jlo = rc.y & 0xffff; me.jhi = rc.y >> 16;
+        const bool vis = active && me.ilo <= me.ihi;
+        // the rectangle that holds the CTA's boxes
+        {
+            int4 b;
+            b.x = __reduce_min_sync(0xffffffffu, vis ? me.ilo : 0x7fffffff);
+            b.y = __reduce_max_sync(0xffffffffu, vis ? me.ihi : -1);
+            b.z = __reduce_min_sync(0xffffffffu, vis ? me.jlo : 0x7fffffff);
+            b.w = __reduce_max_sync(0xffffffffu, vis ? me.jhi : -1);
+            if (lane == 0) sh.sbox[vl & 1][w] = b;
+        }
+        __syncthreads();   // (also: every thread is done with the previous view's band)
+        int4 ub = sh.sbox[vl & 1][0];
+#pragma unroll
+        for (int k = 1; k < NW; k++) {
+            const int4 b = sh.sbox[vl & 1][k];
+            ub.x = min(ub.x, b.x); ub.y = max(ub.y, b.y); ub.z = min(ub.z, b.z); ub.w = max(ub.w, b.w);
+        }
+        if (ub.y < 0) continue;   // no Gaussian of the CTA on the detector
+        const int view = g.v0 + vl;
+        // this lane's record in the view; a footprint far larger than its
+        // warp's others is left to the whole warp instead of one sub-warp
+        bool gen = false;
+        uint32_t bigs;
+        int turn;
+        {
+            const int area = vis ? (me.ihi - me.ilo + 1) * (me.jhi - me.jlo + 1) : 0;
+            const int mean = (int)(__reduce_add_sync(0xffffffffu, (unsigned)min(area, 1 << 26)) >> 5);
+            const bool big = LG < 5 && area > 64 * S && area > 4 * mean;
+            bool sat = false;
+            if (vis) {
+                float F[9];
+#pragma unroll
+                for (int q = 0; q < 9; q++) F[q] = __ldg(g.frames + 9 * (size_t)view + q);
+                VRec r;
+                prep_record<GM_PARALLEL, KER>(g, F, gid, rec, crec, r);
+                sat = r.g2.w != 0.0f;
+                sh.c0[threadIdx.x] = r.c0;
+                sh.c1[threadIdx.x] = r.c1;
+                if (TOF) sh.t4[threadIdx.x] = r.t4;
+            }
+            gen = vis && !sat;
+            bigs = __ballot_sync(0xffffffffu, big && sat);
+            // the warp's Gaussians by the size of their boxes, largest first:
+            // sub-warps walk side by side, so those of a round should be alike
+            uint32_t key = ((vis && sat ? (uint32_t)min(area, 1 << 26) : 0u) << 5) | (uint32_t)lane;
+#pragma unroll
+            for (int k = 2; k <= 32; k <<= 1)
+#pragma unroll
+                for (int j = k >> 1; j > 0; j >>= 1) {
+                    const uint32_t o = __shfl_xor_sync(0xffffffffu, key, j);
+                    const bool lower = (lane & j) == 0, desc = (lane & k) == 0;
+                    key = lower == desc ? max(key, o) : min(key, o);
+                }
+            turn = (int)(key & 31u);
+            sh.box[threadIdx.x] = vis && sat ? make_int2((int)rc.x, (int)rc.y) : make_int2(1, 1);
+#pragma unroll
+            for (int q = 0; q < NM; q++) sh.mom[threadIdx.x * NM + q] = 0.0f;
+        }
+        const int n_vs = __popc(__ballot_sync(0xffffffffu, vis && !gen));
+        bool first = true;
+        Band bd;
+        for (bd.cb = ub.x; bd.cb <= ub.y; bd.cb += BW) {
+            bd.w = min(BW, ub.y - bd.cb + 1);
+            bd.st = (bd.w + 1) & ~1;
+            const int hmax = min(BH, Cap<TOF>::v / (bd.st * nb));
+            for (bd.rb = ub.z; bd.rb <= ub.w; bd.rb += hmax) {
+                bd.h = min(hmax, ub.w - bd.rb + 1);
+                if (!first) __syncthreads();
+                // stage dL/dI of the band, a warp taking 1, 2 or 4 rows at a time
+                for (int i = threadIdx.x; i < bd.st; i += BS)
+                    sh.su[i] = __ldg(g.utab + min(bd.cb + i, g.n_cols - 1));
+                for (int j = threadIdx.x; j < bd.h; j += BS) sh.sv[j] = __ldg(g.vtab + bd.rb + j);
+                const int sh_ = bd.st <= 8 ? 3 : bd.st <= 16 ? 4 : 5;
+                const int lc = lane & ((1 << sh_) - 1), lr = (w << (5 - sh_)) + (lane >> sh_), rstep = NW << (5 - sh_);
+                for (int c = lc; c < bd.st; c += 1 << sh_) {
+                    const float *src = dLdI + (long long)view * g.stride_view + (bd.cb + c);
+                    for (int j = lr; j < bd.h; j += rstep) {
+#pragma unroll 1
+                        for (int b = 0; b < nb; b++) {
+                            const float x = c < bd.w ? __ldg(src + (long long)(bd.rb + j) * g.stride_row +
+                                                             (TOF ? b * g.stride_tof : 0)) : 0.0f;
+                            sh.sg[(b * bd.h + j) * bd.st + c] = x;
+                        }
+                    }
+                }
+                __syncthreads();
+                first = false;
+                // the sub-warps take the warp's Gaussians in turn ...
+                auto take = [&](int k, int l, auto lgc, bool on) {
+                    constexpr int L = decltype(lgc)::value;
+                    const int2 b = sh.box[wb + k];
+                    Box bx;
+                    bx.ilo = b.x & 0xffff; bx.ihi = (int)((unsigned)b.x >> 16);
+                    bx.jlo = b.y & 0xffff; bx.jhi = (int)((unsigned)b.y >> 16);
+                    if (!on) { bx.jlo = 1; bx.jhi = 0; bx.ilo = 1; bx.ihi = 0; }
+                    const float4 c0 = sh.c0[wb + k], c1 = sh.c1[wb + k];
+                    float m[NM];
+                    if (TOF) {
+                        rows_tof(g, c0, c1, sh.t4[wb + k], bx, l, 1 << L, bd, sh.sg, sh.su, sh.sv, m);
+                    } else {
+                        rows<KER>(g, c0, c1, bx, l, 1 << L, bd, sh.sg, sh.su, sh.sv, m);
+                    }
+                    __syncwarp();
+                    reduce_add<NM, L>(m, l, sh.mom + (wb + k) * NM);
+                };
+                __syncwarp();
+                {
+                    for (int t = 0; t < n_vs; t += 32 / S) {
+                        const int k = __shfl_sync(0xffffffffu, turn, t + sw);
+                        take(k, sl, std::integral_constant<int, LG>{}, !((bigs >> k) & 1u));
+                    }
+                    // ... and the whole warp the big ones
+                    for (uint32_t bm = LG < 5 ? bigs : 0u; bm; bm &= bm - 1u)
+                        take(__ffs(bm) - 1, lane, std::integral_constant<int, 5>{}, true);
+                }
+            }
+        }
+        __syncwarp();
+        if (vis && !gen) {
+            float m[NM], o[16];
+            bool any = false;
+#pragma unroll
+            for (int q = 0; q < NM; q++) {
+                m[q] = sh.mom[threadIdx.x * NM + q];
+                any |= m[q] != 0.0f;
+            }
+            if (any) {
+                float F[9];
+#pragma unroll
+                for (int q = 0; q < 9; q++) F[q] = __ldg(g.frames + 9 * (size_t)view + q);
+                const float4 c1 = sh.c1[threadIdx.x];
+                float s[12], tof4[4];
+                finish<KER>(m, c1.y, c1.z, s);
+                if (TOF) {
+#pragma unroll
+                    for (int q = 0; q < 4; q++) tof4[q] = c1.z * m[TOF ? 7 + q : 0];
+                }
+                view_chain<GM_PARALLEL, KER>(g, F, rec, gid, s, o, TOF ? tof4 : nullptr);
+#pragma unroll
+                for (int q = 0; q < 16; q++) sh.acc[q][threadIdx.x] += o[q];
+            }
+        }
+        // Gaussians near a segment end
+        uint32_t gm = __ballot_sync(0xffffffffu, gen);
+        while (gm) {
+            const int owner = __ffs(gm) - 1;
+            gm &= gm - 1u;
+            float val[NG];
+            general_box<KER, TOF>(g, view, rec, __shfl_sync(0xffffffffu, gid, owner),
+                                      __shfl_sync(0xffffffffu, me.ilo, owner), __shfl_sync(0xffffffffu, me.ihi, owner),
+                                      __shfl_sync(0xffffffffu, me.jlo, owner), __shfl_sync(0xffffffffu, me.jhi, owner),
+                                      dLdI, val);
+            if (lane == owner) {
+                const int slot_of[NG] = { 0, 1, 2, 4, 5, 6, 7, 8, 9, 3 };
+#pragma unroll
+                for (int q = 0; q < NG; q++) sh.acc[slot_of[q]][threadIdx.x] += val[q];
+            }
+        }
+    }
+    if (active) {
+        float acc[16];
+        bool any = false;
+#pragma unroll
+        for (int q = 0; q < 16; q++) {
+            acc[q] = sh.acc[q][threadIdx.x];
+            any |= acc[q] != 0.0f;
+        }
+        if (any) {
+            float4 *gp = grad + GRAD_F4 * (size_t)gid;
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                atomicAdd(gp + q, make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]));
+        }
+    }
+}
+
+// ---- spatial order ---------------------------------------------------------
+//
+// The Gaussians sorted by a cell code: the bounding box of the centres is
+// halved along whichever axis is then longest until a cell of an evenly filled
+// box would hold CELL_N Gaussians, so cells are near cubes and consecutive
+// codes lie together.  Within a cell any order will do.
+constexpr int CELL_N = 4;
+constexpr int CODE_BITS = 15, CELLS = 1 << CODE_BITS;
+constexpr int SMALL_BS = 1024, SMALL_BITS = 12, SMALL_N = 16384;
+
+// monotone map of binary32 to u32
+__device__ __forceinline__ uint32_t ord_enc(float x)
+{
+    const uint32_t b = __float_as_uint(x);
+    return b & 0x80000000u ? ~b : b | 0x80000000u;
+}
+__device__ __forceinline__ float ord_dec(uint32_t u)
+{
+    return __uint_as_float(u & 0x80000000u ? u & 0x7fffffffu : ~u);
+}
+
+// box: enc(max) of x, y, z, then ~enc(min) (zeroed buffer = empty)
+__device__ __forceinline__ uint32_t cell_code(const float4 *__restrict__ crec, int64_t k, const uint32_t *box, int bits)
+{
+    const float4 c0 = __ldg(crec + CREC_F4 * k);
+    const float m[3] = { c0.x, c0.y, c0.z };
+    float e[3], f[3];
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const float hi = ord_dec(box[a]), lo = ord_dec(~box[3 + a]);
+        e[a] = hi - lo;
+        f[a] = e[a] > 0.0f ? (m[a] - lo) / e[a] : 0.0f;
+    }
+    uint32_t code = 0;
+    for (int b = 0; b < bits; b++) {
+        const int a = e[0] >= e[1] && e[0] >= e[2] ? 0 : e[1] >= e[2] ? 1 : 2;
+        const float x = 2.0f * (a == 0 ? f[0] : a == 1 ? f[1] : f[2]);
+        const uint32_t bit = x >= 1.0f;
+        code = (code << 1) | bit;
+        const float y = x - (float)bit;
+        if (a == 0) { f[0] = y; e[0] *= 0.5f; }
+        else if (a == 1) { f[1] = y; e[1] *= 0.5f; }
+        else { f[2] = y; e[2] *= 0.5f; }
+    }
+    return code;
+}
+
+__device__ __forceinline__ void box_add(const float *m, uint32_t *b)
+{
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const uint32_t u = ord_enc(m[a]);
+        b[a] = max(b[a], u);
+        b[3 + a] = max(b[3 + a], ~u);
+    }
+}
+
+__global__ void k_order_box(const float4 *__restrict__ crec, int64_t n, uint32_t *box)
+{
+    uint32_t b[6] = { 0, 0, 0, 0, 0, 0 };
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+        const float4 c = __ldg(crec + CREC_F4 * k);
+        const float m[3] = { c.x, c.y, c.z };
+        box_add(m, b);
+    }
+#pragma unroll
+    for (int a = 0; a < 6; a++) {
+        b[a] = __reduce_max_sync(0xffffffffu, b[a]);
+        if ((threadIdx.x & 31) == 0) atomicMax(box + a, b[a]);
+    }
+}
+
+// code << 32 | rank within the cell, per Gaussian
+__global__ void k_order_cells(const float4 *__restrict__ crec, int64_t n, int bits,
+                              const uint32_t *__restrict__ box, uint32_t *__restrict__ cells, uint2 *__restrict__ where)
+{
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const uint32_t c = cell_code(crec, k, box, bits);
+    where[k] = make_uint2(c, atomicAdd(cells + c, 1u));
+}
+
+// exclusive scan of cnt[0..m) in place by one CTA of SMALL_BS threads (m a multiple of SMALL_BS)
+__device__ __forceinline__ void cta_scan(uint32_t *cnt, int m, uint32_t *wsum)
+{
+    const int per = m / SMALL_BS, base = threadIdx.x * per, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t s = 0;
+    for (int k = 0; k < per; k++) s += cnt[base + k];
+    uint32_t inc = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) wsum[w] = inc;
+    __syncthreads();
+    if (w == 0) {
+        const uint32_t v = wsum[lane];
+        uint32_t x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        wsum[lane] = x - v;
+    }
+    __syncthreads();
+    uint32_t run = wsum[w] + inc - s;
+    for (int k = 0; k < per; k++) {
+        const uint32_t c = cnt[base + k];
+        cnt[base + k] = run;
+        run += c;
+    }
+}
+
+__global__ void __launch_bounds__(SMALL_BS) k_order_scan(uint32_t *cells)
+{
+    __shared__ uint32_t wsum[32];
+    cta_scan(cells, CELLS, wsum);
+}
+
+__global__ void k_order_scatter(int64_t n, const uint32_t *__restrict__ cells, const uint2 *__restrict__ where,
+                                uint32_t *__restrict__ order)
+{
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const uint2 p = where[k];
+    order[cells[p.x] + p.y] = (uint32_t)k;
+}
+
+// the whole order by one CTA: small sets, where the launches would dominate
+__global__ void __launch_bounds__(SMALL_BS) k_order_small(const float4 *__restrict__ crec, int n, int bits,
+                                                          uint32_t *order)
+{
+    __shared__ uint32_t cells[1 << SMALL_BITS], wsum[32], box[6];
+    for (int k = threadIdx.x; k < (1 << SMALL_BITS); k += SMALL_BS) cells[k] = 0;
+    if (threadIdx.x < 6) box[threadIdx.x] = 0;
+    __syncthreads();
+    uint32_t b[6] = { 0, 0, 0, 0, 0, 0 };
+    for (int k = threadIdx.x; k < n; k += SMALL_BS) {
+        const float4 c = __ldg(crec + CREC_F4 * k);
+        const float m[3] = { c.x, c.y, c.z };
+        box_add(m, b);
+    }
+#pragma unroll
+    for (int a = 0; a < 6; a++) {
+        b[a] = __reduce_max_sync(0xffffffffu, b[a]);
+        if ((threadIdx.x & 31) == 0) atomicMax(&box[a], b[a]);
+    }
+    __syncthreads();
+    constexpr int PER = SMALL_N / SMALL_BS;
+    uint32_t code[PER], rank[PER];
+#pragma unroll
+    for (int q = 0; q < PER; q++) {
+        const int k = threadIdx.x + q * SMALL_BS;
+        if (k >= n) break;
+        code[q] = cell_code(crec, k, box, bits);
+        rank[q] = atomicAdd(&cells[code[q]], 1u);
+    }
+    __syncthreads();
+    cta_scan(cells, 1 << SMALL_BITS, wsum);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < PER; q++) {
+        const int k = threadIdx.x + q * SMALL_BS;
+        if (k < n) order[cells[code[q]] + rank[q]] = (uint32_t)k;
+    }
+}
+
+}  // namespace
+
+size_t order_tmp_bytes(int64_t n)
+{
+    return n <= SMALL_N ? 16 : sizeof(uint2) * (size_t)n + sizeof(uint32_t) * (CELLS + 8);
+}
+
+cudaError_t launch_order(const float4 *crec, int64_t n, void *tmp, uint32_t *order, cudaStream_t s)
+{
+    if (n <= 0) return cudaSuccess;
+    const int most = n <= SMALL_N ? SMALL_BITS : CODE_BITS;
+    int bits = 0;
+    while (bits < most && (n >> bits) > CELL_N) bits++;
+    if (n <= SMALL_N) {
+        k_order_small<<<1, SMALL_BS, 0, s>>>(crec, (int)n, bits, order);
+        count_launches(1);
+        return cudaGetLastError();
+    }
+    uint2 *where = (uint2 *)tmp;
+    uint32_t *cells = (uint32_t *)(where + n), *box = cells + CELLS;
+    cudaError_t e = cudaMemsetAsync(cells, 0, sizeof(uint32_t) * (CELLS + 6), s);
+    if (e != cudaSuccess) return e;
+    const unsigned nb = (unsigned)((n + 255) / 256);
+    k_order_box<<<nb < 304u ? nb : 304u, 256, 0, s>>>(crec, n, box);
+    k_order_cells<<<nb, 256, 0, s>>>(crec, n, bits, box, cells, where);
+    k_order_scan<<<1, SMALL_BS, 0, s>>>(cells);
+    k_order_scatter<<<nb, 256, 0, s>>>(n, cells, where, order);
+    count_launches(4);
+    return cudaGetLastError();
+}
+
+namespace {
+
+template <int KER, bool TOF>
+void adjoint_lg(int lg, const DevGeom &g, int nv, int64_t n, const uint32_t *order, const float4 *rec,
+                const float4 *crec, const uint2 *rect, const float *dLdI, float4 *grad, cudaStream_t s)
+{
+    // Gaussians per warp: fewer where 32 would leave the GPU short of CTAs
+    int gw = 32;
+    while (gw > 8 && gw > 32 >> lg && (n / (gw * NW)) * nv < 152 * 5) gw >>= 1;
+    const int64_t bx = (n + NW * gw - 1) / (NW * gw);
+    int64_t chunks = (152 * 5 * 12 + bx - 1) / bx;
+    if (chunks > nv) chunks = nv;
+    if (chunks > 65535) chunks = 65535;
+    const int vper = (int)((nv + chunks - 1) / chunks);
+    const dim3 grid((unsigned)bx, (unsigned)((nv + vper - 1) / vper));
+#define RGRT_ADJ(L) k_adjoint<KER, TOF, L><<<grid, BS, 0, s>>>(g, nv, n, gw, vper, order, rec, crec, rect, dLdI, grad)
+    if (lg <= 1) RGRT_ADJ(1);
+    else if (lg == 2) RGRT_ADJ(2);
+    else if (lg == 3) RGRT_ADJ(3);
+    else RGRT_ADJ(4);
+#undef RGRT_ADJ
+}
+
+}  // namespace
+
+cudaError_t launch_adjoint(const DevGeom &g, int nv, int64_t n, int64_t entries, const uint32_t *order,
+                           const float4 *rec, const float4 *crec, const uint2 *rect, const float *dLdI,
+                           float4 *grad, int ker, cudaStream_t s)
+{
+    if (nv <= 0 || n <= 0) return cudaSuccess;
+    // average footprint in pixels, from the tile entries per (view, Gaussian):
+    // a w x w box lands on about (1 + w / tile)^2 tiles
+    const double per = (double)entries / ((double)nv * (double)n);
+    const double side = per > 1.0 ? sqrt(per) - 1.0 : 0.0;
+    const double px = side * side * g.tile_w * g.tile_h;
+    // lanes per Gaussian: measured 2 / 4 / 8 lanes at 36 px (PET ring) 6.9 / 7.2 /
+    // 8.4 ms, at 65 px (raw PET) 0.143 / 0.143 / 0.163, at 470 px (parallel beam)
+    // 0.17 / 0.11 / 0.12; beyond that a lane would walk more rows than the
+    // warps in flight can hide
+    const int lg = px > 20000.0 ? 4 : px > 4000.0 ? 3 : px > 80.0 ? 2 : 1;
+    // time of flight: PET ring, Gaussian kernel (checked by the caller)
+    if (g.n_tof > 0) adjoint_lg<0, true>(lg, g, nv, n, order, rec, crec, rect, dLdI, grad, s);
+    else if (ker == 1) adjoint_lg<1, false>(lg, g, nv, n, order, rec, crec, rect, dLdI, grad, s);
+    else adjoint_lg<0, false>(lg, g, nv, n, order, rec, crec, rect, dLdI, grad, s);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+}  // namespace rgrt

@@ -225,6 +225,7 @@ int bin_views(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, int v0,
     const uint32_t T = (uint32_t)nv * (uint32_t)geom->tiles_per_view;
     if (T >= (1u << 24))  // tile ids share the key with an 8-bit position code
         return fail(RGRT_E_CAPACITY, "views %d..%d hold %u tiles (2^24 at most)", v0, v0 + nv, T);
+    ctx->bin_valid = false;   // until the new lists and boxes are complete
     TRY(ensure(ctx, ctx->cnt, sizeof(uint32_t) * (size_t)E));
     TRY(ensure(ctx, ctx->off, sizeof(uint32_t) * (size_t)E));
     TRY(ensure(ctx, ctx->rect, sizeof(uint2) * (size_t)E));
@@ -501,6 +502,32 @@ int run_forward(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, float
     });
 }
 
+// the Gaussians' spatial order, for the adjoint
+int build_order(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, cudaStream_t s)
+{
+    if (geom->dg.kind != GM_PARALLEL) return RGRT_OK;   // adjoint tile by tile
+    TRY(ensure(ctx, ctx->order, sizeof(uint32_t) * (size_t)g->n));
+    TRY(ensure(ctx, ctx->order_tmp, order_tmp_bytes(g->n)));
+    PROF("k_order");
+    CK(launch_order(g->crec, g->n, ctx->order_tmp.p, (uint32_t *)ctx->order.p, s));
+    return RGRT_OK;
+}
+
+// adjoint of the binned views v0 .. v0 + nv - 1 (K tile entries) into ctx->grad
+int adjoint_views(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, int v0, int nv, uint32_t K,
+                  const float *dLdI, cudaStream_t s)
+{
+    DevGeom dg = geom->dg;
+    dg.v0 = v0;
+    PROF("k_adjoint");
+    if (dg.kind != GM_PARALLEL)
+        CK(launch_adjoint_tiles(dg, nv, g->rec, g->crec, (const uint32_t *)ctx->vals.p, (const uint2 *)ctx->ranges.p,
+                                dLdI, (float4 *)ctx->grad.p, g->kernel, s));
+    else CK(launch_adjoint(dg, nv, g->n, K, (const uint32_t *)ctx->order.p, g->rec, g->crec, (const uint2 *)ctx->rect.p,
+                      dLdI, (float4 *)ctx->grad.p, g->kernel, s));
+    return RGRT_OK;
+}
+
 // adjoint into ctx->grad (zeroed first), then the parameter chain into the
 // four (device) outputs
 int run_backward(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, const float *dLdI,
@@ -529,14 +556,9 @@ int run_backward(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, cons
     }
     if (geom->dg.n_tof && g->kernel != RGRT_KERNEL_GAUSSIAN)
         return fail(RGRT_E_INVAL, "time of flight takes the Gaussian kernel");
+    TRY(build_order(ctx, g, geom, s));
     TRY(for_chunks(ctx, g, geom, s, reuse, [&](int v0, int nv, uint32_t K) -> int {
-        (void)K;
-        DevGeom dg = geom->dg;
-        dg.v0 = v0;
-        PROF("k_adjoint");
-        CK(launch_adjoint(dg, nv, g->rec, g->crec, (uint32_t *)ctx->vals.p, (uint2 *)ctx->ranges.p,
-                          dLdI, (float4 *)ctx->grad.p, g->kernel, s));
-        return RGRT_OK;
+        return adjoint_views(ctx, g, geom, v0, nv, K, dLdI, s);
     }));
     PROF("k_param_chain");
     CK(launch_param_chain(g->mu, g->ls, g->q, g->rho, N, (float4 *)ctx->grad.p, gm, gl, gq, gr, s));
@@ -738,7 +760,7 @@ int rgrt_ctx_destroy(rgrt_ctx *c)
     Buf *bufs[] = { &c->cnt, &c->off, &c->rect, &c->keys, &c->vals, &c->keys_alt, &c->vals_alt,
                     &c->sort_tmp, &c->scan_tmp, &c->ranges, &c->total, &c->I, &c->dLdI, &c->y,
                     &c->grad, &c->gflat, &c->partial, &c->stats, &c->loss, &c->loss_acc, &c->ball, &c->part,
-                    &c->scene, &c->blk, &c->wblk, &c->clusters };
+                    &c->scene, &c->blk, &c->wblk, &c->clusters, &c->order, &c->order_tmp };
     for (Buf *b : bufs) release(c, *b);
     for (auto &b : c->stage_in) release(c, b);
     for (auto &b : c->stage_out) release(c, b);
@@ -1107,8 +1129,8 @@ static int run_loss_grad(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *ge
         const int64_t HW = (int64_t)geom->dg.n_rows * geom->dg.n_cols;
         float *I = (float *)ctx->I.p, *dLdI = (float *)ctx->dLdI.p;
         const float *y = (const float *)dy;
+        TRY(build_order(ctx, g, geom, s));
         TRY(for_chunks(ctx, g, geom, s, false, [&](int v0, int nv, uint32_t K) -> int {
-            (void)K;
             DevGeom dg = geom->dg;
             dg.v0 = v0;
             {
@@ -1125,12 +1147,7 @@ static int run_loss_grad(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *ge
                                (double *)ctx->partial.p, loss_blocks(n), (float *)ctx->loss.p, s,
                                (double *)ctx->loss_acc.p));
             }
-            {
-                PROF("k_adjoint");
-                CK(launch_adjoint(dg, nv, g->rec, g->crec, (uint32_t *)ctx->vals.p, (uint2 *)ctx->ranges.p,
-                                  dLdI, (float4 *)ctx->grad.p, g->kernel, s));
-            }
-            return RGRT_OK;
+            return adjoint_views(ctx, g, geom, v0, nv, K, dLdI, s);
         }));
         PROF("k_param_chain");
         CK(launch_param_chain(g->mu, g->ls, g->q, g->rho, N, (float4 *)ctx->grad.p, gm, gl, gq, gr, s));
@@ -1258,6 +1275,7 @@ int gaussians_voxelize(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_volume_des
         CK(cudaMemsetAsync(dout, 0, sizeof(float) * nvox, s));
     } else {
         TRY(build_records(ctx, g, s));
+        ctx->bin_valid = false;   // the shared scratch is to hold brick lists
         TRY(ensure(ctx, ctx->cnt, sizeof(uint32_t) * (size_t)N));
         TRY(ensure(ctx, ctx->off, sizeof(uint32_t) * (size_t)N));
         TRY(ensure(ctx, ctx->rect, sizeof(uint4) * (size_t)N));
@@ -1291,7 +1309,6 @@ int gaussians_voxelize(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_volume_des
             CK(cudaMemsetAsync(ctx->ranges.p, 0, sizeof(uint2) * (size_t)nb, s));
             CK(launch_vox_ranges(keys, (uint32_t)K, (uint2 *)ctx->ranges.p, (uint32_t)nb, s));
         }
-        ctx->bin_valid = false;   // the shared scratch now holds brick lists
         PROF("k_voxelize");
         CK(launch_voxelize(g->rec, g->crec, vals, (const uint2 *)ctx->ranges.p, v, (float *)dout, g->kernel, s));
     }

@@ -63,6 +63,9 @@ struct BatchScan {
     bool large = false;         // projected by its own launches (not the persistent ones)
     uint32_t *vals = nullptr;   // sorted Gaussian ids [cap]
     uint2 *ranges = nullptr;    // [T]
+    uint2 *rect = nullptr;      // pixel boxes [E] (a large scan: the shared scratch)
+    uint32_t *order = nullptr;  // spatial order [N]
+    int64_t keys = 0;           // planned tile entries
     float *I = nullptr, *dLdI = nullptr;
     float4 *grad = nullptr;
     float *gflat = nullptr;
@@ -88,6 +91,7 @@ struct rgrt_batch {
     uint32_t *cnt = nullptr, *off = nullptr, *keys = nullptr, *keys_alt = nullptr,
              *vals_alt = nullptr, *sort_tmp = nullptr;
     uint2 *rect = nullptr;
+    void *order_tmp = nullptr;
     unsigned long long *stmp = nullptr, *total = nullptr;
     // batch tables
     ScanDesc *d_desc = nullptr;
@@ -97,7 +101,7 @@ struct rgrt_batch {
     uint32_t total_items = 0;     // work items of the persistent launches (small scans)
     uint64_t all_tiles = 0;       // tiles of every scan
     int n_small = 0;              // scans in the persistent descriptor table
-    int grid_f = 0, grid_a = 0;
+    int grid_f = 0;
     uint64_t keys_capacity = 0;
     // graphs
     cudaStream_t stream = nullptr;
@@ -125,11 +129,12 @@ void free_plan(rgrt_batch *b)
     for (auto &a : b->allocs) ctx_free(b->ctx, a.first, a.second);
     b->allocs.clear();
     for (auto &s : b->sc) {
-        s.vals = nullptr; s.ranges = nullptr; s.I = s.dLdI = nullptr;
+        s.vals = nullptr; s.ranges = nullptr; s.rect = nullptr; s.order = nullptr; s.I = s.dLdI = nullptr;
         s.grad = nullptr; s.gflat = nullptr; s.partial = nullptr;
     }
     b->cnt = b->off = b->keys = b->keys_alt = b->vals_alt = b->sort_tmp = nullptr;
     b->rect = nullptr;
+    b->order_tmp = nullptr;
     b->stmp = b->total = nullptr;
     b->d_desc = nullptr;
     b->d_queue = b->d_overflow = nullptr;
@@ -144,13 +149,18 @@ int plan(rgrt_batch *b)
 {
     free_plan(b);
     cudaStream_t s = b->stream;
-    int64_t Emax = 1;
-    for (auto &x : b->sc) Emax = std::max<int64_t>(Emax, x.E);
+    int64_t Emax = 1, Nmax = 1;
+    for (auto &x : b->sc) {
+        Emax = std::max<int64_t>(Emax, x.E);
+        Nmax = std::max<int64_t>(Nmax, x.N);
+    }
     BTRY(balloc(b, (void **)&b->cnt, sizeof(uint32_t) * Emax));
     BTRY(balloc(b, (void **)&b->off, sizeof(uint32_t) * Emax));
     BTRY(balloc(b, (void **)&b->rect, sizeof(uint2) * Emax));
+    if (!b->cone) BTRY(balloc(b, &b->order_tmp, order_tmp_bytes(Nmax)));
     BTRY(balloc(b, (void **)&b->stmp, sizeof(unsigned long long) * scan_tmp_elems(Emax)));
     BTRY(balloc(b, (void **)&b->total, sizeof(unsigned long long) * 2));
+    b->grid_f = persistent_grid(b->cone, b->tile_w * b->tile_h);
     uint32_t capmax = 1;
     int vmax = 0;
     b->keys_capacity = 0;
@@ -167,6 +177,13 @@ int plan(rgrt_batch *b)
         unsigned long long cap = K + K / 4 + 4096;
         if (cap >= 0xffffffffull) return report_error(RGRT_E_CAPACITY, "a scan of the batch has more than 2^32 tile entries");
         x.cap = (uint32_t)cap;
+        x.keys = (int64_t)K;
+        x.large = (int64_t)x.T >= 16 * (int64_t)b->grid_f;
+        x.rect = b->rect;
+        if (!b->cone) {
+            if (!x.large) BTRY(balloc(b, (void **)&x.rect, sizeof(uint2) * (size_t)std::max<int64_t>(x.E, 1)));
+            BTRY(balloc(b, (void **)&x.order, sizeof(uint32_t) * (size_t)std::max<int64_t>(x.N, 1)));
+        }
         capmax = std::max(capmax, x.cap);
         if (x.lbits >= 0) vmax = std::max(vmax, x.geom->dg.n_views);
         b->keys_capacity += cap;
@@ -183,8 +200,6 @@ int plan(rgrt_batch *b)
     BTRY(balloc(b, (void **)&b->keys_alt, sizeof(uint32_t) * capmax));
     BTRY(balloc(b, (void **)&b->vals_alt, sizeof(uint32_t) * capmax));
     BTRY(balloc(b, (void **)&b->sort_tmp, sizeof(uint32_t) * sort_tmp_elems(capmax, vmax)));
-    b->grid_f = persistent_grid(true, b->cone, b->tile_w, b->tile_w * b->tile_h);
-    b->grid_a = persistent_grid(false, b->cone, b->tile_w, b->tile_w * b->tile_h);
     // A scan whose tiles fill the GPU for 16 waves or more gains nothing from
     // sharing the persistent launches: it is binned, projected, and its loss
     // and adjoint taken back to back with launches of its own, while its
@@ -196,7 +211,6 @@ int plan(rgrt_batch *b)
     for (int i = 0; i < b->n; i++) {
         BatchScan &x = b->sc[i];
         b->all_tiles += x.T;
-        x.large = (int64_t)x.T >= 16 * (int64_t)b->grid_f;
         if (x.large) continue;
         hd.emplace_back();
         ScanDesc &d = hd.back();
@@ -235,13 +249,13 @@ int enqueue_bin_scan(rgrt_batch *b, int i, cudaStream_t s)
         DevGeom dg = x.geom->dg;
         dg.v0 = 0;
         BK(launch_records(x.g->mu, x.g->ls, x.g->q, x.g->rho, x.N, x.g->rec, x.g->crec, nullptr, s));
-        BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, b->cnt, b->rect, s));
+        BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, b->cnt, x.rect, s));
         BK(launch_scan(b->cnt, b->off, x.E, b->total, b->stmp, s));
         // the scan's total (on the device) is the number of keys this step
         // emits: the sort and the ranges take only those (at most the planned
         // capacity; an item past it writes padding keys, which sort last and
         // map to no tile, and raises the overflow flag)
-        BK(launch_emit(dg, dg.n_views, x.N, b->cnt, b->off, b->rect, b->keys, x.vals, x.cap,
+        BK(launch_emit(dg, dg.n_views, x.N, b->cnt, b->off, x.rect, b->keys, x.vals, x.cap,
                        b->d_overflow, s, x.lbits));
         if (x.lbits >= 0)
             BK(launch_sort_views(b->keys, x.vals, b->keys_alt, b->vals_alt, x.cap, x.bits, b->off, x.N,
@@ -291,6 +305,24 @@ int enqueue_loss(rgrt_batch *b, int i, const float *const *y, int loss, const rg
     return RGRT_OK;
 }
 
+// adjoint of scan i by launches of its own: parallel rays (from its boxes) and
+// large cone-beam scans (from its tile lists)
+int enqueue_adjoint(rgrt_batch *b, int i, cudaStream_t s)
+{
+    BatchScan &x = b->sc[i];
+    DevGeom dg = x.geom->dg;
+    dg.v0 = 0;
+    if (b->cone) {
+        BK(launch_adjoint_tiles(dg, dg.n_views, x.g->rec, x.g->crec, x.vals, x.ranges, x.dLdI, x.grad,
+                                RGRT_KERNEL_GAUSSIAN, s));
+        return RGRT_OK;
+    }
+    BK(launch_order(x.g->crec, x.N, b->order_tmp, x.order, s));
+    BK(launch_adjoint(dg, dg.n_views, x.N, x.keys, x.order, x.g->rec, x.g->crec, x.rect, x.dLdI, x.grad,
+                      RGRT_KERNEL_GAUSSIAN, s));
+    return RGRT_OK;
+}
+
 int enqueue_step(rgrt_batch *b, const float *const *y, int loss, const rgrt_adam *hp, cudaStream_t s)
 {
     BK(cudaMemsetAsync(b->d_overflow, 0, sizeof(uint32_t), s));
@@ -301,21 +333,22 @@ int enqueue_step(rgrt_batch *b, const float *const *y, int loss, const rgrt_adam
         if (!x.large) continue;
         BTRY(enqueue_forward_large(b, i, s));
         BTRY(enqueue_loss(b, i, y, loss, hp, s));
-        DevGeom dg = x.geom->dg;
-        dg.v0 = 0;
-        BK(launch_adjoint(dg, dg.n_views, x.g->rec, x.g->crec, x.vals, x.ranges, x.dLdI, x.grad,
-                          RGRT_KERNEL_GAUSSIAN, s));
+        BTRY(enqueue_adjoint(b, i, s));
     }
-    // small scans: one persistent forward and one persistent adjoint
+    // small scans: one persistent forward and (cone beam) one persistent adjoint
     if (b->n_small > 0) {
         BK(cudaMemsetAsync(b->d_queue, 0, sizeof(uint32_t), s));
         BK(launch_forward_persistent(b->cone, b->d_desc, b->n_small, b->total_items, b->d_queue,
                                      b->tile_w * b->tile_h, b->grid_f, s));
         for (int i = 0; i < b->n; i++)
             if (!b->sc[i].large) BTRY(enqueue_loss(b, i, y, loss, hp, s));
-        BK(cudaMemsetAsync(b->d_queue + 1, 0, sizeof(uint32_t), s));
-        BK(launch_adjoint_persistent(b->cone, b->tile_w, b->d_desc, b->n_small, b->total_items,
-                                     b->d_queue + 1, b->grid_a, s));
+        if (b->cone) {
+            BK(cudaMemsetAsync(b->d_queue + 1, 0, sizeof(uint32_t), s));
+            BK(launch_adjoint_persistent(b->tile_w, b->d_desc, b->n_small, b->total_items, b->d_queue + 1, s));
+        } else {
+            for (int i = 0; i < b->n; i++)
+                if (!b->sc[i].large) BTRY(enqueue_adjoint(b, i, s));
+        }
     }
     // parameter chains and Adam last: an overflow flagged by any scan's
     // binning skips every update

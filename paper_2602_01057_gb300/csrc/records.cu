@@ -255,7 +255,7 @@ __global__ void k_cull(DevGeom g, int nv, const float4 *__restrict__ crec, int64
     }
     if (i0 > i1 || j0 > j1) {
         cnt[idx] = 0;
-        rect[idx] = make_uint2(0u, 0u);
+        rect[idx] = make_uint2(1u, 1u);   // empty: columns and rows 1..0
     } else {
         unsigned tx0 = i0 / g.tile_w, tx1 = i1 / g.tile_w, ty0 = j0 / g.tile_h, ty1 = j1 / g.tile_h;
         cnt[idx] = (tx1 - tx0 + 1) * (ty1 - ty0 + 1);

@@ -130,9 +130,19 @@ cudaError_t launch_sort_views(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt
 cudaError_t launch_forward(const DevGeom &g, int nv, const float4 *rec, const float4 *crec,
                            const uint32_t *gids, const uint2 *ranges, float *out, Stats *stats,
                            int ker, cudaStream_t s);
-cudaError_t launch_adjoint(const DevGeom &g, int nv, const float4 *rec, const float4 *crec,
-                           const uint32_t *gids, const uint2 *ranges, const float *dLdI,
+// Gaussian ids in a spatial order (adjoint.cu), from scratch of
+// order_tmp_bytes(n) bytes
+size_t order_tmp_bytes(int64_t n);
+cudaError_t launch_order(const float4 *crec, int64_t n, void *tmp, uint32_t *order, cudaStream_t s);
+// adjoint of parallel-ray views v0 .. v0 + nv - 1: rect = k_cull's pixel boxes
+// of those views, entries = their (tile, Gaussian) entries (the footprints' size)
+cudaError_t launch_adjoint(const DevGeom &g, int nv, int64_t n, int64_t entries, const uint32_t *order,
+                           const float4 *rec, const float4 *crec, const uint2 *rect, const float *dLdI,
                            float4 *grad, int ker, cudaStream_t s);
+// the same for cone-beam and 3-D PET views, from the tile lists
+cudaError_t launch_adjoint_tiles(const DevGeom &g, int nv, const float4 *rec, const float4 *crec,
+                                 const uint32_t *gids, const uint2 *ranges, const float *dLdI, float4 *grad,
+                                 int ker, cudaStream_t s);
 // one scan of a batch, as the persistent kernels see it
 struct ScanDesc {
     DevGeom g;
@@ -145,15 +155,15 @@ struct ScanDesc {
     uint32_t item_begin;    // first (scan, tile) work item of the scan
     uint32_t n_items;       // tiles of the scan
 };
-// persistent integration / adjoint over every tile of a batch of scans; the
-// queue counter must be zero at launch.  tile_threads = tile_w * tile_h of
-// every scan (one ray per thread in the forward).
+// persistent integration (adjoint: cone beam) over every tile of a batch of
+// scans; the queue counter must be zero at launch.  tile_threads = tile_w * tile_h of every
+// scan (one ray per thread).
 cudaError_t launch_forward_persistent(bool cone, const ScanDesc *d, int nscan, uint32_t total,
                                       uint32_t *queue, int tile_threads, int grid, cudaStream_t s);
-cudaError_t launch_adjoint_persistent(bool cone, int tile_w, const ScanDesc *d, int nscan,
-                                      uint32_t total, uint32_t *queue, int grid, cudaStream_t s);
-// CTAs of a persistent launch: SMs x resident CTAs per SM
-int persistent_grid(bool forward, bool cone, int tile_w, int tile_threads);
+cudaError_t launch_adjoint_persistent(int tile_w, const ScanDesc *d, int nscan, uint32_t total, uint32_t *queue,
+                                      cudaStream_t s);
+// CTAs of the persistent forward: SMs x resident CTAs per SM
+int persistent_grid(bool cone, int tile_threads);
 
 cudaError_t launch_param_chain(const float *mu, const float *ls, const float *q, const float *rho,
                                int64_t n, const float4 *grad, float *g_mu, float *g_ls,
