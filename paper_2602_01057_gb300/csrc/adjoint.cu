@@ -28,6 +28,7 @@
 // ring from 8.0 to 6.9 ms: a round's lanes then have chords of like length.
 #include <type_traits>
 
+#include "packed.cuh"
 #include "view.cuh"
 
 namespace rgrt {
@@ -40,43 +41,6 @@ constexpr int BH = 256;         // highest band (rows)
 
 // shared floats of the staged band
 template <bool TOF> struct Cap { static constexpr int v = TOF ? 5120 : 4096; };
-
-// ---- packed pairs of binary32 -------------------------------------------
-typedef unsigned long long f2;
-__device__ __forceinline__ f2 pk(float a, float b)
-{
-    f2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void up(f2 x, float &a, float &b)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x));
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c)
-{
-    f2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ f2 mul2(f2 a, f2 b)
-{
-    f2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f2 add2(f2 a, f2 b)
-{
-    f2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ float hadd(f2 x)
-{
-    float a, b;
-    up(x, a, b);
-    return a + b;
-}
 
 // factors of the moments' derivatives: with h = dL/dI times the kernel's
 // profile and p = h arg,  -dL/dQ = A^-3/2 FQ h  and  dL/dA = A^-3/2 (FP p -

@@ -492,11 +492,10 @@ int run_forward(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, float
     }
     ctx->last_keys = 0;
     return for_chunks(ctx, g, geom, s, false, [&](int v0, int nv, uint32_t K) -> int {
-        (void)K;
         DevGeom dg = geom->dg;
         dg.v0 = v0;
         PROF("k_forward");
-        CK(launch_forward(dg, nv, g->rec, g->crec, (uint32_t *)ctx->vals.p, (uint2 *)ctx->ranges.p,
+        CK(launch_forward(dg, nv, K, g->rec, g->crec, (uint32_t *)ctx->vals.p, (uint2 *)ctx->ranges.p,
                           out, st, g->kernel, s));
         return RGRT_OK;
     });
@@ -1135,7 +1134,7 @@ static int run_loss_grad(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *ge
             dg.v0 = v0;
             {
                 PROF("k_forward");
-                CK(launch_forward(dg, nv, g->rec, g->crec, (uint32_t *)ctx->vals.p, (uint2 *)ctx->ranges.p,
+                CK(launch_forward(dg, nv, K, g->rec, g->crec, (uint32_t *)ctx->vals.p, (uint2 *)ctx->ranges.p,
                                   I, st, g->kernel, s));
             }
             const int64_t off = (int64_t)v0 * HW, n = (int64_t)nv * HW;

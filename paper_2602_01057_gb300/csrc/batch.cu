@@ -225,6 +225,7 @@ int plan(rgrt_batch *b)
         d.grad = x.grad;
         d.item_begin = (uint32_t)items;
         d.n_items = x.T;
+        d.parts = forward_parts(x.T, x.keys);   // as a projection of its own would
         items += x.T;
     }
     if (items >= 0xffffffffull) return report_error(RGRT_E_CAPACITY, "too many tiles in the batch");
@@ -276,7 +277,7 @@ int enqueue_forward_large(rgrt_batch *b, int i, cudaStream_t s)
     BatchScan &x = b->sc[i];
     DevGeom dg = x.geom->dg;
     dg.v0 = 0;
-    BK(launch_forward(dg, dg.n_views, x.g->rec, x.g->crec, x.vals, x.ranges, x.I, nullptr,
+    BK(launch_forward(dg, dg.n_views, x.keys, x.g->rec, x.g->crec, x.vals, x.ranges, x.I, nullptr,
                       RGRT_KERNEL_GAUSSIAN, s));
     return RGRT_OK;
 }

@@ -1,16 +1,26 @@
 // Per-tile ray integration (a3).
 //
-// One CTA per detector tile of tile_w x tile_h rays, one ray per thread,
-// warps laid out as 8 x 4 ray blocks.  The tile's Gaussian list (ordered by
+// One CTA per detector tile of tile_w x tile_h rays (or a cluster of up to 8
+// that share the tile's list), two rays per thread, a half- or quarter-warp
+// per block of 8 x 4 or 4 x 4 rays.  The tile's Gaussian list (ordered by
 // footprint position, then id) is walked in chunks: the CTA gathers each
 // chunk's records, turning every Gaussian into its view-space form for this
 // view (see below) together with its detector bounding box, into one of two
-// shared-memory buffers.  A warp skips a Gaussian whose box misses its 8 x 4
-// block, or (cone beam) whose footprint ellipse misses it (a warp-uniform
-// branch); otherwise every lane evaluates its pair and the pair counts when
-// m <= 9 (3-sigma cut).  FP32 throughout, FP32 accumulation per ray.
+// shared-memory buffers.  A block skips a Gaussian whose box misses it, or
+// (cone beam) whose footprint ellipse misses it; otherwise its lanes evaluate
+// their two pairs in packed binary32 and a pair counts when m <= 9 (3-sigma
+// cut).  FP32 throughout, FP32 accumulation per ray.
 // 3-D PET LORs (direction e_w + kappa e_v, kappa per detector column) have a
-// view-space form of their own (prep_record, pet3d_chain).
+// view-space form of their own (prep_record).
+//
+// Bound by issue: per evaluated record 64 pairs take about 26 arithmetic
+// instructions (parallel rays 16), where one ray per thread took the same for
+// 32, and the special-function unit two rsqrt and two ex2 per lane.  Measured
+// on a GB300 against one ray per thread (8 x 4 warps, 4 x 4 half-warps): cone
+// beam 50,000 Gaussians, 180 x 256^2 8.5 -> 6.3 ms; PET ring 200,000, 288 x
+// 329 x 63 8.2 -> 5.7 ms; fully 3-D PET (the pair shares its column's slope
+// terms) 79 -> 62 ms; time of flight 4.05 -> 3.3 ms before the lists were
+// shared (SPLIT_CTAS).
 //
 // The closed form (Eqs. 7-11) for a ray and one Gaussian is
 //   rho sqrt(2 pi / A) exp(-m/2),  A = d^T P d,  m = C - B^2/A,
@@ -33,40 +43,59 @@
 // 5.66 sigma of a segment end (then |w| < 4 is possible); such Gaussians take
 // the general path below, in world coordinates, with the ray re-based at the
 // foot of the perpendicular from mu.
+#include <cooperative_groups.h>
+
+#include "packed.cuh"
 #include "view.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace rgrt {
 namespace {
 
-constexpr int CH = 256;             // records per chunk (one per thread in the prep)
-// chunk buffers of the forward: with two, a chunk's records are prepared into
-// one buffer while slower warps still read the other, and a single barrier
-// per chunk suffices.  The staged records (52 B each) leave the general-path
-// fields in global memory so that two buffers still fit 4 CTAs per SM.
+constexpr int CH = 256;             // records per chunk
+constexpr int FBS = 128;            // most threads of a CTA (two rays each)
+// chunk buffers: with two, a chunk's records are prepared into one buffer
+// while slower warps still read the other, and a single barrier per chunk
+// suffices.  The staged records leave the general-path fields in global
+// memory so that two buffers fit 7 CTAs per SM.
 constexpr int NBUF = 2;
+// A tile's list is shared by 2, 4 or 8 CTAs of a cluster while the launch has
+// fewer CTAs than SPLIT_CTAS (about 9 waves: tile lists are uneven, and a few
+// waves leave most of the SMs waiting for the longest) and a CTA's share of an
+// average list stays above SPLIT_LIST records.  Measured without and with it:
+// 672 tiles of 2,700 records (8 raw PET angles) 0.46 -> 0.165 ms, 2,016 tiles
+// (time of flight, 24 angles) 3.4 -> 2.0, 2,048 of 1,270 (8 cone-beam views)
+// 0.55 -> 0.37, 256 of 350 (parallel beam) 0.080 -> 0.036; at 24,000 tiles
+// (PET ring) 5.7 either way, so those keep one CTA.
+constexpr int64_t SPLIT_CTAS = 8192, SPLIT_LIST = 128;
 
-// the forward's copy of a VRec: the view-space coefficients and the gid
-// (general-path records read mu, rho and P from the global records by gid)
-struct SRec {
-    float4 c0, c1, c2;
-    uint32_t gid;
+// A lane's two rays: neighbouring columns of one row, or (3-D PET, whose ray
+// slope is a column's) neighbouring rows of one column.  The lanes of a group
+// share a block of rays and its lists: 8 x 4 rays per half-warp for the cone
+// beam, whose footprints are large, 4 x 4 rays per quarter-warp for the others,
+// whose footprints span a few bins.
+template <int GM>
+struct Blocks {
+    static constexpr int BWID = GM == GM_CONE ? 8 : 4;
+    static constexpr int LANES = GM == GM_CONE ? 16 : 8;
+    static constexpr int PER_WARP = 32 / LANES;
+    static constexpr int MAX = GM == GM_CONE ? 8 : 16;   // blocks of a tile of 256 rays
 };
 
 // a chunk of staged records in shared memory, one array per field: the
-// preparing threads write consecutive 16-byte (4-byte) words, free of bank
-// conflicts, and a warp reads one record at a time (broadcast)
-struct SChunk {
+// preparing threads write consecutive words, free of bank conflicts, and a
+// group of lanes reads one record at a time (broadcast).  Parallel rays need
+// c0, M_vv and the amplitude only.
+template <bool WIDE> struct SChunk;
+template <> struct SChunk<true> {
     float4 c0[CH], c1[CH], c2[CH];
     uint32_t gid[CH];
-    __device__ __forceinline__ SRec operator[](int j) const
-    {
-        SRec r;
-        r.c0 = c0[j];
-        r.c1 = c1[j];
-        r.c2 = c2[j];
-        r.gid = gid[j];
-        return r;
-    }
+};
+template <> struct SChunk<false> {
+    float4 c0[CH];
+    float2 va[CH];     // k M_vv, alpha / sqrt(A)
+    uint32_t gid[CH];
 };
 
 // the general-path fields of record gid (mu, rho | P00 P01 P02 P11 | P12 P22)
@@ -83,89 +112,37 @@ __device__ __forceinline__ GRec load_grec(const float4 *__restrict__ rec, uint32
     return o;
 }
 
-struct TileCtx {
-    int vl, tx, ty, view, col, row;
-    bool valid;                        // the thread's pixel is on the detector
-    bool live;                         // ... and has a ray (3-D PET: a ring pair)
-    float wu_lo, wu_hi, wv_lo, wv_hi;  // detector box of this warp's (half-warp's) rays
-    float zoff, dz;                    // 3-D PET: mid-height offset of the rows, axial LOR rise
-    float kap0, kap1;                  // 3-D PET: LOR slopes at the tile's extreme columns
-    long long out_idx;
-};
-
-// Half-warp blocks (4 x 4 rays per half-warp) for the parallel-ray and 3-D
-// PET geometries, whose footprints span a few bins; cone-beam footprints are
-// large enough that whole-warp 8 x 4 blocks waste little and build their
-// lists for less.
-template <int GM>
-struct HalfBlocks {
-    static constexpr bool value = GM != GM_CONE;
-};
-
-template <int GM>
-__device__ __forceinline__ TileCtx tile_ctx(const DevGeom &g, uint32_t tile)
-{
-    constexpr bool HALF = HalfBlocks<GM>::value;
-    TileCtx c;
-    int T = g.tiles_x * g.tiles_y;
-    c.vl = (int)(tile / (uint32_t)T);
-    int tin = (int)tile - c.vl * T;
-    c.ty = tin / g.tiles_x;
-    c.tx = tin - c.ty * g.tiles_x;
-    c.view = g.v0 + c.vl;
-    // a warp takes an 8 x 4 block of rays (HALF: each half-warp a 4 x 4 half of it)
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int wpr = g.tile_w >> 3;  // warps per tile row
-    int wx = w % wpr, wy = w / wpr;
-    int c0 = c.tx * g.tile_w + wx * 8 + (HALF ? 4 * (lane >> 4) : 0), r0 = c.ty * g.tile_h + wy * 4;
-    c.col = c0 + (HALF ? (lane & 3) : (lane & 7));
-    c.row = r0 + (HALF ? ((lane >> 2) & 3) : (lane >> 3));
-    c.valid = c.col < g.n_cols && c.row < g.n_rows;
-    int rows = g.n_rows;
-    c.zoff = c.dz = c.kap0 = c.kap1 = 0.0f;
-    if (GM == GM_PET3D) {
-        pet3d_view(g, c.view, c.zoff, c.dz, rows);
-        const int tc0 = c.tx * g.tile_w;
-        pet3d_slopes(g, c.dz, tc0, min(tc0 + g.tile_w - 1, g.n_cols - 1), c.kap0, c.kap1);
-    }
-    c.live = c.valid && c.row < rows;
-    if (c0 < g.n_cols && r0 < rows) {
-        int c1 = min(c0 + (HALF ? 3 : 7), g.n_cols - 1), r1 = min(r0 + 3, rows - 1);
-        c.wu_lo = __ldg(g.utab + c0); c.wu_hi = __ldg(g.utab + c1);
-        c.wv_lo = __ldg(g.vtab + r0) + c.zoff; c.wv_hi = __ldg(g.vtab + r1) + c.zoff;
-    } else {
-        c.wu_lo = INFINITY; c.wu_hi = -INFINITY; c.wv_lo = INFINITY; c.wv_hi = -INFINITY;
-    }
-    c.out_idx = (long long)c.view * g.stride_view + (long long)c.row * g.stride_row + c.col;
-    return c;
-}
-
-// Per chunk: every thread turns one record into its view-space form and tests
-// its detector box against the ray block of every warp of the tile (bit w of
-// msk), or with half-warp blocks of every half-warp (bit 2w + h, h the half of
-// warp w); then each warp compacts, in record order, the records that touch
-// its block (each of its halves' blocks) into a list of view-space records and
-// a list of general ones.  The two halves of a warp walk their own lists side
-// by side: smaller blocks leave fewer lanes evaluating pairs outside the
-// footprint.
+// Per chunk: every thread turns records into their view-space form and tests
+// their detector boxes against the tile's blocks (bit b of msk: block b);
+// then each warp compacts, in record order, the records that touch its groups'
+// blocks into one list per group -- of view-space records, and (rarely) of
+// general ones.  The groups of a warp walk their own lists side by side.
 constexpr uint32_t MSK_VS = 1u << 16;   // msk: the record takes the view-space path
 struct ChunkLists {
     uint8_t vs[16][CH];
     uint8_t gen[16][CH];
 };
 
-template <int GM, int KER, bool TOF>
-__device__ __forceinline__ void prep_chunk(const DevGeom &g, const float *F, const uint32_t *gids,
+// the intervals of the tile's column and row blocks; wbox: every block's box
+// (cone beam, for the ellipse test)
+struct TileBoxes {
+    float2 cu[8], rv[8];
+    float4 wbox[8];
+    int ncb, nrb;      // column and row blocks of the tile
+};
+
+template <int GM, int KER, bool TOF, class Chunk>
+__device__ __forceinline__ bool prep_chunk(const DevGeom &g, const float *F, const uint32_t *gids,
                                            uint32_t base, uint32_t stride, int cnt,
-                                           const float4 *rec, const float4 *crec, SChunk *sv,
-                                           const float4 *wbox, int nw, uint32_t *msk,
-                                           float kap0, float kap1)
+                                           const float4 *rec, const float4 *crec, Chunk *sv,
+                                           const TileBoxes &tb, uint32_t *msk, float kap0, float kap1)
 {
+    bool gen = false;
     for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
         const uint32_t gid = __ldg(gids + base + (uint32_t)i * stride);
         VRec vr;
         prep_record<GM, KER>(g, F, gid, rec, crec, vr, kap0, kap1);
-        if (TOF) {
+        if constexpr (TOF) {
             // time of flight (parallel rays): the pair's value times the
             // kernel of width s^2 = 1/A + sigma_T^2 at t* - t_k (the
             // convolution of the Gaussian's profile along the ray with the
@@ -179,139 +156,98 @@ __device__ __forceinline__ void prep_chunk(const DevGeom &g, const float *F, con
             vr.c2.z = vr.t4.z;
         }
         sv->c0[i] = vr.c0;
-        sv->c1[i] = vr.c1;
-        sv->c2[i] = vr.c2;
+        if constexpr (GM == GM_PARALLEL && !TOF) {
+            sv->va[i] = make_float2(vr.c1.x, vr.c2.w);
+        } else {
+            sv->c1[i] = vr.c1;
+            sv->c2[i] = vr.c2;
+        }
         sv->gid[i] = gid;
         const float4 bb = vr.bb;
-        // a block inside the footprint's box may still miss the footprint
-        // ellipse: skip it when the tangent plane of G at the block centre
-        // stays above tol over the block (a pair with m <= 9 + 9e-4 has
-        // G <= -0.19 A < 0 at K^2 = 9.2, so none is lost).  Cone beam only:
-        // the small footprints of the parallel-ray workloads fill their boxes'
-        // blocks, and the test there cost more than it saved.
-        Conic cn;
-        cn.ok = false;
-        float u0 = 0.0f, v0 = 0.0f;
-        if (GM == GM_CONE) {
-            cn = cone_conic<KER>(vr);
-            u0 = vr.c0.x;
-            v0 = vr.c0.y;
-        }
-        const float tol = 1e-3f * fabsf(cn.f);
         uint32_t m = 0;
-        for (int w = 0; w < (HalfBlocks<GM>::value ? 2 * nw : nw); w++) {
-            const float4 wb = wbox[w];
-            bool hit = !(bb.y < wb.x || bb.x > wb.y || bb.w < wb.z || bb.z > wb.w);
-            if (GM == GM_CONE && hit && cn.ok) {
-                const float cu = 0.5f * (wb.x + wb.y) - u0, cv = 0.5f * (wb.z + wb.w) - v0;
-                const float hu = 0.5f * (wb.y - wb.x), hv = 0.5f * (wb.w - wb.z);
-                const float gu = cn.a * cu + cn.b * cv + cn.d, gv = cn.b * cu + cn.c * cv + cn.e;
-                const float G = cu * (gu + cn.d) + cv * (gv + cn.e) + cn.f;
-                hit = G - 2.0f * (fabsf(gu) * hu + fabsf(gv) * hv) <= tol;
+        if (GM == GM_CONE) {
+            // a block inside the footprint's box may still miss the footprint
+            // ellipse: skip it when the tangent plane of G at the block centre
+            // stays above tol over the block (a pair with m <= 9 + 9e-4 has
+            // G <= -0.19 A < 0 at K^2 = 9.2, so none is lost).  Cone beam only:
+            // the small footprints of the parallel-ray workloads fill their
+            // boxes' blocks, and the test there cost more than it saved.
+            const Conic cn = cone_conic<KER>(vr);
+            const float u0 = vr.c0.x, v0 = vr.c0.y, tol = 1e-3f * fabsf(cn.f);
+            for (int w = 0; w < tb.ncb * tb.nrb; w++) {
+                const float4 wb = tb.wbox[w];
+                bool hit = !(bb.y < wb.x || bb.x > wb.y || bb.w < wb.z || bb.z > wb.w);
+                if (hit && cn.ok) {
+                    const float cu = 0.5f * (wb.x + wb.y) - u0, cv = 0.5f * (wb.z + wb.w) - v0;
+                    const float hu = 0.5f * (wb.y - wb.x), hv = 0.5f * (wb.w - wb.z);
+                    const float gu = cn.a * cu + cn.b * cv + cn.d, gv = cn.b * cu + cn.c * cv + cn.e;
+                    const float G = cu * (gu + cn.d) + cv * (gv + cn.e) + cn.f;
+                    hit = G - 2.0f * (fabsf(gu) * hu + fabsf(gv) * hv) <= tol;
+                }
+                m |= (uint32_t)hit << w;
             }
-            m |= (uint32_t)hit << w;
+        } else {
+            // the blocks are a grid: those hit are columns hit x rows hit
+            uint32_t cm = 0;
+            for (int c = 0; c < tb.ncb; c++) {
+                const float2 x = tb.cu[c];
+                cm |= (uint32_t)!(bb.y < x.x || bb.x > x.y) << c;
+            }
+            for (int r = 0; r < tb.nrb; r++) {
+                const float2 x = tb.rv[r];
+                m |= bb.w < x.x || bb.z > x.y ? 0u : cm << (r * tb.ncb);
+            }
         }
         if (vr.g2.w != 0.0f) m |= MSK_VS;
+        else gen = true;
         msk[i] = m;
     }
+    return gen;
 }
 
-// warp-private compaction; returns the list lengths in nvs, ngen
-// nvs, ngen: the lengths of this lane's lists
-template <bool HALF>
-__device__ __forceinline__ void build_lists(int cnt, const uint32_t *msk, ChunkLists &L, int w,
+// warp-private compaction into the lists of the warp's groups; returns the
+// lengths of this lane's lists
+template <int GM>
+__device__ __forceinline__ void build_lists(int cnt, const uint32_t *msk, bool any_gen, ChunkLists &L, int w,
                                             int lane, int &nvs, int &ngen)
 {
+    constexpr int PW = Blocks<GM>::PER_WARP;
     const uint32_t lt = (1u << lane) - 1u;
-    if (!HALF) {
-        nvs = 0;
-        ngen = 0;
-        for (int b = 0; b < cnt; b += 32) {
-            const int i = b + lane;
-            const uint32_t m = i < cnt ? msk[i] : 0u;
-            const bool in = (m >> w) & 1u;
-            const bool vs = (m & MSK_VS) != 0u;
-            const uint32_t bv = __ballot_sync(0xffffffffu, in && vs);
-            const uint32_t bg = __ballot_sync(0xffffffffu, in && !vs);
-            if (in && vs) L.vs[w][nvs + __popc(bv & lt)] = (uint8_t)i;
-            if (in && !vs) L.gen[w][ngen + __popc(bg & lt)] = (uint8_t)i;
-            nvs += __popc(bv);
-            ngen += __popc(bg);
-        }
-        __syncwarp();
-        return;
-    }
-    int v0 = 0, v1 = 0, g0 = 0, g1 = 0;
+    const int mine = lane / Blocks<GM>::LANES;
+    nvs = 0;
+    ngen = 0;
+    int n[PW], ng[PW];
+#pragma unroll
+    for (int q = 0; q < PW; q++) n[q] = ng[q] = 0;
     for (int b = 0; b < cnt; b += 32) {
         const int i = b + lane;
-        const uint32_t m = i < cnt ? msk[i] : 0u;
-        const bool in0 = (m >> (2 * w)) & 1u, in1 = (m >> (2 * w + 1)) & 1u;
-        const bool vs = (m & MSK_VS) != 0u;
-        const uint32_t bv0 = __ballot_sync(0xffffffffu, in0 && vs);
-        const uint32_t bv1 = __ballot_sync(0xffffffffu, in1 && vs);
-        const uint32_t bg0 = __ballot_sync(0xffffffffu, in0 && !vs);
-        const uint32_t bg1 = __ballot_sync(0xffffffffu, in1 && !vs);
-        if (in0 && vs) L.vs[2 * w][v0 + __popc(bv0 & lt)] = (uint8_t)i;
-        if (in1 && vs) L.vs[2 * w + 1][v1 + __popc(bv1 & lt)] = (uint8_t)i;
-        if (in0 && !vs) L.gen[2 * w][g0 + __popc(bg0 & lt)] = (uint8_t)i;
-        if (in1 && !vs) L.gen[2 * w + 1][g1 + __popc(bg1 & lt)] = (uint8_t)i;
-        v0 += __popc(bv0);
-        v1 += __popc(bv1);
-        g0 += __popc(bg0);
-        g1 += __popc(bg1);
+        const uint32_t mk = i < cnt ? msk[i] : 0u;
+        const uint32_t m = mk >> (w * PW);
+        const bool vs = (mk & MSK_VS) != 0u;
+#pragma unroll
+        for (int q = 0; q < PW; q++) {
+            const bool in = ((m >> q) & 1u) && vs;
+            const uint32_t bal = __ballot_sync(0xffffffffu, in);
+            if (in) L.vs[w * PW + q][n[q] + __popc(bal & lt)] = (uint8_t)i;
+            n[q] += __popc(bal);
+        }
+        if (any_gen) {
+#pragma unroll
+            for (int q = 0; q < PW; q++) {
+                const bool in = ((m >> q) & 1u) && !vs;
+                const uint32_t bal = __ballot_sync(0xffffffffu, in);
+                if (in) L.gen[w * PW + q][ng[q] + __popc(bal & lt)] = (uint8_t)i;
+                ng[q] += __popc(bal);
+            }
+        }
     }
     __syncwarp();
-    const bool h = lane >= 16;
-    nvs = h ? v1 : v0;
-    ngen = h ? g1 : g0;
-}
-
-// the warps' detector boxes, wbox[w] (HALF: the half-warps', wbox[2w + h])
-template <bool HALF>
-__device__ __forceinline__ void warp_box(const TileCtx &c, float4 *wbox)
-{
-    if ((threadIdx.x & (HALF ? 15 : 31)) == 0)
-        wbox[threadIdx.x >> (HALF ? 4 : 5)] = make_float4(c.wu_lo, c.wu_hi, c.wv_lo, c.wv_hi);
-}
-
-// view-space value of one pair (without the |d~| factor of cone beam and
-// 3-D PET); returns arg = QSCALE m (Gaussian: -m log2(e)/2; Epanechnikov:
-// -m/kappa^2).  kap: the ray's slope (3-D PET).
-template <int GM, int KER, class R>
-__device__ __forceinline__ float vs_value(const R &r, float u, float v, float kap, float &arg)
-{
-    const float4 c0 = r.c0, c1 = r.c1, c2 = r.c2;
-    float rA = 1.0f;
-    if (GM == GM_PET3D) {
-        const float du = u - c0.x, vt = fmaf(kap, c0.z, v - c0.y);
-        const float muu = fmaf(fmaf(c1.z, kap, c1.y), kap, c1.x);
-        const float muv2 = fmaf(c2.x, kap, c1.w);
-        const float q = du * (muu * du + muv2 * vt) + c0.w * vt * vt;
-        const float An = fmaf(fmaf(c2.z, kap, c2.y), kap, 1.0f);
-        rA = rsqrt_approx(An);
-        arg = q * (rA * rA);
-        if (KER == 1) {
-            const float c = 1.0f + arg;
-            const float pc = c > 0.0f ? c * sqrt_approx(c) : 0.0f;
-            return c2.w * rA * pc;
+#pragma unroll
+    for (int q = 0; q < PW; q++)
+        if (q == mine) {
+            nvs = n[q];
+            ngen = ng[q];
         }
-        return c2.w * rA * ex2_approx(arg);
-    }
-    const float du = u - c0.x, dv = v - c0.y;
-    const float q = du * (c0.z * du + c0.w * dv) + c1.x * dv * dv;
-    if (GM == GM_CONE) {
-        const float A = c1.y + du * (c1.z + c2.x * du + c2.y * dv) + dv * (c1.w + c2.z * dv);
-        rA = rsqrt_approx(A);
-        arg = q * (rA * rA);
-    } else {
-        arg = q;
-    }
-    if (KER == 1) {
-        const float c = 1.0f + arg;                      // 1 - m / kappa^2
-        const float pc = c > 0.0f ? c * sqrt_approx(c) : 0.0f;
-        return c2.w * rA * pc;
-    }
-    return c2.w * rA * ex2_approx(arg);
 }
 
 // the pair counts (Gaussian: m <= 9; Epanechnikov: inside the support)
@@ -321,129 +257,326 @@ __device__ __forceinline__ bool vs_keep(float arg)
     return KER == 1 ? arg > -1.0f : arg >= CUT_ARG;
 }
 
-// forward integration of tile `tile` of geometry g (one ray per thread)
-template <int GM, bool STATS, int KER, bool TOF = false>
-__device__ __forceinline__ void forward_tile(const DevGeom &g, uint32_t tile,
+// kernel profile of both pairs, arg = QSCALE m (Gaussian: -m log2(e)/2;
+// Epanechnikov: -m/kappa^2)
+template <int KER>
+__device__ __forceinline__ f2 profile2(float a0, float a1)
+{
+    if (KER == 1) {
+        const float x = 1.0f + a0, y = 1.0f + a1;        // 1 - m / kappa^2
+        return pk(x > 0.0f ? x * sqrt_approx(x) : 0.0f, y > 0.0f ? y * sqrt_approx(y) : 0.0f);
+    }
+    return pk(ex2_approx(a0), ex2_approx(a1));
+}
+
+// View-space values of a record for the lane's two rays (without the |d~|
+// factor of cone beam and 3-D PET).  u, v: the rays' coordinates; kap: their
+// slope (3-D PET).
+__device__ __forceinline__ f2 quad2(float Muu, float Muv2, float Mvv, f2 du, float dv)
+{
+    // du (Muu du + 2 Muv dv) + Mvv dv dv
+    const f2 t = fma2(pk(Muu, Muu), du, pk(Muv2 * dv, Muv2 * dv));
+    const float s = Mvv * dv * dv;
+    return fma2(du, t, pk(s, s));
+}
+
+template <int KER>
+__device__ __forceinline__ f2 value_parallel(const float4 &c0, float Mvv, float alpha, f2 u, float v, float &a0,
+                                             float &a1)
+{
+    const f2 du = add2(u, pk(-c0.x, -c0.x));
+    up(quad2(c0.z, c0.w, Mvv, du, v - c0.y), a0, a1);
+    return mul2(pk(alpha, alpha), profile2<KER>(a0, a1));
+}
+
+template <int KER>
+__device__ __forceinline__ f2 value_cone(const float4 &c0, const float4 &c1, const float4 &c2, f2 u, float v,
+                                         float &a0, float &a1)
+{
+    const f2 du = add2(u, pk(-c0.x, -c0.x));
+    const float dv = v - c0.y;
+    const f2 q = quad2(c0.z, c0.w, c1.x, du, dv);
+    // A = c1.y + du (c1.z + c2.x du + c2.y dv) + dv (c1.w + c2.z dv)
+    const f2 DV = pk(dv, dv);
+    const f2 in = fma2(pk(c2.y, c2.y), DV, fma2(pk(c2.x, c2.x), du, pk(c1.z, c1.z)));
+    const float ot = fmaf(c2.z, dv, c1.w);
+    float x, y;
+    up(fma2(DV, pk(ot, ot), fma2(du, in, pk(c1.y, c1.y))), x, y);
+    const f2 rA = pk(rsqrt_approx(x), rsqrt_approx(y));
+    up(mul2(q, mul2(rA, rA)), a0, a1);
+    return mul2(mul2(pk(c2.w, c2.w), rA), profile2<KER>(a0, a1));
+}
+
+template <int KER>
+__device__ __forceinline__ f2 value_pet3d(const float4 &c0, const float4 &c1, const float4 &c2, float u, f2 v,
+                                          float kap, float &a0, float &a1)
+{
+    const float du = u - c0.x;
+    const float muu = fmaf(fmaf(c1.z, kap, c1.y), kap, c1.x), muv2 = fmaf(c2.x, kap, c1.w);
+    const f2 vt = fma2(pk(kap, kap), pk(c0.z, c0.z), add2(v, pk(-c0.y, -c0.y)));
+    // du (muu du + muv2 v~) + S_uu v~ v~
+    const f2 DU = pk(du, du);
+    const f2 t = fma2(pk(muu, muu), DU, mul2(pk(muv2, muv2), vt));
+    const f2 q = fma2(mul2(pk(c0.w, c0.w), vt), vt, mul2(DU, t));
+    const float rA = rsqrt_approx(fmaf(fmaf(c2.z, kap, c2.y), kap, 1.0f));
+    const float iA = rA * rA, al = c2.w * rA;
+    up(mul2(q, pk(iA, iA)), a0, a1);
+    return mul2(pk(al, al), profile2<KER>(a0, a1));
+}
+
+// Forward integration of tile `tile` of geometry g (two rays per thread).  A
+// tile's list may be cut into `parts`: part p takes every parts-th chunk, and a
+// ray's sum is that of the parts, added in their order.  They belong to the
+// CTAs of a cluster, the first adding the others' sums read from their shared
+// memory, or (SEQ) to this CTA one after the other, with the same result.
+template <int GM, bool STATS, int KER, bool TOF = false, bool SEQ = false>
+__device__ __forceinline__ void forward_tile(const DevGeom &g, uint32_t tile, uint32_t part, uint32_t parts,
                                              const float4 *__restrict__ rec,
                                              const float4 *__restrict__ crec,
                                              const uint32_t *__restrict__ gids,
                                              const uint2 *__restrict__ ranges,
                                              float *__restrict__ out, Stats *stats)
 {
-    __shared__ SChunk sv_buf[NBUF];
+    using B = Blocks<GM>;
+    constexpr bool CONE = GM == GM_CONE, P3 = GM == GM_PET3D, WIDE = GM != GM_PARALLEL || TOF;
+    __shared__ SChunk<WIDE> sv_buf[NBUF];
     __shared__ ChunkLists lists;
     __shared__ uint32_t msk_buf[NBUF][CH];
-    __shared__ float4 wbox[16];
+    __shared__ TileBoxes tb;
     __shared__ float Fs[9];
-    constexpr bool CONE = GM == GM_CONE;
-    const TileCtx c = tile_ctx<GM>(g, tile);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    constexpr bool HALF = HalfBlocks<GM>::value;
-    const int hw = HALF ? threadIdx.x >> 4 : w;   // this lane's lists
-    if (threadIdx.x < 9) Fs[threadIdx.x] = __ldg(g.frames + 9 * (size_t)c.view + threadIdx.x);
-    warp_box<HALF>(c, wbox);
+    __shared__ int s_gen[2];
+    const int T = g.tiles_x * g.tiles_y;
+    const int vl = (int)(tile / (uint32_t)T);
+    const int tin = (int)tile - vl * T;
+    const int ty = tin / g.tiles_x, tx = tin - ty * g.tiles_x;
+    const int view = g.v0 + vl, tc0 = tx * g.tile_w, tr0 = ty * g.tile_h;
+    int rows = g.n_rows;                // rows with a ray
+    float zoff = 0.0f, dz = 0.0f, kap0 = 0.0f, kap1 = 0.0f;
+    if (P3) {
+        pet3d_view(g, view, zoff, dz, rows);
+        pet3d_slopes(g, dz, tc0, min(tc0 + g.tile_w - 1, g.n_cols - 1), kap0, kap1);
+    }
+    const int ncb = g.tile_w / B::BWID, nrb = g.tile_h >> 2;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int blk = w * B::PER_WARP + lane / B::LANES;     // this lane's block (and list)
+    // the lane's two rays
+    const int l = lane & (B::LANES - 1);
+    const int lc = P3 ? l & 3 : 2 * (l & (B::BWID / 2 - 1)), lr = P3 ? 2 * (l >> 2) : l / (B::BWID / 2);
+    const int by = blk / ncb, col = tc0 + (blk - by * ncb) * B::BWID + lc, row = tr0 + 4 * by + lr;
+    const int col1 = col + (P3 ? 0 : 1), row1 = row + (P3 ? 1 : 0);
+    const bool in = blk < ncb * nrb;
+    const bool valid0 = in && col < g.n_cols && row < g.n_rows, valid1 = in && col1 < g.n_cols && row1 < g.n_rows;
+    const bool live0 = valid0 && row < rows, live1 = valid1 && row1 < rows;
+    // the blocks' detector boxes (empty past the detector or the last ring pair)
+    if (threadIdx.x < 9) Fs[threadIdx.x] = __ldg(g.frames + 9 * (size_t)view + threadIdx.x);
+    if (threadIdx.x < ncb) {
+        const int c = tc0 + threadIdx.x * B::BWID;
+        tb.cu[threadIdx.x] = c < g.n_cols ? make_float2(__ldg(g.utab + c), __ldg(g.utab + min(c + B::BWID - 1, g.n_cols - 1)))
+                                          : make_float2(INFINITY, -INFINITY);
+    }
+    if (threadIdx.x >= 16 && threadIdx.x < 16 + nrb) {
+        const int r = tr0 + 4 * ((int)threadIdx.x - 16);
+        tb.rv[threadIdx.x - 16] = r < rows ? make_float2(__ldg(g.vtab + r) + zoff, __ldg(g.vtab + min(r + 3, rows - 1)) + zoff)
+                                           : make_float2(INFINITY, -INFINITY);
+    }
+    if (threadIdx.x == 0) {
+        tb.ncb = ncb;
+        tb.nrb = nrb;
+        s_gen[0] = s_gen[1] = 0;
+    }
     __syncthreads();
+    if (CONE) {
+        if (threadIdx.x < ncb * nrb) {
+            const float2 a = tb.cu[threadIdx.x % ncb], b = tb.rv[threadIdx.x / ncb];
+            const bool none = a.x > a.y || b.x > b.y;
+            tb.wbox[threadIdx.x] = none ? make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY)
+                                        : make_float4(a.x, a.y, b.x, b.y);
+        }
+        __syncthreads();
+    }
     float F[9];
 #pragma unroll
     for (int i = 0; i < 9; i++) F[i] = Fs[i];
-    const float u = __ldg(g.utab + min(c.col, g.n_cols - 1));
-    const float v = __ldg(g.vtab + min(c.row, g.n_rows - 1)) + c.zoff;
-    const float kap = GM == GM_PET3D ? pet3d_slope(g, c.dz, u) : 0.0f;
-    const float L = CONE ? sqrtf(u * u + v * v + g.dsd * g.dsd)
-                  : GM == GM_PET3D ? sqrtf(1.0f + kap * kap) : 1.0f;
+    const float u0 = __ldg(g.utab + min(col, g.n_cols - 1)), u1 = __ldg(g.utab + min(col1, g.n_cols - 1));
+    const float v0 = __ldg(g.vtab + min(row, g.n_rows - 1)) + zoff, v1 = __ldg(g.vtab + min(row1, g.n_rows - 1)) + zoff;
+    const f2 U = pk(u0, u1), V = pk(v0, v1);
+    const float kap = P3 ? pet3d_slope(g, dz, u0) : 0.0f;
     const uint2 rg = ranges[tile];
-    float acc_vs = 0.0f, acc_gen = 0.0f;
+    f2 acc = 0;
+    float gen0 = 0.0f, gen1 = 0.0f;
     // time of flight (parallel rays, Gaussian kernel): one sum per bin
-    float acc_t[TOF ? TOF_MAX : 1];
+    f2 acc_t[TOF ? TOF_MAX : 1];
 #pragma unroll
-    for (int q = 0; q < (TOF ? TOF_MAX : 1); q++) acc_t[q] = 0.0f;
-    unsigned n_eval = 0, n_kept = 0;
+    for (int q = 0; q < (TOF ? TOF_MAX : 1); q++) acc_t[q] = 0;
+    unsigned n_eval = 0, n_kept0 = 0, n_kept1 = 0;
     // chunk c takes list entries c, c + nch, c + 2 nch, ...: the lists are
     // ordered by footprint position, and interleaving spreads every chunk
-    // over the whole tile, which keeps the warps' shares of it even
+    // over the whole tile, which keeps the groups' shares of it even
     const uint32_t nlist = rg.y - rg.x;
-    const uint32_t nch = (nlist + CH - 1) / CH;
-    for (uint32_t ch = 0; ch < nch; ch++) {
-        const int cnt = (int)((nlist - ch + nch - 1) / nch);
-        const SChunk &sv = sv_buf[ch % NBUF];
-        uint32_t *msk = msk_buf[ch % NBUF];
-        prep_chunk<GM, KER, TOF>(g, F, gids, rg.x + ch, nch, cnt, rec, crec, &sv_buf[ch % NBUF], wbox, nw, msk,
-                                 c.kap0, c.kap1);
+    const uint32_t nch = ((nlist + CH - 1) / CH + parts - 1) / parts * parts;
+    f2 sum = 0, gsum = 0;      // SEQ: the parts before
+    int buf = 0;
+next_part:
+    for (uint32_t ch = part; ch < nch; ch += parts, buf ^= 1) {
+        const int cnt = nlist > ch ? (int)((nlist - ch + nch - 1) / nch) : 0;
+        const SChunk<WIDE> &sv = sv_buf[buf];
+        uint32_t *msk = msk_buf[buf];
+        if (prep_chunk<GM, KER, TOF>(g, F, gids, rg.x + ch, nch, cnt, rec, crec, &sv_buf[buf], tb, msk, kap0, kap1))
+            s_gen[buf] = 1;
         // every thread has prepared this chunk and (with two buffers) left the
         // previous one, whose buffer the next chunk's preparation reuses
         __syncthreads();
+        const bool any_gen = s_gen[buf] != 0;
         int nvs, ngen;
-        build_lists<HALF>(cnt, msk, lists, w, lane, nvs, ngen);
-        int k = 0;
-        if (TOF) {
-            for (; k < nvs; k++) {
-                const SRec r = sv[lists.vs[hw][k]];
-                float a0;
-                const float v0 = vs_value<GM, KER>(r, u, v, kap, a0);
-                if (STATS) n_kept += vs_keep<KER>(a0);
-                if (!vs_keep<KER>(a0)) continue;
-                const float ts = r.c2.x + r.c2.y * (u - r.c0.x) + r.c2.z * (v - r.c0.y) - g.tof_t0;
-                const float vn = v0 * r.c1.z;
+        build_lists<GM>(cnt, msk, any_gen, lists, w, lane, nvs, ngen);
+        const uint8_t *lst = lists.vs[blk & (B::MAX - 1)];
+        if constexpr (TOF) {
+            for (int k = 0; k < nvs; k++) {
+                const int j = lst[k];
+                const float4 c0 = sv.c0[j], c1 = sv.c1[j], c2 = sv.c2[j];
+                float a0, a1;
+                const f2 val = value_parallel<KER>(c0, c1.x, c2.w, U, v0, a0, a1);
+                const bool k0 = vs_keep<KER>(a0), k1 = vs_keep<KER>(a1);
+                if (STATS) {
+                    n_kept0 += k0;
+                    n_kept1 += k1;
+                }
+                if (!k0 && !k1) continue;
+                float x0, x1;
+                up(mul2(val, pk(c1.z, c1.z)), x0, x1);
+                const f2 vn = pk(k0 ? x0 : 0.0f, k1 ? x1 : 0.0f);
+                // t* - t_0, then one bin after the other
+                const float dv = v0 - c0.y;
+                const float t0 = fmaf(c2.z, dv, fmaf(c2.y, u0 - c0.x, c2.x)) - g.tof_t0;
+                const float t1 = fmaf(c2.z, dv, fmaf(c2.y, u1 - c0.x, c2.x)) - g.tof_t0;
+                const f2 ts = pk(t0, t1), H = pk(g.tof_h, g.tof_h), S = pk(c1.y, c1.y);
 #pragma unroll
                 for (int b = 0; b < TOF_MAX; b++) {
                     if (b >= g.n_tof) break;
-                    const float x = ts - (float)b * g.tof_h;
-                    acc_t[b] = fmaf(vn, ex2_approx(r.c1.y * x * x), acc_t[b]);
+                    const f2 x = fma2(pk(-(float)b, -(float)b), H, ts);
+                    float y0, y1;
+                    up(mul2(mul2(S, x), x), y0, y1);
+                    acc_t[b] = fma2(vn, pk(ex2_approx(y0), ex2_approx(y1)), acc_t[b]);
+                }
+            }
+        } else {
+            for (int k = 0; k < nvs; k++) {
+                const int j = lst[k];
+                float a0, a1;
+                f2 val;
+                if constexpr (GM == GM_PARALLEL) {
+                    const float2 va = sv.va[j];
+                    val = value_parallel<KER>(sv.c0[j], va.x, va.y, U, v0, a0, a1);
+                } else if constexpr (CONE) {
+                    val = value_cone<KER>(sv.c0[j], sv.c1[j], sv.c2[j], U, v0, a0, a1);
+                } else {
+                    val = value_pet3d<KER>(sv.c0[j], sv.c1[j], sv.c2[j], u0, V, kap, a0, a1);
+                }
+                float x0, x1;
+                up(val, x0, x1);
+                acc = add2(acc, pk(vs_keep<KER>(a0) ? x0 : 0.0f, vs_keep<KER>(a1) ? x1 : 0.0f));
+                if (STATS) {
+                    n_kept0 += vs_keep<KER>(a0);
+                    n_kept1 += vs_keep<KER>(a1);
                 }
             }
         }
-        for (; k + 1 < nvs; k += 2) {
-            const int j0 = lists.vs[hw][k], j1 = lists.vs[hw][k + 1];
-            float a0, a1;
-            const float v0 = vs_value<GM, KER>(sv[j0], u, v, kap, a0);
-            const float v1 = vs_value<GM, KER>(sv[j1], u, v, kap, a1);
-            acc_vs += vs_keep<KER>(a0) ? v0 : 0.0f;
-            acc_vs += vs_keep<KER>(a1) ? v1 : 0.0f;
-            if (STATS) n_kept += vs_keep<KER>(a0) + vs_keep<KER>(a1);
-        }
-        if (k < nvs) {
-            float a0;
-            const float v0 = vs_value<GM, KER>(sv[lists.vs[hw][k]], u, v, kap, a0);
-            acc_vs += vs_keep<KER>(a0) ? v0 : 0.0f;
-            if (STATS) n_kept += vs_keep<KER>(a0);
-        }
         if (ngen > 0) {
-            const Ray ray = make_ray<GM>(g, F, u, v, kap);
             for (int k2 = 0; k2 < ngen; k2++) {
-                const GRec r = load_grec(rec, sv.gid[lists.gen[hw][k2]]);
-                PairGeo q;
-                pair_geo(ray, r, q);
-                if (STATS) n_kept += q.m <= PAIR_CUT2;
-                if (TOF) {
-                    if (q.m <= PAIR_CUT2) {
+                const GRec r = load_grec(rec, sv.gid[lists.gen[blk & (B::MAX - 1)][k2]]);
+                for (int e = 0; e < 2; e++) {
+                    const Ray ray = make_ray<GM>(g, F, e ? u1 : u0, e ? v1 : v0, kap);
+                    PairGeo q;
+                    pair_geo(ray, r, q);
+                    if (STATS) (e ? n_kept1 : n_kept0) += q.m <= PAIR_CUT2;
+                    if (!(q.m <= PAIR_CUT2)) continue;
+                    if constexpr (TOF) {
 #pragma unroll
                         for (int b = 0; b < TOF_MAX; b++) {
                             if (b >= g.n_tof) break;
-                            acc_t[b] += general_value<KER>(q, r.g0.w, g.tof_t0 + (float)b * g.tof_h, g.tof_tau);
+                            const float x = general_value<KER>(q, r.g0.w, g.tof_t0 + (float)b * g.tof_h, g.tof_tau);
+                            acc_t[b] = add2(acc_t[b], pk(e ? 0.0f : x, e ? x : 0.0f));
                         }
+                    } else {
+                        (e ? gen1 : gen0) += general_value<KER>(q, r.g0.w);
                     }
-                    continue;
                 }
-                const float val = general_value<KER>(q, r.g0.w);
-                acc_gen += q.m <= PAIR_CUT2 ? val : 0.0f;
             }
         }
         if (STATS) n_eval += nvs + ngen;
-        if (NBUF == 1) __syncthreads();
+        // this chunk's flag is read; the next use of it is two chunks on
+        if (any_gen) {
+            __syncthreads();
+            if (threadIdx.x == 0) s_gen[buf] = 0;
+        }
     }
-    if (TOF) {
-        if (c.valid) {
+    if (SEQ && parts > 1) {
+        const f2 gg = pk(gen0, gen1);
+        sum = part == 0 ? acc : add2(sum, acc);
+        gsum = part == 0 ? gg : add2(gsum, gg);
+        if (++part < parts) {
+            acc = 0;
+            gen0 = gen1 = 0.0f;
+            goto next_part;
+        }
+        acc = sum;
+        up(gsum, gen0, gen1);
+        part = 0;
+    }
+    if (!SEQ && parts > 1) {
+        // per thread: the sums of its two rays (TOF: bin by bin), in the chunk buffers
+        constexpr int NS = TOF ? TOF_MAX : 2;
+        f2 *mine = reinterpret_cast<f2 *>(&sv_buf[0]);
+        static_assert(sizeof(sv_buf) >= sizeof(f2) * NS * FBS, "a thread's sums fit the chunk buffers");
+        __syncthreads();
+        if constexpr (TOF) {
 #pragma unroll
-            for (int b = 0; b < TOF_MAX; b++) {
-                if (b >= g.n_tof) break;
-                out[c.out_idx + (long long)b * g.stride_tof] = c.live ? acc_t[b] : 0.0f;
+            for (int b = 0; b < TOF_MAX; b++) mine[b * FBS + threadIdx.x] = acc_t[b];
+        } else {
+            mine[threadIdx.x] = acc;
+            mine[FBS + threadIdx.x] = pk(gen0, gen1);
+        }
+        cg::cluster_group cluster = cg::this_cluster();
+        cluster.sync();
+        if (part == 0) {
+            for (uint32_t r = 1; r < parts; r++) {
+                const f2 *o = cluster.map_shared_rank(mine, r);
+                if constexpr (TOF) {
+#pragma unroll
+                    for (int b = 0; b < TOF_MAX; b++) acc_t[b] = add2(acc_t[b], o[b * FBS + threadIdx.x]);
+                } else {
+                    float x, y;
+                    acc = add2(acc, o[threadIdx.x]);
+                    up(o[FBS + threadIdx.x], x, y);
+                    gen0 += x;
+                    gen1 += y;
+                }
             }
         }
-    } else if (c.valid) {
-        out[c.out_idx] = c.live ? acc_gen + L * acc_vs : 0.0f;
+        cluster.sync();   // the others' shared memory stays until it has been read
+    }
+    const bool store0 = valid0 && part == 0, store1 = valid1 && part == 0;
+    const long long i0 = (long long)view * g.stride_view + (long long)row * g.stride_row + col;
+    const long long i1 = (long long)view * g.stride_view + (long long)row1 * g.stride_row + col1;
+    if constexpr (TOF) {
+#pragma unroll
+        for (int b = 0; b < TOF_MAX; b++) {
+            if (b >= g.n_tof) break;
+            float x0, x1;
+            up(acc_t[b], x0, x1);
+            if (store0) out[i0 + (long long)b * g.stride_tof] = x0;
+            if (store1) out[i1 + (long long)b * g.stride_tof] = x1;
+        }
+    } else {
+        float x0, x1;
+        up(acc, x0, x1);
+        const float L0 = CONE ? sqrtf(u0 * u0 + v0 * v0 + g.dsd * g.dsd) : P3 ? sqrtf(1.0f + kap * kap) : 1.0f;
+        const float L1 = CONE ? sqrtf(u1 * u1 + v1 * v1 + g.dsd * g.dsd) : L0;
+        if (store0) out[i0] = live0 ? gen0 + L0 * x0 : 0.0f;
+        if (store1) out[i1] = live1 ? gen1 + L1 * x1 : 0.0f;
     }
     if (STATS) {
-        unsigned long long e = c.live ? n_eval : 0, kk = c.live ? n_kept : 0;
+        unsigned long long e = (live0 ? n_eval : 0) + (live1 ? n_eval : 0), kk = (live0 ? n_kept0 : 0) + (live1 ? n_kept1 : 0);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             e += __shfl_xor_sync(0xffffffffu, e, o);
@@ -457,30 +590,31 @@ __device__ __forceinline__ void forward_tile(const DevGeom &g, uint32_t tile,
 }
 
 template <int GM, bool STATS, int KER>
-__global__ void __launch_bounds__(256, 4) k_forward(DevGeom g, const float4 *__restrict__ rec,
+__global__ void __launch_bounds__(FBS, GM == GM_PARALLEL ? 7 : 6) k_forward(DevGeom g, uint32_t parts, const float4 *__restrict__ rec,
                                                     const float4 *__restrict__ crec,
                                                     const uint32_t *__restrict__ gids,
                                                     const uint2 *__restrict__ ranges,
                                                     float *__restrict__ out, Stats *stats)
 {
-    forward_tile<GM, STATS, KER>(g, blockIdx.x, rec, crec, gids, ranges, out, stats);
+    forward_tile<GM, STATS, KER>(g, blockIdx.x / parts, blockIdx.x % parts, parts, rec, crec, gids, ranges, out, stats);
 }
 
 // time-of-flight sinograms (PET ring, Gaussian kernel): one sum per bin per ray
 template <bool STATS>
-__global__ void __launch_bounds__(256, 2) k_forward_tof(DevGeom g, const float4 *__restrict__ rec,
+__global__ void __launch_bounds__(FBS, 5) k_forward_tof(DevGeom g, uint32_t parts, const float4 *__restrict__ rec,
                                                         const float4 *__restrict__ crec,
                                                         const uint32_t *__restrict__ gids,
                                                         const uint2 *__restrict__ ranges,
                                                         float *__restrict__ out, Stats *stats)
 {
-    forward_tile<GM_PARALLEL, STATS, 0, true>(g, blockIdx.x, rec, crec, gids, ranges, out, stats);
+    forward_tile<GM_PARALLEL, STATS, 0, true>(g, blockIdx.x / parts, blockIdx.x % parts, parts, rec, crec, gids,
+                                              ranges, out, stats);
 }
 
 // Persistent form over a batch of scans: every CTA takes (scan, tile) work
 // items until all are done (next_item).
 template <bool CONE>
-__global__ void __launch_bounds__(256, 4) k_forward_persistent(const ScanDesc *__restrict__ d,
+__global__ void __launch_bounds__(FBS, CONE ? 6 : 7) k_forward_persistent(const ScanDesc *__restrict__ d,
                                                                int nscan, uint32_t total,
                                                                uint32_t *queue)
 {
@@ -488,51 +622,75 @@ __global__ void __launch_bounds__(256, 4) k_forward_persistent(const ScanDesc *_
     int scan;
     while (next_item(d, nscan, total, queue, item, scan)) {
         const ScanDesc &sd = d[scan];
-        forward_tile<CONE ? GM_CONE : GM_PARALLEL, false, 0>(sd.g, item - sd.item_begin, sd.rec, sd.crec, sd.gids, sd.ranges,
+        forward_tile<CONE ? GM_CONE : GM_PARALLEL, false, 0, false, true>(sd.g, item - sd.item_begin, 0, sd.parts, sd.rec, sd.crec, sd.gids, sd.ranges,
                                   sd.out, nullptr);
     }
 }
 
 }  // namespace
 
+namespace {
+// two rays per thread, whole warps
+int forward_threads(int tile_rays) { return (tile_rays / 2 + 31) & ~31; }
+}  // namespace
+
 cudaError_t launch_forward_persistent(bool cone, const ScanDesc *d, int nscan, uint32_t total,
-                                      uint32_t *queue, int tile_threads, int grid, cudaStream_t s)
+                                      uint32_t *queue, int tile_rays, int grid, cudaStream_t s)
 {
     if (total == 0) return cudaSuccess;
-    if (cone) k_forward_persistent<true><<<grid, tile_threads, 0, s>>>(d, nscan, total, queue);
-    else k_forward_persistent<false><<<grid, tile_threads, 0, s>>>(d, nscan, total, queue);
+    const int bs = forward_threads(tile_rays);
+    if (cone) k_forward_persistent<true><<<grid, bs, 0, s>>>(d, nscan, total, queue);
+    else k_forward_persistent<false><<<grid, bs, 0, s>>>(d, nscan, total, queue);
     count_launches(1);
     return cudaGetLastError();
 }
 
-int persistent_grid(bool cone, int tile_threads)
+int persistent_grid(bool cone, int tile_rays)
 {
-    return cone ? grid_for(k_forward_persistent<true>, tile_threads)
-                : grid_for(k_forward_persistent<false>, tile_threads);
+    const int bs = forward_threads(tile_rays);
+    return cone ? grid_for(k_forward_persistent<true>, bs) : grid_for(k_forward_persistent<false>, bs);
 }
 
-cudaError_t launch_forward(const DevGeom &g, int nv, const float4 *rec, const float4 *crec,
+uint32_t forward_parts(int64_t tiles, int64_t entries)
+{
+    uint32_t parts = 1;
+    while (parts < 8 && tiles * parts < SPLIT_CTAS && entries / (tiles * parts) >= SPLIT_LIST) parts *= 2;
+    return parts;
+}
+
+cudaError_t launch_forward(const DevGeom &g, int nv, int64_t entries, const float4 *rec, const float4 *crec,
                            const uint32_t *gids, const uint2 *ranges, float *out, Stats *stats,
                            int ker, cudaStream_t s)
 {
-    unsigned nt = (unsigned)nv * g.tiles_x * g.tiles_y;
-    if (nt == 0) return cudaSuccess;
-    int bs = g.tile_w * g.tile_h;
-#define RGRT_FWD(M, S, K) k_forward<M, S, K><<<nt, bs, 0, s>>>(g, rec, crec, gids, ranges, out, stats)
+    const int64_t nt = (int64_t)nv * g.tiles_x * g.tiles_y;
+    if (nt <= 0) return cudaSuccess;
+    const uint32_t parts = forward_parts(nt, entries);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = parts;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(nt * parts));
+    cfg.blockDim = dim3(forward_threads(g.tile_w * g.tile_h));
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = parts > 1 ? 1 : 0;
+    cudaError_t e;
+#define RGRT_FWD(M, S, K) e = cudaLaunchKernelEx(&cfg, k_forward<M, S, K>, g, parts, rec, crec, gids, ranges, out, stats)
 #define RGRT_FWD_K(M, K) { if (stats) RGRT_FWD(M, true, K); else RGRT_FWD(M, false, K); }
 #define RGRT_FWD_M(K)                                  \
     if (g.kind == GM_CONE) RGRT_FWD_K(GM_CONE, K)      \
     else if (g.kind == GM_PET3D) RGRT_FWD_K(GM_PET3D, K) \
     else RGRT_FWD_K(GM_PARALLEL, K)
     if (g.n_tof > 0) {   // PET ring, Gaussian kernel (checked by the caller)
-        if (stats) k_forward_tof<true><<<nt, bs, 0, s>>>(g, rec, crec, gids, ranges, out, stats);
-        else k_forward_tof<false><<<nt, bs, 0, s>>>(g, rec, crec, gids, ranges, out, stats);
+        if (stats) e = cudaLaunchKernelEx(&cfg, k_forward_tof<true>, g, parts, rec, crec, gids, ranges, out, stats);
+        else e = cudaLaunchKernelEx(&cfg, k_forward_tof<false>, g, parts, rec, crec, gids, ranges, out, stats);
     } else if (ker == 1) { RGRT_FWD_M(1) } else { RGRT_FWD_M(0) }
 #undef RGRT_FWD_M
 #undef RGRT_FWD_K
 #undef RGRT_FWD
     count_launches(1);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace rgrt

@@ -127,7 +127,10 @@ cudaError_t launch_sort_views(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt
                               const unsigned long long *n_dev = nullptr);
 
 // ker: kernel of the primitives (RGRT_KERNEL_GAUSSIAN / RGRT_KERNEL_EPANECHNIKOV)
-cudaError_t launch_forward(const DevGeom &g, int nv, const float4 *rec, const float4 *crec,
+// parts that a tile's list of a launch is cut into, from its tiles and entries
+uint32_t forward_parts(int64_t tiles, int64_t entries);
+// entries: (tile, Gaussian) entries of the views
+cudaError_t launch_forward(const DevGeom &g, int nv, int64_t entries, const float4 *rec, const float4 *crec,
                            const uint32_t *gids, const uint2 *ranges, float *out, Stats *stats,
                            int ker, cudaStream_t s);
 // Gaussian ids in a spatial order (adjoint.cu), from scratch of
@@ -154,16 +157,16 @@ struct ScanDesc {
     float4 *grad;           // adjoint accumulator
     uint32_t item_begin;    // first (scan, tile) work item of the scan
     uint32_t n_items;       // tiles of the scan
+    uint32_t parts;         // of every tile's list (forward_parts)
 };
 // persistent integration (adjoint: cone beam) over every tile of a batch of
-// scans; the queue counter must be zero at launch.  tile_threads = tile_w * tile_h of every
-// scan (one ray per thread).
+// scans; the queue counter must be zero at launch.  tile_rays = tile_w * tile_h of every scan.
 cudaError_t launch_forward_persistent(bool cone, const ScanDesc *d, int nscan, uint32_t total,
-                                      uint32_t *queue, int tile_threads, int grid, cudaStream_t s);
+                                      uint32_t *queue, int tile_rays, int grid, cudaStream_t s);
 cudaError_t launch_adjoint_persistent(int tile_w, const ScanDesc *d, int nscan, uint32_t total, uint32_t *queue,
                                       cudaStream_t s);
 // CTAs of the persistent forward: SMs x resident CTAs per SM
-int persistent_grid(bool cone, int tile_threads);
+int persistent_grid(bool cone, int tile_rays);
 
 cudaError_t launch_param_chain(const float *mu, const float *ls, const float *q, const float *rho,
                                int64_t n, const float4 *grad, float *g_mu, float *g_ls,
