@@ -520,7 +520,7 @@ int adjoint_views(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, int
     dg.v0 = v0;
     PROF("k_adjoint");
     if (dg.kind != GM_PARALLEL)
-        CK(launch_adjoint_tiles(dg, nv, g->rec, g->crec, (const uint32_t *)ctx->vals.p, (const uint2 *)ctx->ranges.p,
+        CK(launch_adjoint_tiles(dg, nv, K, g->rec, g->crec, (const uint32_t *)ctx->vals.p, (const uint2 *)ctx->ranges.p,
                                 dLdI, (float4 *)ctx->grad.p, g->kernel, s));
     else CK(launch_adjoint(dg, nv, g->n, K, (const uint32_t *)ctx->order.p, g->rec, g->crec, (const uint2 *)ctx->rect.p,
                       dLdI, (float4 *)ctx->grad.p, g->kernel, s));

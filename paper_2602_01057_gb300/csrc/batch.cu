@@ -314,7 +314,7 @@ int enqueue_adjoint(rgrt_batch *b, int i, cudaStream_t s)
     DevGeom dg = x.geom->dg;
     dg.v0 = 0;
     if (b->cone) {
-        BK(launch_adjoint_tiles(dg, dg.n_views, x.g->rec, x.g->crec, x.vals, x.ranges, x.dLdI, x.grad,
+        BK(launch_adjoint_tiles(dg, dg.n_views, x.keys, x.g->rec, x.g->crec, x.vals, x.ranges, x.dLdI, x.grad,
                                 RGRT_KERNEL_GAUSSIAN, s));
         return RGRT_OK;
     }

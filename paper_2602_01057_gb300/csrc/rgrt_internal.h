@@ -143,7 +143,7 @@ cudaError_t launch_adjoint(const DevGeom &g, int nv, int64_t n, int64_t entries,
                            const float4 *rec, const float4 *crec, const uint2 *rect, const float *dLdI,
                            float4 *grad, int ker, cudaStream_t s);
 // the same for cone-beam and 3-D PET views, from the tile lists
-cudaError_t launch_adjoint_tiles(const DevGeom &g, int nv, const float4 *rec, const float4 *crec,
+cudaError_t launch_adjoint_tiles(const DevGeom &g, int nv, int64_t entries, const float4 *rec, const float4 *crec,
                                  const uint32_t *gids, const uint2 *ranges, const float *dLdI, float4 *grad,
                                  int ker, cudaStream_t s);
 // one scan of a batch, as the persistent kernels see it
