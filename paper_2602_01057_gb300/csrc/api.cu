@@ -276,10 +276,11 @@ int bin_views(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, int v0,
         if (by_view)
             CK(launch_sort_views(keys, vals, (uint32_t *)ctx->keys_alt.p, (uint32_t *)ctx->vals_alt.p,
                                  (uint32_t)K, lbits + 8, (const uint32_t *)ctx->off.p, N, nv,
-                                 (uint32_t *)ctx->sort_tmp.p, s, &in_alt));
+                                 (uint32_t *)ctx->sort_tmp.p, s, &in_alt, nullptr, sort_shift(dg)));
         else
             CK(launch_sort(keys, vals, (uint32_t *)ctx->keys_alt.p, (uint32_t *)ctx->vals_alt.p,
-                           (uint32_t)K, ceil_log2(T) + 8, (uint32_t *)ctx->sort_tmp.p, s, &in_alt));
+                           (uint32_t)K, ceil_log2(T) + 8, (uint32_t *)ctx->sort_tmp.p, s, &in_alt, nullptr,
+                           sort_shift(dg)));
         if (in_alt) {   // adopt the buffers that hold the result
             std::swap(ctx->keys, ctx->keys_alt);
             std::swap(ctx->vals, ctx->vals_alt);

@@ -260,10 +260,10 @@ int enqueue_bin_scan(rgrt_batch *b, int i, cudaStream_t s)
                        b->d_overflow, s, x.lbits));
         if (x.lbits >= 0)
             BK(launch_sort_views(b->keys, x.vals, b->keys_alt, b->vals_alt, x.cap, x.bits, b->off, x.N,
-                                 dg.n_views, b->sort_tmp, s, nullptr, b->total));
+                                 dg.n_views, b->sort_tmp, s, nullptr, b->total, sort_shift(dg)));
         else
             BK(launch_sort(b->keys, x.vals, b->keys_alt, b->vals_alt, x.cap, x.bits, b->sort_tmp, s, nullptr,
-                           b->total));
+                           b->total, sort_shift(dg)));
         BK(cudaMemsetAsync(x.ranges, 0, sizeof(uint2) * (size_t)x.T, s));
         BK(launch_ranges(b->keys, x.cap, x.ranges, x.T, s, b->total, (uint32_t)x.geom->tiles_per_view,
                          x.lbits));

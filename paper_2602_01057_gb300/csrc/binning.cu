@@ -600,7 +600,7 @@ size_t sort_tmp_elems(uint32_t n, int ns)
 namespace {
 
 cudaError_t sort_passes(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
-                        uint32_t n, int bits, uint32_t *tmp, const SortLayout &L, SortSegs sg,
+                        uint32_t n, int shift0, int bits, uint32_t *tmp, const SortLayout &L, SortSegs sg,
                         cudaStream_t s, bool *in_alt, const unsigned long long *n_dev)
 {
     uint32_t *hist = tmp;
@@ -609,10 +609,10 @@ cudaError_t sort_passes(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint
     unsigned long long *stot = (unsigned long long *)(tmp + L.stot);
     const uint32_t nb = L.nb;
     uint32_t *src_k = keys, *src_v = vals, *dst_k = keys_alt, *dst_v = vals_alt;
-    int passes = (bits + 7) / 8;
+    int passes = (bits - shift0 + 7) / 8;
     if (passes < 1) passes = 1;
     for (int p = 0; p < passes; p++) {
-        int shift = 8 * p;
+        int shift = shift0 + 8 * p;
         k_sort_hist<<<nb, SORT_BS, 0, s>>>(src_k, n, shift, hist, nb, n_dev, sg);
         cudaError_t e = launch_scan(hist, offs, (int64_t)L.hn, stot, stmp, s);
         if (e != cudaSuccess) return e;
@@ -636,17 +636,18 @@ cudaError_t sort_passes(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint
 
 cudaError_t launch_sort(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
                         uint32_t n, int bits, uint32_t *tmp, cudaStream_t s, bool *in_alt,
-                        const unsigned long long *n_dev)
+                        const unsigned long long *n_dev, int shift)
 {
     if (in_alt) *in_alt = false;
     if (n == 0) return cudaSuccess;
-    return sort_passes(keys, vals, keys_alt, vals_alt, n, bits, tmp, sort_layout(n, 0), SortSegs(), s,
+    return sort_passes(keys, vals, keys_alt, vals_alt, n, shift, bits, tmp, sort_layout(n, 0), SortSegs(), s,
                        in_alt, n_dev);
 }
 
 cudaError_t launch_sort_views(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
                               uint32_t n, int bits, const uint32_t *off, int64_t stride, int nv,
-                              uint32_t *tmp, cudaStream_t s, bool *in_alt, const unsigned long long *n_dev)
+                              uint32_t *tmp, cudaStream_t s, bool *in_alt, const unsigned long long *n_dev,
+                              int shift)
 {
     if (in_alt) *in_alt = false;
     if (n == 0 || nv <= 0) return cudaSuccess;
@@ -660,7 +661,7 @@ cudaError_t launch_sort_views(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt
     k_sort_spans<<<(L.nb + 255) / 256, 256, 0, s>>>(L.nb, n, n_dev, sg, span);
     count_launches(2);
     sg.span = span;
-    return sort_passes(keys, vals, keys_alt, vals_alt, n, bits, tmp, L, sg, s, in_alt, n_dev);
+    return sort_passes(keys, vals, keys_alt, vals_alt, n, shift, bits, tmp, L, sg, s, in_alt, n_dev);
 }
 
 cudaError_t launch_ranges(const uint32_t *keys, uint32_t n_keys, uint2 *ranges, uint32_t n_tiles,

@@ -53,12 +53,17 @@ namespace cg = cooperative_groups;
 namespace rgrt {
 namespace {
 
-constexpr int CH = 256;             // records per chunk
+// records per chunk: at most 256 (8-bit list entries); 192 leave room for two
+// more CTAs per SM, which the geometries of small footprints, waiting at the
+// chunk barrier, use (3-D PET forward 61.8 -> 58.7 ms; cone beam 6.27 -> 6.32)
+template <int GM> struct Chunk {
+    static constexpr int N = GM == GM_CONE ? 256 : 192;
+};
 constexpr int FBS = 128;            // most threads of a CTA (two rays each)
 // chunk buffers: with two, a chunk's records are prepared into one buffer
 // while slower warps still read the other, and a single barrier per chunk
 // suffices.  The staged records leave the general-path fields in global
-// memory so that two buffers fit 7 CTAs per SM.
+// memory so that two buffers fit 6 to 8 CTAs per SM.
 constexpr int NBUF = 2;
 // A tile's list is shared by 2, 4 or 8 CTAs of a cluster while the launch has
 // fewer CTAs than SPLIT_CTAS (about 9 waves: tile lists are uneven, and a few
@@ -87,12 +92,11 @@ struct Blocks {
 // preparing threads write consecutive words, free of bank conflicts, and a
 // group of lanes reads one record at a time (broadcast).  Parallel rays need
 // c0, M_vv and the amplitude only.
-template <bool WIDE> struct SChunk;
-template <> struct SChunk<true> {
+template <bool WIDE, int CH> struct SChunk {
     float4 c0[CH], c1[CH], c2[CH];
     uint32_t gid[CH];
 };
-template <> struct SChunk<false> {
+template <int CH> struct SChunk<false, CH> {
     float4 c0[CH];
     float2 va[CH];     // k M_vv, alpha / sqrt(A)
     uint32_t gid[CH];
@@ -118,9 +122,9 @@ __device__ __forceinline__ GRec load_grec(const float4 *__restrict__ rec, uint32
 // blocks into one list per group -- of view-space records, and (rarely) of
 // general ones.  The groups of a warp walk their own lists side by side.
 constexpr uint32_t MSK_VS = 1u << 16;   // msk: the record takes the view-space path
-struct ChunkLists {
-    uint8_t vs[16][CH];
-    uint8_t gen[16][CH];
+template <int NB, int CH> struct ChunkLists {
+    uint8_t vs[NB][CH];
+    uint8_t gen[NB][CH];
 };
 
 // the intervals of the tile's column and row blocks; wbox: every block's box
@@ -131,10 +135,10 @@ struct TileBoxes {
     int ncb, nrb;      // column and row blocks of the tile
 };
 
-template <int GM, int KER, bool TOF, class Chunk>
+template <int GM, int KER, bool TOF, class Staged>
 __device__ __forceinline__ bool prep_chunk(const DevGeom &g, const float *F, const uint32_t *gids,
                                            uint32_t base, uint32_t stride, int cnt,
-                                           const float4 *rec, const float4 *crec, Chunk *sv,
+                                           const float4 *rec, const float4 *crec, Staged *sv,
                                            const TileBoxes &tb, uint32_t *msk, float kap0, float kap1)
 {
     bool gen = false;
@@ -207,8 +211,8 @@ __device__ __forceinline__ bool prep_chunk(const DevGeom &g, const float *F, con
 
 // warp-private compaction into the lists of the warp's groups; returns the
 // lengths of this lane's lists
-template <int GM>
-__device__ __forceinline__ void build_lists(int cnt, const uint32_t *msk, bool any_gen, ChunkLists &L, int w,
+template <int GM, class Lists>
+__device__ __forceinline__ void build_lists(int cnt, const uint32_t *msk, bool any_gen, Lists &L, int w,
                                             int lane, int &nvs, int &ngen)
 {
     constexpr int PW = Blocks<GM>::PER_WARP;
@@ -339,8 +343,9 @@ __device__ __forceinline__ void forward_tile(const DevGeom &g, uint32_t tile, ui
 {
     using B = Blocks<GM>;
     constexpr bool CONE = GM == GM_CONE, P3 = GM == GM_PET3D, WIDE = GM != GM_PARALLEL || TOF;
-    __shared__ SChunk<WIDE> sv_buf[NBUF];
-    __shared__ ChunkLists lists;
+    constexpr int CH = Chunk<GM>::N;
+    __shared__ SChunk<WIDE, CH> sv_buf[NBUF];
+    __shared__ ChunkLists<B::MAX, CH> lists;
     __shared__ uint32_t msk_buf[NBUF][CH];
     __shared__ TileBoxes tb;
     __shared__ float Fs[9];
@@ -419,7 +424,7 @@ __device__ __forceinline__ void forward_tile(const DevGeom &g, uint32_t tile, ui
 next_part:
     for (uint32_t ch = part; ch < nch; ch += parts, buf ^= 1) {
         const int cnt = nlist > ch ? (int)((nlist - ch + nch - 1) / nch) : 0;
-        const SChunk<WIDE> &sv = sv_buf[buf];
+        const SChunk<WIDE, CH> &sv = sv_buf[buf];
         uint32_t *msk = msk_buf[buf];
         if (prep_chunk<GM, KER, TOF>(g, F, gids, rg.x + ch, nch, cnt, rec, crec, &sv_buf[buf], tb, msk, kap0, kap1))
             s_gen[buf] = 1;
@@ -590,7 +595,7 @@ next_part:
 }
 
 template <int GM, bool STATS, int KER>
-__global__ void __launch_bounds__(FBS, GM == GM_PARALLEL ? 7 : 6) k_forward(DevGeom g, uint32_t parts, const float4 *__restrict__ rec,
+__global__ void __launch_bounds__(FBS, GM == GM_CONE ? 6 : 7) k_forward(DevGeom g, uint32_t parts, const float4 *__restrict__ rec,
                                                     const float4 *__restrict__ crec,
                                                     const uint32_t *__restrict__ gids,
                                                     const uint2 *__restrict__ ranges,
