@@ -377,7 +377,7 @@ int for_ray_ranges(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, cu
     TRY(ensure(ctx, ctx->part, sizeof(float4) * 2 * (size_t)parts));
     TRY(ensure(ctx, ctx->scene, sizeof(float4) * 2));
     TRY(ensure(ctx, ctx->blk, sizeof(float4) * 2 * (size_t)T));
-    TRY(ensure(ctx, ctx->wblk, sizeof(float4) * 8 * (size_t)T));
+    TRY(ensure(ctx, ctx->wblk, sizeof(float4) * RAYS_WBLK_F4 * RAYS_WPB * (size_t)T));
     const size_t TL = (size_t)T * RAYS_WPB;   // one list per warp
     TRY(ensure(ctx, ctx->cnt, sizeof(uint32_t) * TL));
     TRY(ensure(ctx, ctx->off, sizeof(uint32_t) * TL));

@@ -200,9 +200,11 @@ int rays_blocks(int64_t n_rays);       // ray blocks (128 rays each)
 int rays_ball_parts(int64_t n);        // partial scene boxes of the ball pass
 // balls (n float4), partial boxes (2 x parts), scene box (2), block lines
 // (2 x blocks) and per-block Gaussian counts
-// wblk: the same bound per 32-ray warp (4 per block, 2 float4 each)
+// wblk: per 32-ray warp (4 per block) the same bound and a slab, RAYS_WBLK_F4
+// float4 each
 // clusters: scratch of rays_cluster_bytes(n) bytes (the bounding balls in
 // Morton order, their ids, the cluster balls and the sort's buffers)
+constexpr int RAYS_WBLK_F4 = 3;
 size_t rays_cluster_bytes(int64_t n);
 cudaError_t launch_rays_bin(const float4 *ro, const float4 *rd, int64_t n_rays, const float4 *rec,
                             int64_t n, float4 *ball, float4 *part, float4 *scene, float4 *blk,
