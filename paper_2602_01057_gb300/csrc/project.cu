@@ -595,7 +595,7 @@ next_part:
 }
 
 template <int GM, bool STATS, int KER>
-__global__ void __launch_bounds__(FBS, GM == GM_CONE ? 6 : 7) k_forward(DevGeom g, uint32_t parts, const float4 *__restrict__ rec,
+__global__ void __launch_bounds__(FBS, GM == GM_PARALLEL ? 7 : 6) k_forward(DevGeom g, uint32_t parts, const float4 *__restrict__ rec,
                                                     const float4 *__restrict__ crec,
                                                     const uint32_t *__restrict__ gids,
                                                     const uint2 *__restrict__ ranges,
