@@ -86,23 +86,27 @@ __global__ void k_scan_top(unsigned long long *part, int64_t nb, unsigned long l
     if (threadIdx.x == 0) *total = carry_sh;
 }
 
+__device__ __forceinline__ int scan_at(int i) { return i + i / SCAN_IPT; }
+
 __global__ void k_scan_down(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, int64_t n,
                             const unsigned long long *__restrict__ part)
 {
-    __shared__ uint32_t sm[SCAN_TILE];
+    // a word of padding every SCAN_IPT: a thread's items are then 17 words from
+    // its neighbour's, on another bank
+    __shared__ uint32_t sm[SCAN_TILE + SCAN_BS];
     __shared__ uint32_t wsum[SCAN_BS / 32];
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     int t = threadIdx.x, lane = t & 31, w = t >> 5;
 #pragma unroll
     for (int i = 0; i < SCAN_IPT; i++) {
         int64_t x = base + (int64_t)i * SCAN_BS + t;
-        sm[i * SCAN_BS + t] = x < n ? in[x] : 0u;
+        sm[scan_at(i * SCAN_BS + t)] = x < n ? in[x] : 0u;
     }
     __syncthreads();
     uint32_t loc[SCAN_IPT];
     uint32_t s = 0;
 #pragma unroll
-    for (int j = 0; j < SCAN_IPT; j++) { loc[j] = sm[t * SCAN_IPT + j]; s += loc[j]; }
+    for (int j = 0; j < SCAN_IPT; j++) { loc[j] = sm[scan_at(t * SCAN_IPT + j)]; s += loc[j]; }
     uint32_t inc = s;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -124,12 +128,12 @@ __global__ void k_scan_down(const uint32_t *__restrict__ in, uint32_t *__restric
     __syncthreads();
     uint32_t run = (uint32_t)part[blockIdx.x] + wsum[w] + inc - s;
 #pragma unroll
-    for (int j = 0; j < SCAN_IPT; j++) { sm[t * SCAN_IPT + j] = run; run += loc[j]; }
+    for (int j = 0; j < SCAN_IPT; j++) { sm[scan_at(t * SCAN_IPT + j)] = run; run += loc[j]; }
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < SCAN_IPT; i++) {
         int64_t x = base + (int64_t)i * SCAN_BS + t;
-        if (x < n) out[x] = sm[i * SCAN_BS + t];
+        if (x < n) out[x] = sm[scan_at(i * SCAN_BS + t)];
     }
 }
 
@@ -139,7 +143,8 @@ __global__ void k_scan_down(const uint32_t *__restrict__ in, uint32_t *__restric
 // sorting by it orders each tile's list by footprint position (Gaussians of
 // the same position keep ascending ids, the sort being stable).
 // One thread per (view of the chunk, Gaussian) item; a CTA's 256 items own
-// one contiguous output range (the offsets are their exclusive scan).  With
+// one contiguous output range (the offsets are their exclusive scan, a CTA's
+// items are of one view).  With
 // STAGE the range is staged in shared memory and written out coalesced when
 // it fits -- worth it when items emit several keys each (large footprints);
 // with a key or two per item the direct writes are as compact and the
@@ -155,14 +160,15 @@ __device__ __forceinline__ void emit_item(const DevGeom &g, int vl, uint32_t k, 
 {
     const int i0 = r.x & 0xffff, i1 = r.x >> 16, j0 = r.y & 0xffff, j1 = r.y >> 16;
     const int tw = g.tile_w, th = g.tile_h;
-    const int tx0 = i0 / tw, tx1 = i1 / tw, ty0 = j0 / th, ty1 = j1 / th;
+    const TileDiv d(g);
+    const int tx0 = d.x(i0), tx1 = d.x(i1), ty0 = d.y(j0), ty1 = d.y(j1);
     const uint32_t tbase = lbits >= 0 ? (uint32_t)vl << lbits : (uint32_t)vl * (uint32_t)(g.tiles_x * g.tiles_y);
     for (int ty = ty0; ty <= ty1; ty++) {
         const int jl = max(j0 - ty * th, 0), jh = min(j1 - ty * th, th - 1);
-        const uint32_t rb = (uint32_t)(((jl + jh) * 8) / th);
+        const uint32_t rb = (uint32_t)d.y((jl + jh) * 8);
         for (int tx = tx0; tx <= tx1; tx++) {
             const int il = max(i0 - tx * tw, 0), ih = min(i1 - tx * tw, tw - 1);
-            const uint32_t cb = (uint32_t)(((il + ih) * 8) / tw);
+            const uint32_t cb = (uint32_t)d.x((il + ih) * 8);
             kd[o] = ((tbase + (uint32_t)ty * (uint32_t)g.tiles_x + (uint32_t)tx) << 8) | (rb << 4) | cb;
             vd[o] = k;
             o++;
@@ -179,16 +185,17 @@ __global__ void __launch_bounds__(EMIT_BS) k_emit(DevGeom g, int nv, int64_t n,
                                                   uint32_t cap, uint32_t *overflow, int lbits)
 {
     __shared__ uint32_t sk[STAGE ? EMIT_STAGE : 1], sv[STAGE ? EMIT_STAGE : 1];
-    const int64_t tot = (int64_t)nv * n;
-    const int64_t first = (int64_t)blockIdx.x * EMIT_BS;
-    const int64_t last = min(first + EMIT_BS, tot) - 1;
+    for (int vl = blockIdx.y; vl < nv; vl += gridDim.y) {
+    const int64_t end = (int64_t)(vl + 1) * n;
+    const int64_t first = (int64_t)vl * n + (int64_t)blockIdx.x * EMIT_BS;
+    const int64_t last = min(first + EMIT_BS, end) - 1;
     const int64_t idx = first + threadIdx.x;
     const uint64_t rs = off[first], re = (uint64_t)off[last] + cnt[last];
     // staged only when the whole range fits the buffer (an item past the
     // capacity writes nothing, as in the direct path)
     const bool staged = STAGE && re - rs <= (uint64_t)EMIT_STAGE && re <= (uint64_t)cap;
     uint32_t c = 0;
-    if (idx < tot) {
+    if (idx < end) {
         c = cnt[idx];
         if (c != 0) {
             const uint32_t o = off[idx];
@@ -198,19 +205,20 @@ __global__ void __launch_bounds__(EMIT_BS) k_emit(DevGeom g, int nv, int64_t n,
                 // last, maps to no tile), so that no slot is left stale
                 for (uint32_t e = o; e < cap && e < o + c; e++) keys[e] = 0xffffffffu;
             } else {
-                const int vl = (int)(idx / n);
                 const uint32_t k = (uint32_t)(idx - (int64_t)vl * n);
                 if (staged) emit_item(g, vl, k, rect[idx], o - (uint32_t)rs, sk, sv, lbits);
                 else emit_item(g, vl, k, rect[idx], o, keys, vals, lbits);
             }
         }
     }
-    if (!staged) return;     // uniform over the CTA
+    if (!staged) continue;     // uniform over the CTA
     __syncthreads();
     const uint32_t m = (uint32_t)(re - rs);
     for (uint32_t e = threadIdx.x; e < m; e += EMIT_BS) {
         keys[rs + e] = sk[e];
         vals[rs + e] = sv[e];
+    }
+    __syncthreads();   // the staged range is out before another view's comes in
     }
 }
 
@@ -561,7 +569,7 @@ cudaError_t launch_emit(const DevGeom &g, int nv, int64_t n, const uint32_t *cnt
 {
     int64_t tot = (int64_t)nv * n;
     if (tot <= 0) return cudaSuccess;
-    const unsigned grid = (unsigned)((tot + EMIT_BS - 1) / EMIT_BS);
+    const dim3 grid((unsigned)((n + EMIT_BS - 1) / EMIT_BS), (unsigned)(nv < 65535 ? nv : 65535));
     if ((double)cap >= 3.0 * (double)tot)
         k_emit<true><<<grid, EMIT_BS, 0, s>>>(g, nv, n, cnt, off, rect, keys, vals, cap, overflow, lbits);
     else

@@ -178,40 +178,103 @@ __device__ __forceinline__ int upper_idx_g(const float *tab, int n, float x, flo
     return i - 1;
 }
 
-// one thread per (view of the chunk, Gaussian), view-major
+// A Gaussian in a view's frame: the quantities that its detector box follows from
+struct CullFrame {
+    float mu_u, mu_v, mu_w, suu, svv, sww, suw, svw;
+};
+
+// By the specification's general forms.  Every frame here is a rotation about
+// z -- e_v = (0, 0, 1), e_u and e_w in the transaxial plane -- and for finite
+// values the products with its zeros change no sum, so the short forms below
+// give the same numbers; where one of them is not finite (an overflowed
+// covariance times a zero is a NaN) the general ones decide.
+template <bool CONE, bool P3>
+__device__ __forceinline__ CullFrame cull_frame(const float *m, const float *Sg, const float *F)
+{
+    const float eu[3] = { __ldg(F + 0), __ldg(F + 1), __ldg(F + 2) };
+    const float ew[3] = { __ldg(F + 6), __ldg(F + 7), __ldg(F + 8) };
+    CullFrame c;
+    c.mu_u = A(M(m[0], eu[0]), M(m[1], eu[1]));
+    c.mu_v = m[2];
+    c.suu = A(M(eu[0], A(M(Sg[0], eu[0]), M(Sg[1], eu[1]))), M(eu[1], A(M(Sg[1], eu[0]), M(Sg[3], eu[1]))));
+    c.svv = Sg[5];
+    c.mu_w = c.sww = c.suw = c.svw = 0.0f;
+    if (CONE || P3) {
+        const float t0 = A(M(Sg[0], ew[0]), M(Sg[1], ew[1])), t1 = A(M(Sg[1], ew[0]), M(Sg[3], ew[1]));
+        c.mu_w = A(M(m[0], ew[0]), M(m[1], ew[1]));
+        c.sww = A(M(ew[0], t0), M(ew[1], t1));
+        c.suw = A(M(eu[0], t0), M(eu[1], t1));
+        c.svw = A(M(Sg[2], ew[0]), M(Sg[4], ew[1]));
+    }
+    const float all = c.mu_u + c.mu_v + c.mu_w + c.suu + c.svv + c.sww + c.suw + c.svw + (Sg[2] + Sg[4]);
+    if (!isfinite(all)) {
+        const float ev[3] = { __ldg(F + 3), __ldg(F + 4), __ldg(F + 5) };
+        c.mu_u = dot_spec(m, eu);
+        c.mu_v = dot_spec(m, ev);
+        c.mu_w = dot_spec(m, ew);
+        c.suu = form_spec(Sg, eu, eu);
+        c.svv = form_spec(Sg, ev, ev);
+        c.sww = form_spec(Sg, ew, ew);
+        c.suw = form_spec(Sg, eu, ew);
+        c.svw = form_spec(Sg, ev, ew);
+    }
+    return c;
+}
+
+// number of tiles and pixel box of columns i0..i1, rows j0..j1
+__device__ __forceinline__ void cull_write(const DevGeom &g, int i0, int i1, int j0, int j1, uint32_t *cnt, uint2 *rect)
+{
+    if (i0 > i1 || j0 > j1) {
+        *cnt = 0;
+        *rect = make_uint2(1u, 1u);   // empty: columns and rows 1..0
+        return;
+    }
+    const TileDiv d(g);
+    const unsigned tx0 = d.x(i0), tx1 = d.x(i1), ty0 = d.y(j0), ty1 = d.y(j1);
+    *cnt = (tx1 - tx0 + 1) * (ty1 - ty0 + 1);
+    // pixel box (the tiles follow from it)
+    *rect = make_uint2((unsigned)i0 | ((unsigned)i1 << 16), (unsigned)j0 | ((unsigned)j1 << 16));
+}
+
+// one thread per (view of the chunk, Gaussian), view-major; 3-D PET: one per
+// (angle, Gaussian), which takes the chunk's ring differences of that angle in
+// turn (they share the frame and the columns)
+template <int GM>
 __global__ void k_cull(DevGeom g, int nv, const float4 *__restrict__ crec, int64_t n,
                        uint32_t *__restrict__ cnt, uint2 *__restrict__ rect)
 {
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)nv * n) return;
-    int vl = (int)(idx / n);
-    int64_t k = idx - (int64_t)vl * n;
-    const float *F = g.frames + 9 * (size_t)(g.v0 + vl);
-    float eu[3] = { __ldg(F + 0), __ldg(F + 1), __ldg(F + 2) };
-    float ev[3] = { __ldg(F + 3), __ldg(F + 4), __ldg(F + 5) };
-    float ew[3] = { __ldg(F + 6), __ldg(F + 7), __ldg(F + 8) };
-    float4 c0 = crec[CREC_F4 * k], c1 = crec[CREC_F4 * k + 1], c2 = crec[CREC_F4 * k + 2];
-    float m[3] = { c0.x, c0.y, c0.z };
-    float Sg[6] = { c1.x, c1.y, c1.z, c1.w, c2.x, c2.y };
+    constexpr bool CONE = GM == GM_CONE, P3 = GM == GM_PET3D;
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const float4 c0 = crec[CREC_F4 * k], c1 = crec[CREC_F4 * k + 1], c2 = crec[CREC_F4 * k + 2];
+    const float m[3] = { c0.x, c0.y, c0.z };
+    const float Sg[6] = { c1.x, c1.y, c1.z, c1.w, c2.x, c2.y };
     const float K2 = CULL_K2;
-    float mu_u = dot_spec(m, eu), mu_v = dot_spec(m, ev);
-    float ulo = -INFINITY, uhi = INFINITY, vlo = -INFINITY, vhi = INFINITY;
-    if (g.kind == 1) {
-        float aw = A(dot_spec(m, ew), g.dso);
-        float suu = form_spec(Sg, eu, eu), svv = form_spec(Sg, ev, ev), sww = form_spec(Sg, ew, ew);
-        float suw = form_spec(Sg, eu, ew), svw = form_spec(Sg, ev, ew);
-        float lo, hi;
-        if (cone_spec(K2, g.dsd, mu_u, aw, suu, suw, sww, lo, hi)) { ulo = lo; uhi = hi; }
-        if (cone_spec(K2, g.dsd, mu_v, aw, svv, svw, sww, lo, hi)) { vlo = lo; vhi = hi; }
-    } else {
-        float hu = __fsqrt_rn(M(K2, form_spec(Sg, eu, eu)));
-        float hv = __fsqrt_rn(M(K2, form_spec(Sg, ev, ev)));
-        ulo = S(mu_u, hu); uhi = A(mu_u, hu); vlo = S(mu_v, hv); vhi = A(mu_v, hv);
-    }
-    int i0 = lower_idx_g(g.utab, g.n_cols, ulo, g.u0, g.uinv);
-    int i1 = upper_idx_g(g.utab, g.n_cols, uhi, g.u0, g.uinv);
-    int j0, j1;
-    if (g.kind == GM_PET3D) {
+    const int nf = P3 ? min(nv, g.n_ang) : nv;
+    for (int vf = blockIdx.y; vf < nf; vf += gridDim.y) {
+        const CullFrame c = cull_frame<CONE, P3>(m, Sg, g.frames + 9 * (size_t)(g.v0 + vf));
+        float ulo = -INFINITY, uhi = INFINITY, vlo = -INFINITY, vhi = INFINITY;
+        if (CONE) {
+            const float aw = A(c.mu_w, g.dso);
+            float lo, hi;
+            if (cone_spec(K2, g.dsd, c.mu_u, aw, c.suu, c.suw, c.sww, lo, hi)) { ulo = lo; uhi = hi; }
+            if (cone_spec(K2, g.dsd, c.mu_v, aw, c.svv, c.svw, c.sww, lo, hi)) { vlo = lo; vhi = hi; }
+        } else {
+            const float hu = __fsqrt_rn(M(K2, c.suu));
+            ulo = S(c.mu_u, hu); uhi = A(c.mu_u, hu);
+            if (!P3) {
+                const float hv = __fsqrt_rn(M(K2, c.svv));
+                vlo = S(c.mu_v, hv); vhi = A(c.mu_v, hv);
+            }
+        }
+        const int i0 = lower_idx_g(g.utab, g.n_cols, ulo, g.u0, g.uinv);
+        const int i1 = upper_idx_g(g.utab, g.n_cols, uhi, g.u0, g.uinv);
+        if (!P3) {
+            const int j0 = lower_idx_g(g.vtab, g.n_rows, vlo, g.v0f, g.vinv);
+            const int j1 = upper_idx_g(g.vtab, g.n_rows, vhi, g.v0f, g.vinv);
+            cull_write(g, i0, i1, j0, j1, cnt + (int64_t)vf * n + k, rect + (int64_t)vf * n + k);
+            continue;
+        }
         // 3-D PET: the LOR of radial position s and mid-height z has
         // direction e_w + kappa e_v, kappa = dz / (2 sqrt(R^2 - s^2)), and
         // a . x = z along it for a = e_v - kappa e_w, so it can meet the
@@ -220,47 +283,40 @@ __global__ void k_cull(DevGeom g, int nv, const float4 *__restrict__ crec, int64
         // i0..i1 the union of these intervals is spanned by their values at
         // the two extreme slopes.  Rows are ring pairs (mid-heights
         // vtab + zoff); rows past the segment's last pair hold no LOR.
-        j0 = 0;
-        j1 = -1;
+        float h2a = 0.0f, h2b = 0.0f;
         if (i0 <= i1) {
-            const int delta = pet3d_delta(g, g.v0 + vl), ad = abs(delta);
-            const float dz = M((float)delta, g.ring_pitch), zoff = M(M(0.5f, (float)ad), g.ring_pitch);
             const float ua = __ldg(g.utab + i0), ub = __ldg(g.utab + i1);
             const float amin = (ua <= 0.0f && ub >= 0.0f) ? 0.0f : fminf(fabsf(ua), fabsf(ub));
             const float amax = fmaxf(fabsf(ua), fabsf(ub));
-            const float h2a = S(g.radius2, M(amin, amin)), h2b = S(g.radius2, M(amax, amax));
-            const int last = g.n_rows - 1 - ad;
-            if (!(h2b > 0.0f)) {
-                j1 = last;
-            } else {
-                const float mu_w = dot_spec(m, ew);
-                const float svv = form_spec(Sg, ev, ev), svw = form_spec(Sg, ev, ew), sww = form_spec(Sg, ew, ew);
-                float zlo = INFINITY, zhi = -INFINITY;
-#pragma unroll
-                for (int e = 0; e < 2; e++) {
-                    const float kap = __fdiv_rn(M(0.5f, dz), __fsqrt_rn(e ? h2b : h2a));
-                    const float zc = S(mu_v, M(kap, mu_w));
-                    const float t = A(S(svv, M(M(2.0f, kap), svw)), M(M(kap, kap), sww));
-                    const float half = __fsqrt_rn(fmaxf(M(K2, t), 0.0f));
-                    zlo = fminf(zlo, S(zc, half));
-                    zhi = fmaxf(zhi, A(zc, half));
-                }
-                j0 = lower_idx_g(g.vtab, g.n_rows, S(zlo, zoff), g.v0f, g.vinv);
-                j1 = min(upper_idx_g(g.vtab, g.n_rows, S(zhi, zoff), g.v0f, g.vinv), last);
-            }
+            h2a = S(g.radius2, M(amin, amin));
+            h2b = S(g.radius2, M(amax, amax));
         }
-    } else {
-        j0 = lower_idx_g(g.vtab, g.n_rows, vlo, g.v0f, g.vinv);
-        j1 = upper_idx_g(g.vtab, g.n_rows, vhi, g.v0f, g.vinv);
-    }
-    if (i0 > i1 || j0 > j1) {
-        cnt[idx] = 0;
-        rect[idx] = make_uint2(1u, 1u);   // empty: columns and rows 1..0
-    } else {
-        unsigned tx0 = i0 / g.tile_w, tx1 = i1 / g.tile_w, ty0 = j0 / g.tile_h, ty1 = j1 / g.tile_h;
-        cnt[idx] = (tx1 - tx0 + 1) * (ty1 - ty0 + 1);
-        // pixel box (the tiles follow from it)
-        rect[idx] = make_uint2((unsigned)i0 | ((unsigned)i1 << 16), (unsigned)j0 | ((unsigned)j1 << 16));
+        const float sa = __fsqrt_rn(h2a), sb = __fsqrt_rn(h2b);
+        for (int vl = vf; vl < nv; vl += g.n_ang) {
+            int j0 = 0, j1 = -1;
+            if (i0 <= i1) {
+                const int delta = pet3d_delta(g, g.v0 + vl), ad = abs(delta);
+                const float dz = M((float)delta, g.ring_pitch), zoff = M(M(0.5f, (float)ad), g.ring_pitch);
+                const int last = g.n_rows - 1 - ad;
+                if (!(h2b > 0.0f)) {
+                    j1 = last;
+                } else {
+                    float zlo = INFINITY, zhi = -INFINITY;
+#pragma unroll
+                    for (int e = 0; e < 2; e++) {
+                        const float kap = __fdiv_rn(M(0.5f, dz), e ? sb : sa);
+                        const float zc = S(c.mu_v, M(kap, c.mu_w));
+                        const float t = A(S(c.svv, M(M(2.0f, kap), c.svw)), M(M(kap, kap), c.sww));
+                        const float half = __fsqrt_rn(fmaxf(M(K2, t), 0.0f));
+                        zlo = fminf(zlo, S(zc, half));
+                        zhi = fmaxf(zhi, A(zc, half));
+                    }
+                    j0 = lower_idx_g(g.vtab, g.n_rows, S(zlo, zoff), g.v0f, g.vinv);
+                    j1 = min(upper_idx_g(g.vtab, g.n_rows, S(zhi, zoff), g.v0f, g.vinv), last);
+                }
+            }
+            cull_write(g, i0, i1, j0, j1, cnt + (int64_t)vl * n + k, rect + (int64_t)vl * n + k);
+        }
     }
 }
 
@@ -279,10 +335,12 @@ cudaError_t launch_records(const float *mu, const float *ls, const float *q, con
 cudaError_t launch_cull(const DevGeom &g, int nv, const float4 *crec, int64_t n, uint32_t *cnt,
                         uint2 *rect, cudaStream_t s)
 {
-    int64_t tot = (int64_t)nv * n;
-    if (tot <= 0) return cudaSuccess;
-    int bs = 256;
-    k_cull<<<(unsigned)((tot + bs - 1) / bs), bs, 0, s>>>(g, nv, crec, n, cnt, rect);
+    if (nv <= 0 || n <= 0) return cudaSuccess;
+    const int nf = g.kind == GM_PET3D && nv > g.n_ang ? g.n_ang : nv;
+    const dim3 grid((unsigned)((n + 255) / 256), (unsigned)(nf < 65535 ? nf : 65535));
+    if (g.kind == GM_CONE) k_cull<GM_CONE><<<grid, 256, 0, s>>>(g, nv, crec, n, cnt, rect);
+    else if (g.kind == GM_PET3D) k_cull<GM_PET3D><<<grid, 256, 0, s>>>(g, nv, crec, n, cnt, rect);
+    else k_cull<GM_PARALLEL><<<grid, 256, 0, s>>>(g, nv, crec, n, cnt, rect);
     count_launches(1);
     return cudaGetLastError();
 }

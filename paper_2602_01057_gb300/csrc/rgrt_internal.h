@@ -51,6 +51,17 @@ int64_t desc_rays(const rgrt_geom_desc *d);
 // pointers.
 void geom_tables(const rgrt_geom_desc *d, float *tab, DevGeom &dg);
 
+// Tile indices of pixels below 65,536 without divisions: tile widths are powers
+// of two, and ceil(2^32 / h) reproduces j / h for h <= 32.
+struct TileDiv {
+    int sx;
+    uint32_t my;
+    __host__ __device__ explicit TileDiv(const DevGeom &g)
+        : sx(3 + (g.tile_w >> 4)), my(0xffffffffu / (uint32_t)g.tile_h + 1u) {}
+    __host__ __device__ int x(int i) const { return i >> sx; }
+    __host__ __device__ int y(int j) const { return (int)(((uint64_t)(uint32_t)j * my) >> 32); }
+};
+
 // Per-Gaussian records built once per parameter version.
 //   rec  : 5 float4 = (mu, rho), (P00 P01 P02 P11), (P12 P22 S00 S01),
 //          (S02 S11 S12 S22), (sigma_max, 0, 0, 0);  P = Sigma^-1, S = Sigma/det Sigma
