@@ -21,9 +21,9 @@
 // lanes that wait for a longer chord of the same round).  Against one Gaussian
 // per thread and tile (record gathers, box searches, a chain and 16 atomics
 // for each of the 1.9 tiles of a PET footprint), measured on a GB300: PET ring
-// of 288 x 329 x 63, 200,000 Gaussians 9.6 -> 6.9 ms; 8 raw angles, 100,000
-// 0.73 -> 0.15 ms; 24 angles x 13 time-of-flight bins 4.96 -> 3.7 ms; parallel
-// beam, 1,000 Gaussians on 16 x 64^2 0.34 -> 0.11 ms (that one had 256 CTAs of
+// of 288 x 329 x 63, 200,000 Gaussians 9.6 -> 6.85 ms; 8 raw angles, 100,000
+// 0.73 -> 0.14 ms; 24 angles x 13 time-of-flight bins 4.96 -> 2.87 ms; parallel
+// beam, 1,000 Gaussians on 16 x 64^2 0.34 -> 0.09 ms (that one had 256 CTAs of
 // serial pixels).  Sorting a warp's Gaussians by box area per view took the
 // ring from 8.0 to 6.9 ms: a round's lanes then have chords of like length.
 #include <type_traits>
@@ -166,28 +166,45 @@ __device__ __forceinline__ void rows_tof(const DevGeom &g, const float4 &c0, con
     const int plane = bd.h * bd.st;
 #pragma unroll
     for (int q = 0; q < 11; q++) m[q] = 0.0f;
-    const f2 NS = pk(ns, ns);
-    for (; j <= je; j += dr) {
-        const float dv = sv[j] - v0;
-        const float dv2 = dv * dv, a1 = c0.w * dv, a0 = c1.x * dv2;
-        int ia = ilo, ie = ihi;
-        if (g.uinv != 0.0f && c0.z < 0.0f) chord(c0.z, a1, a0 - chord_cut<0>(), xc, g.uinv, ia, ie);
-        for (int i = ia & ~1; i <= ie; i += 2) {
+    const f2 NS = pk(ns, ns), TH = pk(g.tof_h, g.tof_h), MINUS1 = pk(-1.0f, -1.0f);
+    // one flat loop over the lane's (row, column pair) items: a pair costs a loop
+    // over the bins, so a lane goes on to its next row rather than waiting for
+    // the longest chord of each, and 5 CTAs per SM, for the spills that 6 cost
+    // (24 angles x 13 bins: 3.27 -> 2.87 ms)
+    int i = 1, ie = 0;
+    float dv = 0.0f, a1 = 0.0f, a0 = 0.0f;
+    j -= dr;
+    while (true) {
+        if (i > ie) {
+            j += dr;
+            if (j > je) break;
+            dv = sv[j] - v0;
+            const float dv2 = dv * dv;
+            a1 = c0.w * dv;
+            a0 = c1.x * dv2;
+            i = ilo;
+            ie = ihi;
+            if (g.uinv != 0.0f && c0.z < 0.0f) chord(c0.z, a1, a0 - chord_cut<0>(), xc, g.uinv, i, ie);
+            i &= ~1;
+        }
+        if (i <= ie) {
             const float2 uu = *reinterpret_cast<const float2 *>(su + i);
+            const int at = i;
+            i += 2;
             const float du0 = uu.x - u0, du1 = uu.y - u0;
             const float q0 = fmaf(fmaf(c0.z, du0, a1), du0, a0), q1 = fmaf(fmaf(c0.z, du1, a1), du1, a0);
             const float e0 = profile<0>(q0), e1 = profile<0>(q1);
-            if (e0 == 0.0f && e1 == 0.0f) continue;
             const float tb = t4.x + t4.z * dv - g.tof_t0;
             const f2 ts = pk(tb + t4.y * du0, tb + t4.y * du1);
-            f2 Ge = 0, D1 = 0, D2 = 0;
-            const float *gp = sg + j * bd.st + i;
-            for (int b = 0; b < g.n_tof; b++) {
-                const float t = -(float)b * g.tof_h;
-                const f2 x = add2(ts, pk(t, t)), x2 = mul2(x, x), y = mul2(NS, x2);
+            f2 Ge = 0, D1 = 0, D2 = 0, nb = 0;      // nb: minus the bin
+            const float *gp = sg + j * bd.st + at;
+#pragma unroll 2
+            for (int b = 0; b < g.n_tof; b++, gp += plane) {
+                const f2 x = fma2(nb, TH, ts), x2 = mul2(x, x);
+                nb = add2(nb, MINUS1);
                 float y0, y1;
-                up(y, y0, y1);
-                const float2 gg = *reinterpret_cast<const float2 *>(gp + b * plane);
+                up(mul2(NS, x2), y0, y1);
+                const float2 gg = *reinterpret_cast<const float2 *>(gp);
                 const f2 gw = mul2(pk(gg.x, gg.y), pk(ex2_approx(y0), ex2_approx(y1)));
                 Ge = add2(Ge, gw);
                 D1 = fma2(gw, x, D1);
@@ -201,7 +218,7 @@ __device__ __forceinline__ void rows_tof(const DevGeom &g, const float4 &c0, con
                 up(D2, d20, d21);
                 const float du = k ? du1 : du0, e = k ? e1 : e0, q = k ? q1 : q0;
                 const float ge = (k ? G1 : G0) * nrm;
-                const float v1 = e * ((k ? d11 : d10) * (-nrm * is2));              // val sum g_k dW_k/dt*
+                const float v1 = e * ((k ? d11 : d10) * (-nrm * is2));     // val sum g_k dW_k/dt*
                 const float v2 = e * (0.5f * is2 * (nrm * is2 * (k ? d21 : d20) - ge));   // val sum g_k dW_k/ds^2
                 const float h = ge * e, hd = h * du;
                 m[0] += h;
@@ -307,7 +324,7 @@ template <bool TOF> struct Shared {
 };
 
 template <int KER, bool TOF, int LG>
-__global__ void __launch_bounds__(BS, 6) k_adjoint(DevGeom g, int nv, int64_t n, int gw, int vper,
+__global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, int64_t n, int gw, int vper,
                                                    const uint32_t *__restrict__ order,
                                                    const float4 *__restrict__ rec,
                                                    const float4 *__restrict__ crec,
@@ -406,15 +423,24 @@ __global__ void __launch_bounds__(BS, 6) k_adjoint(DevGeom g, int nv, int64_t n,
                 for (int j = threadIdx.x; j < bd.h; j += BS) sh.sv[j] = __ldg(g.vtab + bd.rb + j);
                 const int sh_ = bd.st <= 8 ? 3 : bd.st <= 16 ? 4 : 5;
                 const int lc = lane & ((1 << sh_) - 1), lr = (w << (5 - sh_)) + (lane >> sh_), rstep = NW << (5 - sh_);
+                // (time of flight: plane by plane), four loads in flight (PET ring
+                // 7.1 -> 6.85 ms against one)
+                const int nr = TOF ? nb * bd.h : bd.h;
+                const float ih = 1.0f / (float)bd.h;
                 for (int c = lc; c < bd.st; c += 1 << sh_) {
-                    const float *src = dLdI + (long long)view * g.stride_view + (bd.cb + c);
-                    for (int j = lr; j < bd.h; j += rstep) {
-#pragma unroll 1
-                        for (int b = 0; b < nb; b++) {
-                            const float x = c < bd.w ? __ldg(src + (long long)(bd.rb + j) * g.stride_row +
-                                                             (TOF ? b * g.stride_tof : 0)) : 0.0f;
-                            sh.sg[(b * bd.h + j) * bd.st + c] = x;
+                    const float *src = dLdI + (long long)view * g.stride_view + (long long)bd.rb * g.stride_row + (bd.cb + c);
+                    for (int j0 = lr; j0 < nr; j0 += 4 * rstep) {
+                        float x[4];
+#pragma unroll
+                        for (int u = 0; u < 4; u++) {
+                            const int jj = j0 + u * rstep, b = TOF ? (int)(((float)jj + 0.5f) * ih) : 0;
+                            x[u] = 0.0f;
+                            if (jj < nr && c < bd.w)
+                                x[u] = __ldg(src + (long long)(jj - b * bd.h) * g.stride_row + (TOF ? b * g.stride_tof : 0));
                         }
+#pragma unroll
+                        for (int u = 0; u < 4; u++)
+                            if (j0 + u * rstep < nr) sh.sg[(j0 + u * rstep) * bd.st + c] = x[u];
                     }
                 }
                 __syncthreads();
@@ -565,8 +591,11 @@ __device__ __forceinline__ void box_add(const float *m, uint32_t *b)
     }
 }
 
-__global__ void k_order_box(const float4 *__restrict__ crec, int64_t n, uint32_t *box)
+__global__ void __launch_bounds__(256) k_order_box(const float4 *__restrict__ crec, int64_t n, uint32_t *box)
 {
+    __shared__ uint32_t sb[6];
+    if (threadIdx.x < 6) sb[threadIdx.x] = 0;
+    __syncthreads();
     uint32_t b[6] = { 0, 0, 0, 0, 0, 0 };
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const float4 c = __ldg(crec + CREC_F4 * k);
@@ -576,8 +605,10 @@ __global__ void k_order_box(const float4 *__restrict__ crec, int64_t n, uint32_t
 #pragma unroll
     for (int a = 0; a < 6; a++) {
         b[a] = __reduce_max_sync(0xffffffffu, b[a]);
-        if ((threadIdx.x & 31) == 0) atomicMax(box + a, b[a]);
+        if ((threadIdx.x & 31) == 0) atomicMax(&sb[a], b[a]);
     }
+    __syncthreads();
+    if (threadIdx.x < 6) atomicMax(box + threadIdx.x, sb[threadIdx.x]);
 }
 
 // code << 32 | rank within the cell, per Gaussian
@@ -590,12 +621,19 @@ __global__ void k_order_cells(const float4 *__restrict__ crec, int64_t n, int bi
     where[k] = make_uint2(c, atomicAdd(cells + c, 1u));
 }
 
-// exclusive scan of cnt[0..m) in place by one CTA of SMALL_BS threads (m a multiple of SMALL_BS)
-__device__ __forceinline__ void cta_scan(uint32_t *cnt, int m, uint32_t *wsum)
+// exclusive scan of cnt[0..4 V SMALL_BS) in place by one CTA of SMALL_BS
+// threads, V 16-byte loads each
+template <int V>
+__device__ __forceinline__ void cta_scan(uint32_t *cnt, uint32_t *wsum)
 {
-    const int per = m / SMALL_BS, base = threadIdx.x * per, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint4 *p = reinterpret_cast<uint4 *>(cnt) + V * threadIdx.x;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint4 q[V];
     uint32_t s = 0;
-    for (int k = 0; k < per; k++) s += cnt[base + k];
+#pragma unroll
+    for (int j = 0; j < V; j++) q[j] = p[j];
+#pragma unroll
+    for (int j = 0; j < V; j++) s += q[j].x + q[j].y + q[j].z + q[j].w;
     uint32_t inc = s;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -616,17 +654,22 @@ __device__ __forceinline__ void cta_scan(uint32_t *cnt, int m, uint32_t *wsum)
     }
     __syncthreads();
     uint32_t run = wsum[w] + inc - s;
-    for (int k = 0; k < per; k++) {
-        const uint32_t c = cnt[base + k];
-        cnt[base + k] = run;
-        run += c;
+#pragma unroll
+    for (int j = 0; j < V; j++) {
+        uint4 o;
+        o.x = run;
+        o.y = o.x + q[j].x;
+        o.z = o.y + q[j].y;
+        o.w = o.z + q[j].z;
+        run = o.w + q[j].w;
+        p[j] = o;
     }
 }
 
 __global__ void __launch_bounds__(SMALL_BS) k_order_scan(uint32_t *cells)
 {
     __shared__ uint32_t wsum[32];
-    cta_scan(cells, CELLS, wsum);
+    cta_scan<CELLS / (4 * SMALL_BS)>(cells, wsum);
 }
 
 __global__ void k_order_scatter(int64_t n, const uint32_t *__restrict__ cells, const uint2 *__restrict__ where,
@@ -642,7 +685,8 @@ __global__ void k_order_scatter(int64_t n, const uint32_t *__restrict__ cells, c
 __global__ void __launch_bounds__(SMALL_BS) k_order_small(const float4 *__restrict__ crec, int n, int bits,
                                                           uint32_t *order)
 {
-    __shared__ uint32_t cells[1 << SMALL_BITS], wsum[32], box[6];
+    __shared__ __align__(16) uint32_t cells[1 << SMALL_BITS];
+    __shared__ uint32_t wsum[32], box[6];
     for (int k = threadIdx.x; k < (1 << SMALL_BITS); k += SMALL_BS) cells[k] = 0;
     if (threadIdx.x < 6) box[threadIdx.x] = 0;
     __syncthreads();
@@ -668,7 +712,7 @@ __global__ void __launch_bounds__(SMALL_BS) k_order_small(const float4 *__restri
         rank[q] = atomicAdd(&cells[code[q]], 1u);
     }
     __syncthreads();
-    cta_scan(cells, 1 << SMALL_BITS, wsum);
+    cta_scan<(1 << SMALL_BITS) / (4 * SMALL_BS)>(cells, wsum);
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < PER; q++) {
@@ -695,12 +739,13 @@ cudaError_t launch_order(const float4 *crec, int64_t n, void *tmp, uint32_t *ord
         count_launches(1);
         return cudaGetLastError();
     }
-    uint2 *where = (uint2 *)tmp;
-    uint32_t *cells = (uint32_t *)(where + n), *box = cells + CELLS;
+    // the counters first: they are read as 16-byte vectors
+    uint32_t *cells = (uint32_t *)tmp, *box = cells + CELLS;
+    uint2 *where = (uint2 *)(box + 8);
     cudaError_t e = cudaMemsetAsync(cells, 0, sizeof(uint32_t) * (CELLS + 6), s);
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)((n + 255) / 256);
-    k_order_box<<<nb < 304u ? nb : 304u, 256, 0, s>>>(crec, n, box);
+    k_order_box<<<nb < 152u ? nb : 152u, 256, 0, s>>>(crec, n, box);
     k_order_cells<<<nb, 256, 0, s>>>(crec, n, bits, box, cells, where);
     k_order_scan<<<1, SMALL_BS, 0, s>>>(cells);
     k_order_scatter<<<nb, 256, 0, s>>>(n, cells, where, order);
@@ -714,9 +759,11 @@ template <int KER, bool TOF>
 void adjoint_lg(int lg, const DevGeom &g, int nv, int64_t n, const uint32_t *order, const float4 *rec,
                 const float4 *crec, const uint2 *rect, const float *dLdI, float4 *grad, cudaStream_t s)
 {
-    // Gaussians per warp: fewer where 32 would leave the GPU short of CTAs
+    // Gaussians per warp: fewer where 32 would leave the GPU short of CTAs (10
+    // per SM; 1,000 Gaussians on 16 x 64^2 pixels: 0.117 ms at 8 and 5 CTAs per
+    // SM, 0.088 at 2)
     int gw = 32;
-    while (gw > 8 && gw > 32 >> lg && (n / (gw * NW)) * nv < 152 * 5) gw >>= 1;
+    while (gw > 2 && (n / (gw * NW)) * nv < 152 * 10) gw >>= 1;
     const int64_t bx = (n + NW * gw - 1) / (NW * gw);
     int64_t chunks = (152 * 5 * 12 + bx - 1) / bx;
     if (chunks > nv) chunks = nv;
