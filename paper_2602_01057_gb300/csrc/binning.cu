@@ -137,6 +137,73 @@ __global__ void k_scan_down(const uint32_t *__restrict__ in, uint32_t *__restric
     }
 }
 
+// The whole scan by one CTA: up to SCAN_SMALL values, where two of the three
+// launches above would only add their latency (16,000 counts 17 -> 8 us between events).  A
+// thread takes 4 `per` values as 16-byte loads, all issued before the first is
+// used.
+constexpr int SCAN_SMALL_BS = 1024, SCAN_SMALL_VEC = 8;
+constexpr int64_t SCAN_SMALL = 4 * SCAN_SMALL_VEC * SCAN_SMALL_BS;
+
+__global__ void __launch_bounds__(SCAN_SMALL_BS) k_scan_small(const uint32_t *__restrict__ in, uint32_t *__restrict__ out,
+                                                              int n, int per, unsigned long long *total)
+{
+    __shared__ unsigned long long wsum[32];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int base = 4 * per * t;
+    uint4 q[SCAN_SMALL_VEC];
+#pragma unroll
+    for (int j = 0; j < SCAN_SMALL_VEC; j++) {
+        const int k = base + 4 * j;
+        q[j] = make_uint4(0u, 0u, 0u, 0u);
+        if (j < per && k + 3 < n) q[j] = *reinterpret_cast<const uint4 *>(in + k);
+        else if (j < per && k < n) {
+            q[j].x = in[k];
+            if (k + 1 < n) q[j].y = in[k + 1];
+            if (k + 2 < n) q[j].z = in[k + 2];
+        }
+    }
+    unsigned long long s = 0;
+#pragma unroll
+    for (int j = 0; j < SCAN_SMALL_VEC; j++) s += (unsigned long long)q[j].x + q[j].y + q[j].z + q[j].w;
+    unsigned long long inc = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) wsum[w] = inc;
+    __syncthreads();
+    if (w == 0) {
+        const unsigned long long v = wsum[lane];
+        unsigned long long x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) *total = x;
+        wsum[lane] = x - v;
+    }
+    __syncthreads();
+    uint32_t run = (uint32_t)(wsum[w] + inc - s);
+#pragma unroll
+    for (int j = 0; j < SCAN_SMALL_VEC; j++) {
+        const int k = base + 4 * j;
+        uint4 o;
+        o.x = run;
+        o.y = o.x + q[j].x;
+        o.z = o.y + q[j].y;
+        o.w = o.z + q[j].z;
+        run = o.w + q[j].w;
+        if (j < per && k + 3 < n) *reinterpret_cast<uint4 *>(out + k) = o;
+        else if (j < per && k < n) {
+            out[k] = o.x;
+            if (k + 1 < n) out[k + 1] = o.y;
+            if (k + 2 < n) out[k + 2] = o.z;
+        }
+    }
+}
+
 // one thread per (view of the chunk, Gaussian): write its tiles' keys.
 // key = tile id << 8 | position code, the code being the 4-bit row and
 // column buckets of the centre of the Gaussian's pixel box within the tile:
@@ -246,7 +313,7 @@ __device__ __forceinline__ uint32_t sort_count(uint32_t n, const unsigned long l
 struct SortSegs {
     const uint32_t *tile_start = nullptr;
     const uint32_t *seg_start = nullptr;
-    const uint4 *span = nullptr;   // [nb]: every tile's (lo, hi, hb, hs), from k_sort_spans
+    const uint4 *span = nullptr;   // [nb]: every tile's (lo, hi, hb, hs), from k_sort_segments or k_sort_spans
     int ns = 0;
 };
 
@@ -449,8 +516,8 @@ __global__ void __launch_bounds__(SORT_BS) k_sort_scatter(const uint32_t *__rest
 // off[v stride] (the scan of the per-(view, Gaussian) counts) and takes
 // ceil(len / SORT_TILE) sort tiles; one block scans the tile counts.
 __global__ void k_sort_segments(const uint32_t *__restrict__ off, int64_t stride, int ns, uint32_t n,
-                                const unsigned long long *n_dev, uint32_t *__restrict__ tile_start,
-                                uint32_t *__restrict__ seg_start)
+                                const unsigned long long *n_dev, uint32_t *tile_start, uint32_t *seg_start,
+                                uint32_t span_nb, uint4 *__restrict__ span)
 {
     __shared__ uint32_t wsum[32];
     __shared__ uint32_t carry;
@@ -487,6 +554,16 @@ __global__ void k_sort_segments(const uint32_t *__restrict__ off, int64_t stride
             carry += tot;
         }
         __syncthreads();
+    }
+    // few sort tiles (2,048: two per thread): their spans here too, from the
+    // tables just written, which saves a launch
+    SortSegs sg;
+    sg.tile_start = tile_start;
+    sg.seg_start = seg_start;
+    sg.ns = ns;
+    for (uint32_t b = threadIdx.x; b < span_nb; b += blockDim.x) {
+        const TileSpan t = tile_span(b, span_nb, n, sg);
+        span[b] = make_uint4(t.lo, t.hi, (uint32_t)t.hb, (uint32_t)t.hs);
     }
 }
 
@@ -555,6 +632,12 @@ cudaError_t launch_scan(const uint32_t *in, uint32_t *out, int64_t n, unsigned l
                         unsigned long long *tmp, cudaStream_t s)
 {
     if (n <= 0) return cudaMemsetAsync(total, 0, sizeof(unsigned long long), s);
+    if (n <= SCAN_SMALL && (((uintptr_t)in | (uintptr_t)out) & 15u) == 0) {
+        const int per = (int)((n + 4 * SCAN_SMALL_BS - 1) / (4 * SCAN_SMALL_BS));
+        k_scan_small<<<1, SCAN_SMALL_BS, 0, s>>>(in, out, (int)n, per, total);
+        count_launches(1);
+        return cudaGetLastError();
+    }
     int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
     k_scan_reduce<<<(unsigned)nb, SCAN_BS, 0, s>>>(in, n, tmp);
     k_scan_top<<<1, 1024, 0, s>>>(tmp, nb, total);
@@ -664,10 +747,11 @@ cudaError_t launch_sort_views(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt
     sg.tile_start = tmp + L.tiles;
     sg.seg_start = tmp + L.segs;
     sg.ns = nv;
-    k_sort_segments<<<1, 1024, 0, s>>>(off, stride, nv, n, n_dev, tmp + L.tiles, tmp + L.segs);
     uint4 *span = reinterpret_cast<uint4 *>(tmp + L.span);
-    k_sort_spans<<<(L.nb + 255) / 256, 256, 0, s>>>(L.nb, n, n_dev, sg, span);
-    count_launches(2);
+    const bool few = L.nb <= 2048;
+    k_sort_segments<<<1, 1024, 0, s>>>(off, stride, nv, n, n_dev, tmp + L.tiles, tmp + L.segs, few ? L.nb : 0u, span);
+    if (!few) k_sort_spans<<<(L.nb + 255) / 256, 256, 0, s>>>(L.nb, n, n_dev, sg, span);
+    count_launches(few ? 1 : 2);
     sg.span = span;
     return sort_passes(keys, vals, keys_alt, vals_alt, n, shift, bits, tmp, L, sg, s, in_alt, n_dev);
 }

@@ -63,3 +63,23 @@ def test_forward_and_adjoint_tile_shapes(env, oracle, kind, tile, n):
         g = o.cpu().numpy().astype(np.float64)
         clip = np.clip(g, ref["lo"][key], ref["hi"][key])
         assert np.linalg.norm(g - clip) < GRAD_TOL * np.linalg.norm(ref[key]), key
+
+
+@pytest.mark.parametrize("n", [1, 6, 4095, 4097, 16383, 16384, 16385])
+def test_count_scan_sizes(env, n):
+    """The scan of the tile counts by one CTA and by three launches (2 views:
+    more than 32,768 counts): the projection is linear in the set, so the two
+    halves of a set of tiny Gaussians add up to it (binary32 sums of fewer than
+    100 terms a pixel: 1e-5 relative L2)."""
+    torch, rg, ctx = env
+    geom = rg.Geometry(ctx, synth.geom_parallel(2, 64, 64, 0.03, 0.03, -4.0, 4.0))
+    G = synth.gaussians_uniform(n, 52, half_box=0.9, log_sigma=math.log(0.01))
+    t = {k: torch.from_numpy(np.ascontiguousarray(G[k])).cuda() for k in ("mu", "ls", "q", "rho")}
+    t["rho"] = t["rho"].abs()
+
+    def forward(a, b):
+        gs = rg.Gaussians(ctx, *[t[k][a:b].contiguous() for k in ("mu", "ls", "q", "rho")])
+        return rg.project_forward(ctx, gs, geom, torch.empty(geom.n_rays, device="cuda")).double()
+    whole, cuts = forward(0, n), sorted({0, n // 3, n})
+    parts = sum(forward(a, b) for a, b in zip(cuts, cuts[1:]))
+    assert torch.linalg.norm(whole - parts) <= 1e-5 * torch.linalg.norm(whole)
