@@ -1200,13 +1200,10 @@ int loss_step(rgrt_ctx *ctx, rgrt_gauss *g, const rgrt_geom *geom, const float *
         }
         float bc1 = (float)(1.0 - pow((double)hp->beta1, (double)t));
         float bc2 = (float)(1.0 - pow((double)hp->beta2, (double)t));
-        float *ps[4] = { g->mu, g->ls, g->q, g->rho };
-        const int64_t off[4] = { 0, 3 * N, 6 * N, 10 * N }, len[4] = { 3 * N, 3 * N, 4 * N, N };
-        const float lr[4] = { hp->lr_mu, hp->lr_logscale, hp->lr_quat, hp->lr_rho };
+        const AdamArrays arr = { { g->mu, g->ls, g->q, g->rho },
+                                 { hp->lr_mu, hp->lr_logscale, hp->lr_quat, hp->lr_rho } };
         PROF("k_adam");
-        for (int k = 0; k < 4; k++)
-            CK(launch_adam(ps[k], gf + off[k], g->adam_m + off[k], g->adam_v + off[k], len[k], lr[k],
-                           hp->beta1, hp->beta2, hp->eps, bc1, bc2, nullptr, nullptr, s));
+        CK(launch_adam(arr, gf, g->adam_m, g->adam_v, N, hp->beta1, hp->beta2, hp->eps, bc1, bc2, nullptr, nullptr, s));
         g->version++;
     }
     if (loss_out) CK(cudaMemcpyAsync(loss_out, ctx->loss.p, sizeof(float), cudaMemcpyDefault, s));

@@ -361,12 +361,10 @@ int enqueue_step(rgrt_batch *b, const float *const *y, int loss, const rgrt_adam
         const int64_t N = x.N;
         BK(launch_param_chain(g->mu, g->ls, g->q, g->rho, N, x.grad, gf, gf + 3 * N, gf + 6 * N,
                               gf + 10 * N, s));
-        float *ps[4] = { g->mu, g->ls, g->q, g->rho };
-        const int64_t offs[4] = { 0, 3 * N, 6 * N, 10 * N }, len[4] = { 3 * N, 3 * N, 4 * N, N };
-        const float lr[4] = { hp->lr_mu, hp->lr_logscale, hp->lr_quat, hp->lr_rho };
-        for (int k = 0; k < 4; k++)
-            BK(launch_adam(ps[k], gf + offs[k], g->adam_m + offs[k], g->adam_v + offs[k], len[k], lr[k],
-                           hp->beta1, hp->beta2, hp->eps, 1.0f, 1.0f, b->d_bc, b->d_overflow, s));
+        const AdamArrays arr = { { g->mu, g->ls, g->q, g->rho },
+                                 { hp->lr_mu, hp->lr_logscale, hp->lr_quat, hp->lr_rho } };
+        BK(launch_adam(arr, gf, g->adam_m, g->adam_v, N, hp->beta1, hp->beta2, hp->eps, 1.0f, 1.0f, b->d_bc,
+                       b->d_overflow, s));
     }
     return RGRT_OK;
 }

@@ -194,10 +194,16 @@ cudaError_t launch_loss(int kind, const float *I, const float *y, int64_t n, flo
                         float eps, const float *mult, const float *add, float *dLdI, double *partial,
                         int nblk, float *loss_out, cudaStream_t s, double *acc = nullptr);
 int loss_blocks(int64_t n);
-// Adam; bc_dev (optional) supplies the bias corrections (1 - beta^t) from
-// device memory instead of bc1, bc2; skip (optional) leaves everything
-// unchanged when *skip != 0
-cudaError_t launch_adam(float *p, const float *g, float *m, float *v, int64_t n, float lr,
+// Adam on every parameter array of n Gaussians (mu, log-scale, quaternion, rho
+// and their learning rates; g, m, v hold 11 n values in that order); bc_dev
+// (optional) supplies the bias corrections (1 - beta^t) from device memory
+// instead of bc1, bc2; skip (optional) leaves everything unchanged when
+// *skip != 0
+struct AdamArrays {
+    float *p[4];
+    float lr[4];
+};
+cudaError_t launch_adam(const AdamArrays &p, const float *g, float *m, float *v, int64_t n,
                         float beta1, float beta2, float eps, float bc1, float bc2,
                         const float *bc_dev, const uint32_t *skip, cudaStream_t s);
 
