@@ -53,8 +53,8 @@ template <> struct Fac<1> {
     static constexpr float FQ = 1.5f / 7.0f, FP = -2.0f;
 };
 
-// the kernel's profile of a pair: e^{-m/2} inside the cut (Gaussian), sqrt(c)
-// inside the support (Epanechnikov, c = 1 + arg)
+// the kernel's profile of a pair: e^{-m/2} (Gaussian), sqrt(c) inside the
+// support (Epanechnikov, c = 1 + arg)
 template <int KER>
 __device__ __forceinline__ float profile(float arg)
 {
@@ -62,7 +62,15 @@ __device__ __forceinline__ float profile(float arg)
         const float c = 1.0f + arg;
         return c > 0.0f ? sqrt_approx(c) : 0.0f;
     }
-    return arg >= CUT_ARG ? ex2_approx(arg) : 0.0f;
+    return ex2_approx(arg);
+}
+
+// the Gaussian's cut acts on x (dL/dI or what is made of it), so that an
+// infinite or NaN dL/dI outside the cut adds nothing
+template <int KER>
+__device__ __forceinline__ float cut(float arg, float x)
+{
+    return KER == 1 || arg >= CUT_ARG ? x : 0.0f;
 }
 
 struct Box {
@@ -128,7 +136,7 @@ __device__ __forceinline__ void rows(const DevGeom &g, const float4 &c0, const f
             const f2 q = fma2(fma2(Muu, du, A1), du, A0);
             float qx, qy;
             up(q, qx, qy);
-            const f2 h = mul2(pk(gg.x, gg.y), pk(profile<KER>(qx), profile<KER>(qy)));
+            const f2 h = mul2(pk(cut<KER>(qx, gg.x), cut<KER>(qy, gg.y)), pk(profile<KER>(qx), profile<KER>(qy)));
             const f2 hd = mul2(h, du);
             h0 = add2(h0, h);
             h1 = add2(h1, hd);
@@ -217,9 +225,9 @@ __device__ __forceinline__ void rows_tof(const DevGeom &g, const float4 &c0, con
                 up(D1, d10, d11);
                 up(D2, d20, d21);
                 const float du = k ? du1 : du0, e = k ? e1 : e0, q = k ? q1 : q0;
-                const float ge = (k ? G1 : G0) * nrm;
-                const float v1 = e * ((k ? d11 : d10) * (-nrm * is2));     // val sum g_k dW_k/dt*
-                const float v2 = e * (0.5f * is2 * (nrm * is2 * (k ? d21 : d20) - ge));   // val sum g_k dW_k/ds^2
+                const float ge = cut<0>(q, k ? G1 : G0) * nrm;
+                const float v1 = e * (cut<0>(q, k ? d11 : d10) * (-nrm * is2));     // val sum g_k dW_k/dt*
+                const float v2 = e * (0.5f * is2 * (nrm * is2 * cut<0>(q, k ? d21 : d20) - ge));   // val sum g_k dW_k/ds^2
                 const float h = ge * e, hd = h * du;
                 m[0] += h;
                 m[1] += hd;

@@ -256,7 +256,7 @@ __device__ __forceinline__ void adjoint_tile(const DevGeom &g, uint32_t tile, ui
 #pragma unroll 1
                 for (int j = jlo; j <= jhi; j += 2) {
                     const f2 vt = add2(pk(svr[j], svr[j + 1]), VT0);
-                    const f2 gl = pk(gc[j * TW], gc[(j + 1) * TW]);
+                    float g0 = gc[j * TW], g1 = gc[(j + 1) * TW];
                     // du (muu du + muv2 v~) + S_uu v~^2
                     const f2 q = mul2(fma2(fma2(Cvv, vt, LQ), vt, KQ), IA);
                     float q0, q1, e0, e1;
@@ -266,10 +266,13 @@ __device__ __forceinline__ void adjoint_tile(const DevGeom &g, uint32_t tile, ui
                         e0 = x0 > 0.0f ? sqrt_approx(x0) : 0.0f;
                         e1 = x1 > 0.0f ? sqrt_approx(x1) : 0.0f;
                     } else {
-                        e0 = q0 >= CUT_ARG ? ex2_approx(q0) : 0.0f;
-                        e1 = q1 >= CUT_ARG ? ex2_approx(q1) : 0.0f;
+                        // the cut acts on g: an infinite or NaN g outside it adds nothing
+                        g0 = q0 >= CUT_ARG ? g0 : 0.0f;
+                        g1 = q1 >= CUT_ARG ? g1 : 0.0f;
+                        e0 = ex2_approx(q0);
+                        e1 = ex2_approx(q1);
                     }
-                    const f2 h = mul2(gl, pk(e0, e1));
+                    const f2 h = mul2(pk(g0, g1), pk(e0, e1));
                     const f2 hd = mul2(h, vt);
                     h0 = add2(h0, h);
                     hv = add2(hv, hd);

@@ -80,3 +80,42 @@ def test_parallel_adjoint_matches_oracle(env, oracle, name, kernel):
         clip = np.clip(got, ref["lo"][key], ref["hi"][key])
         e = np.linalg.norm(got - clip) / max(np.linalg.norm(ref[key]), 1e-30)
         assert e < GRAD_TOL, f"{key}: {e:.2e}"
+
+
+def _tof():
+    return synth.with_tof_bins(synth.geom_pet(2, 65, 5, 400.0, 288, 20.0), 5, 40.0, 30.0)
+
+
+# one Gaussian well inside the field of view: (half-axis, geometry)
+MASKED = {
+    "parallel": lambda: (0.12, _parallel(2, 48, 48, 0.03)),
+    "cone": lambda: (0.12, synth.geom_cone(2, 48, 48, 0.06, 0.06, 3.0, 6.0)),
+    "ring": lambda: (20.0, synth.geom_pet(2, 65, 21, 400.0, 288, 9.0)),
+    "ring_tof": lambda: (20.0, _tof()),
+    "pet3d": lambda: (20.0, synth.geom_pet3d(2, 65, 9, 400.0, 288, 9.0, 2)),
+}
+
+
+@pytest.mark.parametrize("bad", [math.nan, math.inf])
+@pytest.mark.parametrize("name", list(MASKED))
+def test_non_finite_weight_outside_the_cut_adds_nothing(env, name, bad):
+    """A NaN or infinite dL/dI where the Gaussian contributes nothing leaves its
+    gradient as a zero there does.  Tolerance: both sum the same terms, up to
+    the order of a few atomic additions in binary32."""
+    torch, rg, ctx = env
+    s, gd = MASKED[name]()
+    geom = rg.Geometry(ctx, gd)
+    f = dict(dtype=torch.float32, device="cuda")
+    gs = rg.Gaussians(ctx, torch.tensor([[0.4 * s, -0.3 * s, 0.2 * s]], **f),
+                      torch.log(torch.tensor([[s, 0.5 * s, 0.7 * s]], **f)),
+                      torch.tensor([[0.9, 0.1, -0.3, 0.2]], **f), torch.tensor([1.0], **f))
+    img = rg.project_forward(ctx, gs, geom, torch.empty(geom.n_rays, device="cuda"))
+    empty = img.reshape(-1) == 0.0
+    assert 0 < int(empty.sum()) < empty.numel()
+    w = torch.from_numpy(synth.random_weights(geom.n_rays, 6)).cuda().reshape(-1)
+    res = []
+    for fill in (0.0, bad):
+        outs = [torch.empty(sh, device="cuda") for sh in ((1, 3), (1, 3), (1, 4), (1,))]
+        rg.project_backward(ctx, gs, geom, torch.where(empty, torch.full_like(w, fill), w), *outs)
+        res.append(torch.cat([o.reshape(-1) for o in outs]).double().cpu())
+    assert torch.linalg.norm(res[1] - res[0]) <= 1e-5 * torch.linalg.norm(res[0])
