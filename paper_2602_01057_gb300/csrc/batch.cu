@@ -1,13 +1,14 @@
 // Batched form: one optimisation step (or one forward pass) over many
 // independent scans -- each with its own Gaussians and geometry -- as a single
-// stream of work.  The scans are binned one after another.  A scan large
-// enough to fill the GPU for 16 waves of tiles is projected, its loss taken
+// stream of work.  Small scans are binned on a few streams side by side.  A scan
+// large enough to fill the GPU for 16 waves of tiles is projected, its loss taken
 // and back-projected right after its binning, with launches of its own (its
 // lists and records are still in L2 for the adjoint).  The smaller scans
 // share ONE persistent launch that integrates every (scan, tile) work item,
 // taken from an atomic counter (uneven scans fill the GPU together instead of
-// leaving it under-filled one by one), then their losses and ONE persistent
-// adjoint launch.  The parameter chains and the Adam updates of every scan
+// leaving it under-filled one by one), then their losses and the adjoint: ONE
+// persistent launch (cone beam, from the tile lists), or one per scan (parallel
+// rays, from the boxes).  The parameter chains and the Adam updates of every scan
 // come last.  The whole step is captured once in a CUDA graph and replayed,
 // so a step costs one graph launch and one small read-back (losses and the
 // key-capacity overflow flag) instead of a host round trip per scan.
@@ -18,8 +19,8 @@
 // entries no longer fit, the emit kernel raises the overflow flag, every Adam
 // update of that step is skipped on the device, and the host re-plans,
 // re-captures and repeats the step.  Only the sorted Gaussian ids and tile ranges of a scan
-// are kept per scan; counts, keys and sort buffers are shared scratch sized
-// for the largest scan.
+// are kept per scan (parallel rays: the boxes as well); counts, keys and sort
+// buffers are scratch of a stream, sized for the largest of its scans.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -61,6 +62,7 @@ struct BatchScan {
     int bits = 0, nblk = 1;
     int lbits = -1;             // >= 0: keys sorted view by view (see launch_sort_views)
     bool large = false;         // projected by its own launches (not the persistent ones)
+    int lane = 0;               // the stream and scratch it is binned with
     uint32_t *vals = nullptr;   // sorted Gaussian ids [cap]
     uint2 *ranges = nullptr;    // [T]
     uint2 *rect = nullptr;      // pixel boxes [E] (a large scan: the shared scratch)
@@ -81,18 +83,37 @@ int ceil_log2_b(uint64_t x)
 
 }  // namespace
 
+// A stream of the captured step and the binning scratch of its scans.
+struct Lane {
+    cudaStream_t s = nullptr;
+    cudaEvent_t ev = nullptr;
+    uint32_t *cnt = nullptr, *off = nullptr, *keys = nullptr, *keys_alt = nullptr,
+             *vals_alt = nullptr, *sort_tmp = nullptr;
+    uint2 *rect = nullptr;
+    void *order_tmp = nullptr;
+    unsigned long long *stmp = nullptr, *total = nullptr;
+};
+
+// Small scans are binned on LANES streams of the captured graph: one scan's
+// launches leave most of the GPU idle and wait for one another (24 cone-beam
+// scans of 5,000 Gaussians, 40 views of 96^2: a step 10.2 ms on 1 lane, 9.4 on
+// 2, 9.1 on 4, 9.0 on 8).  LANE_BYTES bounds the scratch of the lanes after the
+// first; they also leave at least 15/16 of what the context's memory budget
+// still allows to others.
+constexpr int LANES = 4;
+constexpr size_t LANE_BYTES = (size_t)256 << 20;
+
 struct rgrt_batch {
     rgrt_ctx *ctx = nullptr;
     int n = 0;
     bool cone = false;
     int tile_w = 16, tile_h = 16;
     std::vector<BatchScan> sc;
-    // shared binning scratch
-    uint32_t *cnt = nullptr, *off = nullptr, *keys = nullptr, *keys_alt = nullptr,
-             *vals_alt = nullptr, *sort_tmp = nullptr;
-    uint2 *rect = nullptr;
-    void *order_tmp = nullptr;
-    unsigned long long *stmp = nullptr, *total = nullptr;
+    // lane 0: the batch's own stream, scratch for every scan; the others'
+    // scratch holds the small scans.  One lane if scans share a Gaussian set.
+    Lane lane[LANES];
+    int n_lanes = 1;
+    bool distinct = true;
     // batch tables
     ScanDesc *d_desc = nullptr;
     uint32_t *d_queue = nullptr, *d_overflow = nullptr;
@@ -132,10 +153,13 @@ void free_plan(rgrt_batch *b)
         s.vals = nullptr; s.ranges = nullptr; s.rect = nullptr; s.order = nullptr; s.I = s.dLdI = nullptr;
         s.grad = nullptr; s.gflat = nullptr; s.partial = nullptr;
     }
-    b->cnt = b->off = b->keys = b->keys_alt = b->vals_alt = b->sort_tmp = nullptr;
-    b->rect = nullptr;
-    b->order_tmp = nullptr;
-    b->stmp = b->total = nullptr;
+    for (Lane &l : b->lane) {
+        l.cnt = l.off = l.keys = l.keys_alt = l.vals_alt = l.sort_tmp = nullptr;
+        l.rect = nullptr;
+        l.order_tmp = nullptr;
+        l.stmp = l.total = nullptr;
+    }
+    b->n_lanes = 1;
     b->d_desc = nullptr;
     b->d_queue = b->d_overflow = nullptr;
     b->d_loss = b->d_bc = nullptr;
@@ -144,48 +168,84 @@ void free_plan(rgrt_batch *b)
     b->exec_step = b->exec_fwd = nullptr;
 }
 
+// A lane's scratch: E (view, Gaussian) pairs and cap keys of one scan at a time.
+struct Need {
+    int64_t E = 1, N = 1;
+    uint32_t cap = 1;
+    int views = 0;
+    bool order = false;
+};
+
+size_t lane_bytes(const Need &n)
+{
+    return sizeof(uint32_t) * (2 * (size_t)n.E + 3 * (size_t)n.cap + sort_tmp_elems(n.cap, n.views)) +
+           sizeof(uint2) * (size_t)n.E + (n.order ? order_tmp_bytes(n.N) : 0) +
+           sizeof(unsigned long long) * (scan_tmp_elems(n.E) + 2);
+}
+
+int alloc_count(rgrt_batch *b, Lane &l, const Need &n)
+{
+    BTRY(balloc(b, (void **)&l.cnt, sizeof(uint32_t) * n.E));
+    BTRY(balloc(b, (void **)&l.off, sizeof(uint32_t) * n.E));
+    BTRY(balloc(b, (void **)&l.rect, sizeof(uint2) * n.E));
+    if (n.order) BTRY(balloc(b, &l.order_tmp, order_tmp_bytes(n.N)));
+    BTRY(balloc(b, (void **)&l.stmp, sizeof(unsigned long long) * scan_tmp_elems(n.E)));
+    BTRY(balloc(b, (void **)&l.total, sizeof(unsigned long long) * 2));
+    return RGRT_OK;
+}
+
+int alloc_keys(rgrt_batch *b, Lane &l, const Need &n)
+{
+    BTRY(balloc(b, (void **)&l.keys, sizeof(uint32_t) * n.cap));
+    BTRY(balloc(b, (void **)&l.keys_alt, sizeof(uint32_t) * n.cap));
+    BTRY(balloc(b, (void **)&l.vals_alt, sizeof(uint32_t) * n.cap));
+    BTRY(balloc(b, (void **)&l.sort_tmp, sizeof(uint32_t) * sort_tmp_elems(n.cap, n.views)));
+    return RGRT_OK;
+}
+
 // measure every scan's key count with one real binning pass, size the buffers
 int plan(rgrt_batch *b)
 {
     free_plan(b);
     cudaStream_t s = b->stream;
-    int64_t Emax = 1, Nmax = 1;
+    Lane &l0 = b->lane[0];
+    Need all, small;   // of every scan, of the small ones
+    all.order = small.order = !b->cone;
     for (auto &x : b->sc) {
-        Emax = std::max<int64_t>(Emax, x.E);
-        Nmax = std::max<int64_t>(Nmax, x.N);
+        all.E = std::max<int64_t>(all.E, x.E);
+        all.N = std::max<int64_t>(all.N, x.N);
     }
-    BTRY(balloc(b, (void **)&b->cnt, sizeof(uint32_t) * Emax));
-    BTRY(balloc(b, (void **)&b->off, sizeof(uint32_t) * Emax));
-    BTRY(balloc(b, (void **)&b->rect, sizeof(uint2) * Emax));
-    if (!b->cone) BTRY(balloc(b, &b->order_tmp, order_tmp_bytes(Nmax)));
-    BTRY(balloc(b, (void **)&b->stmp, sizeof(unsigned long long) * scan_tmp_elems(Emax)));
-    BTRY(balloc(b, (void **)&b->total, sizeof(unsigned long long) * 2));
+    BTRY(alloc_count(b, l0, all));
     b->grid_f = persistent_grid(b->cone, b->tile_w * b->tile_h);
-    uint32_t capmax = 1;
-    int vmax = 0;
+    int n_small = 0;
     b->keys_capacity = 0;
     for (int i = 0; i < b->n; i++) {
         BatchScan &x = b->sc[i];
         DevGeom dg = x.geom->dg;
         dg.v0 = 0;
         BK(launch_records(x.g->mu, x.g->ls, x.g->q, x.g->rho, x.N, x.g->rec, x.g->crec, nullptr, s));
-        BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, b->cnt, b->rect, s));
-        BK(launch_scan(b->cnt, b->off, x.E, b->total, b->stmp, s));
+        BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, l0.cnt, l0.rect, s));
+        BK(launch_scan(l0.cnt, l0.off, x.E, l0.total, l0.stmp, s));
         unsigned long long K = 0;
-        BK(cudaMemcpyAsync(&K, b->total, sizeof(K), cudaMemcpyDeviceToHost, s));
+        BK(cudaMemcpyAsync(&K, l0.total, sizeof(K), cudaMemcpyDeviceToHost, s));
         BK(cudaStreamSynchronize(s));
         unsigned long long cap = K + K / 4 + 4096;
         if (cap >= 0xffffffffull) return report_error(RGRT_E_CAPACITY, "a scan of the batch has more than 2^32 tile entries");
         x.cap = (uint32_t)cap;
         x.keys = (int64_t)K;
         x.large = (int64_t)x.T >= 16 * (int64_t)b->grid_f;
-        x.rect = b->rect;
         if (!b->cone) {
             if (!x.large) BTRY(balloc(b, (void **)&x.rect, sizeof(uint2) * (size_t)std::max<int64_t>(x.E, 1)));
             BTRY(balloc(b, (void **)&x.order, sizeof(uint32_t) * (size_t)std::max<int64_t>(x.N, 1)));
         }
-        capmax = std::max(capmax, x.cap);
-        if (x.lbits >= 0) vmax = std::max(vmax, x.geom->dg.n_views);
+        if (!x.large) n_small++;
+        for (Need *n : { &all, &small }) {
+            if (n == &small && x.large) continue;
+            n->E = std::max<int64_t>(n->E, x.E);
+            n->N = std::max<int64_t>(n->N, x.N);
+            n->cap = std::max(n->cap, x.cap);
+            if (x.lbits >= 0) n->views = std::max(n->views, x.geom->dg.n_views);
+        }
         b->keys_capacity += cap;
         BTRY(balloc(b, (void **)&x.vals, sizeof(uint32_t) * (size_t)x.cap));
         BTRY(balloc(b, (void **)&x.ranges, sizeof(uint2) * (size_t)x.T));
@@ -196,10 +256,31 @@ int plan(rgrt_batch *b)
         x.nblk = loss_blocks(x.R);
         BTRY(balloc(b, (void **)&x.partial, sizeof(double) * (size_t)x.nblk));
     }
-    BTRY(balloc(b, (void **)&b->keys, sizeof(uint32_t) * capmax));
-    BTRY(balloc(b, (void **)&b->keys_alt, sizeof(uint32_t) * capmax));
-    BTRY(balloc(b, (void **)&b->vals_alt, sizeof(uint32_t) * capmax));
-    BTRY(balloc(b, (void **)&b->sort_tmp, sizeof(uint32_t) * sort_tmp_elems(capmax, vmax)));
+    BTRY(alloc_keys(b, l0, all));
+    BTRY(balloc(b, (void **)&b->d_desc, sizeof(ScanDesc) * std::max(n_small, 1)));
+    BTRY(balloc(b, (void **)&b->d_queue, sizeof(uint32_t) * 2));
+    BTRY(balloc(b, (void **)&b->d_overflow, sizeof(uint32_t)));
+    BTRY(balloc(b, (void **)&b->d_loss, sizeof(float) * b->n));
+    BTRY(balloc(b, (void **)&b->d_bc, sizeof(float) * 2));
+    // the other lanes are a convenience: as many as the bound and the memory allow
+    const size_t each = lane_bytes(small), left = b->ctx->budget - std::min(b->ctx->budget, b->ctx->used);
+    const size_t most = std::min(LANE_BYTES, left / 16);
+    while (b->distinct && b->n_lanes < LANES && b->n_lanes < n_small && each * b->n_lanes <= most) {
+        Lane &l = b->lane[b->n_lanes];
+        const size_t before = b->allocs.size();
+        if (alloc_count(b, l, small) != RGRT_OK || alloc_keys(b, l, small) != RGRT_OK) {
+            cudaGetLastError();
+            for (; b->allocs.size() > before; b->allocs.pop_back())
+                ctx_free(b->ctx, b->allocs.back().first, b->allocs.back().second);
+            break;
+        }
+        b->n_lanes++;
+    }
+    int turn = 0;
+    for (auto &x : b->sc) {
+        x.lane = x.large ? 0 : turn++ % b->n_lanes;
+        if (!x.rect) x.rect = b->lane[x.lane].rect;
+    }
     // A scan whose tiles fill the GPU for 16 waves or more gains nothing from
     // sharing the persistent launches: it is binned, projected, and its loss
     // and adjoint taken back to back with launches of its own, while its
@@ -231,41 +312,56 @@ int plan(rgrt_batch *b)
     if (items >= 0xffffffffull) return report_error(RGRT_E_CAPACITY, "too many tiles in the batch");
     b->total_items = (uint32_t)items;
     b->n_small = (int)hd.size();
-    BTRY(balloc(b, (void **)&b->d_desc, sizeof(ScanDesc) * std::max<size_t>(hd.size(), 1)));
     if (!hd.empty())
         BK(cudaMemcpyAsync(b->d_desc, hd.data(), sizeof(ScanDesc) * hd.size(), cudaMemcpyHostToDevice, s));
-    BTRY(balloc(b, (void **)&b->d_queue, sizeof(uint32_t) * 2));
-    BTRY(balloc(b, (void **)&b->d_overflow, sizeof(uint32_t)));
-    BTRY(balloc(b, (void **)&b->d_loss, sizeof(float) * b->n));
-    BTRY(balloc(b, (void **)&b->d_bc, sizeof(float) * 2));
     BK(cudaStreamSynchronize(s));
     return RGRT_OK;
 }
 
+// The batch's stream goes on when the lanes are done; the lanes go on from where
+// it is.
+int join_lanes(rgrt_batch *b)
+{
+    for (int i = 1; i < b->n_lanes; i++) {
+        BK(cudaEventRecord(b->lane[i].ev, b->lane[i].s));
+        BK(cudaStreamWaitEvent(b->stream, b->lane[i].ev, 0));
+    }
+    return RGRT_OK;
+}
+
+int fork_lanes(rgrt_batch *b)
+{
+    BK(cudaEventRecord(b->lane[0].ev, b->stream));
+    for (int i = 1; i < b->n_lanes; i++) BK(cudaStreamWaitEvent(b->lane[i].s, b->lane[0].ev, 0));
+    return RGRT_OK;
+}
+
 // binning of scan i into its own sorted id list and tile ranges
-int enqueue_bin_scan(rgrt_batch *b, int i, cudaStream_t s)
+int enqueue_bin_scan(rgrt_batch *b, int i)
 {
     {
         BatchScan &x = b->sc[i];
+        Lane &l = b->lane[x.lane];
+        cudaStream_t s = l.s;
         DevGeom dg = x.geom->dg;
         dg.v0 = 0;
         BK(launch_records(x.g->mu, x.g->ls, x.g->q, x.g->rho, x.N, x.g->rec, x.g->crec, nullptr, s));
-        BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, b->cnt, x.rect, s));
-        BK(launch_scan(b->cnt, b->off, x.E, b->total, b->stmp, s));
+        BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, l.cnt, x.rect, s));
+        BK(launch_scan(l.cnt, l.off, x.E, l.total, l.stmp, s));
         // the scan's total (on the device) is the number of keys this step
         // emits: the sort and the ranges take only those (at most the planned
         // capacity; an item past it writes padding keys, which sort last and
         // map to no tile, and raises the overflow flag)
-        BK(launch_emit(dg, dg.n_views, x.N, b->cnt, b->off, x.rect, b->keys, x.vals, x.cap,
+        BK(launch_emit(dg, dg.n_views, x.N, l.cnt, l.off, x.rect, l.keys, x.vals, x.cap,
                        b->d_overflow, s, x.lbits));
         if (x.lbits >= 0)
-            BK(launch_sort_views(b->keys, x.vals, b->keys_alt, b->vals_alt, x.cap, x.bits, b->off, x.N,
-                                 dg.n_views, b->sort_tmp, s, nullptr, b->total, sort_shift(dg)));
+            BK(launch_sort_views(l.keys, x.vals, l.keys_alt, l.vals_alt, x.cap, x.bits, l.off, x.N,
+                                 dg.n_views, l.sort_tmp, s, nullptr, l.total, sort_shift(dg)));
         else
-            BK(launch_sort(b->keys, x.vals, b->keys_alt, b->vals_alt, x.cap, x.bits, b->sort_tmp, s, nullptr,
-                           b->total, sort_shift(dg)));
+            BK(launch_sort(l.keys, x.vals, l.keys_alt, l.vals_alt, x.cap, x.bits, l.sort_tmp, s, nullptr,
+                           l.total, sort_shift(dg)));
         BK(cudaMemsetAsync(x.ranges, 0, sizeof(uint2) * (size_t)x.T, s));
-        BK(launch_ranges(b->keys, x.cap, x.ranges, x.T, s, b->total, (uint32_t)x.geom->tiles_per_view,
+        BK(launch_ranges(l.keys, x.cap, x.ranges, x.T, s, l.total, (uint32_t)x.geom->tiles_per_view,
                          x.lbits));
     }
     return RGRT_OK;
@@ -285,10 +381,12 @@ int enqueue_forward_large(rgrt_batch *b, int i, cudaStream_t s)
 int enqueue_forward(rgrt_batch *b, cudaStream_t s)
 {
     BK(cudaMemsetAsync(b->d_overflow, 0, sizeof(uint32_t), s));
+    BTRY(fork_lanes(b));
     for (int i = 0; i < b->n; i++) {
-        BTRY(enqueue_bin_scan(b, i, s));
+        BTRY(enqueue_bin_scan(b, i));
         if (b->sc[i].large) BTRY(enqueue_forward_large(b, i, s));
     }
+    BTRY(join_lanes(b));
     if (b->n_small > 0) {
         BK(cudaMemsetAsync(b->d_queue, 0, sizeof(uint32_t), s));
         BK(launch_forward_persistent(b->cone, b->d_desc, b->n_small, b->total_items, b->d_queue,
@@ -318,7 +416,7 @@ int enqueue_adjoint(rgrt_batch *b, int i, cudaStream_t s)
                                 RGRT_KERNEL_GAUSSIAN, s));
         return RGRT_OK;
     }
-    BK(launch_order(x.g->crec, x.N, b->order_tmp, x.order, s));
+    BK(launch_order(x.g->crec, x.N, b->lane[x.lane].order_tmp, x.order, s));
     BK(launch_adjoint(dg, dg.n_views, x.N, x.keys, x.order, x.g->rec, x.g->crec, x.rect, x.dLdI, x.grad,
                       RGRT_KERNEL_GAUSSIAN, s));
     return RGRT_OK;
@@ -328,31 +426,37 @@ int enqueue_step(rgrt_batch *b, const float *const *y, int loss, const rgrt_adam
 {
     BK(cudaMemsetAsync(b->d_overflow, 0, sizeof(uint32_t), s));
     // large scans: binning, forward, loss and adjoint back to back
+    BTRY(fork_lanes(b));
     for (int i = 0; i < b->n; i++) {
-        BTRY(enqueue_bin_scan(b, i, s));
+        BTRY(enqueue_bin_scan(b, i));
         BatchScan &x = b->sc[i];
         if (!x.large) continue;
         BTRY(enqueue_forward_large(b, i, s));
         BTRY(enqueue_loss(b, i, y, loss, hp, s));
         BTRY(enqueue_adjoint(b, i, s));
     }
+    BTRY(join_lanes(b));
     // small scans: one persistent forward and (cone beam) one persistent adjoint
     if (b->n_small > 0) {
         BK(cudaMemsetAsync(b->d_queue, 0, sizeof(uint32_t), s));
         BK(launch_forward_persistent(b->cone, b->d_desc, b->n_small, b->total_items, b->d_queue,
                                      b->tile_w * b->tile_h, b->grid_f, s));
+        BTRY(fork_lanes(b));
         for (int i = 0; i < b->n; i++)
-            if (!b->sc[i].large) BTRY(enqueue_loss(b, i, y, loss, hp, s));
+            if (!b->sc[i].large) BTRY(enqueue_loss(b, i, y, loss, hp, b->lane[b->sc[i].lane].s));
         if (b->cone) {
+            BTRY(join_lanes(b));
             BK(cudaMemsetAsync(b->d_queue + 1, 0, sizeof(uint32_t), s));
             BK(launch_adjoint_persistent(b->tile_w, b->d_desc, b->n_small, b->total_items, b->d_queue + 1, s));
         } else {
             for (int i = 0; i < b->n; i++)
-                if (!b->sc[i].large) BTRY(enqueue_adjoint(b, i, s));
+                if (!b->sc[i].large) BTRY(enqueue_adjoint(b, i, b->lane[b->sc[i].lane].s));
+            BTRY(join_lanes(b));
         }
     }
     // parameter chains and Adam last: an overflow flagged by any scan's
     // binning skips every update
+    BTRY(fork_lanes(b));
     for (int i = 0; i < b->n; i++) {
         BatchScan &x = b->sc[i];
         if (x.N == 0) continue;
@@ -360,7 +464,15 @@ int enqueue_step(rgrt_batch *b, const float *const *y, int loss, const rgrt_adam
         float *gf = x.gflat;
         const int64_t N = x.N;
         BK(launch_param_chain(g->mu, g->ls, g->q, g->rho, N, x.grad, gf, gf + 3 * N, gf + 6 * N,
-                              gf + 10 * N, s));
+                              gf + 10 * N, b->lane[x.lane].s));
+    }
+    BTRY(join_lanes(b));
+    for (int i = 0; i < b->n; i++) {
+        BatchScan &x = b->sc[i];
+        if (x.N == 0) continue;
+        rgrt_gauss *g = x.g;
+        float *gf = x.gflat;
+        const int64_t N = x.N;
         const AdamArrays arr = { { g->mu, g->ls, g->q, g->rho },
                                  { hp->lr_mu, hp->lr_logscale, hp->lr_quat, hp->lr_rho } };
         BK(launch_adam(arr, gf, g->adam_m, g->adam_v, N, hp->beta1, hp->beta2, hp->eps, 1.0f, 1.0f, b->d_bc,
@@ -462,6 +574,7 @@ int rgrt_batch_create(rgrt_ctx *ctx, int n_scans, rgrt_gauss *const *g, const rg
             return report_error(RGRT_E_INVAL,
                                 "all scans of a batch need the same ray kind and tile shape");
         }
+        for (int k = 0; k < i; k++) b->distinct = b->distinct && g[k] != g[i];
         BatchScan &x = b->sc[i];
         x.g = g[i];
         x.geom = geom[i];
@@ -480,6 +593,11 @@ int rgrt_batch_create(rgrt_ctx *ctx, int n_scans, rgrt_gauss *const *g, const rg
     cudaError_t e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming);
+    b->lane[0].s = b->stream;
+    for (Lane &l : b->lane) {
+        if (e == cudaSuccess && !l.s) e = cudaStreamCreateWithFlags(&l.s, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&l.ev, cudaEventDisableTiming);
+    }
     if (e == cudaSuccess) e = cudaMallocHost((void **)&b->h_pin, sizeof(float) * (3 + n_scans));
     if (e != cudaSuccess) {
         rgrt_batch_destroy(b);
@@ -503,6 +621,10 @@ int rgrt_batch_destroy(rgrt_batch *b)
     free_plan(b);
     if (b->ev_in) cudaEventDestroy(b->ev_in);
     if (b->ev_out) cudaEventDestroy(b->ev_out);
+    for (Lane &l : b->lane) {
+        if (l.ev) cudaEventDestroy(l.ev);
+        if (l.s && l.s != b->stream) cudaStreamDestroy(l.s);
+    }
     if (b->stream) cudaStreamDestroy(b->stream);
     if (b->h_pin) cudaFreeHost(b->h_pin);
     delete b;

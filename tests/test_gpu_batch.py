@@ -217,3 +217,27 @@ def test_batch_tile_lists_match_the_oracle(env, oracle):
             assert np.array_equal(start, rstart), (rep, i)
             tile = np.repeat(np.arange(start.size - 1), np.diff(start))
             assert np.array_equal(gid[np.lexsort((gid, tile))], rgid), (rep, i)
+
+
+@pytest.mark.parametrize("shared", [False, True])
+@pytest.mark.parametrize("kind", ["parallel", "cone"])
+def test_batch_bins_scans_side_by_side(env, kind, shared):
+    """More scans than binning streams, of both ray kinds and uneven sizes, and
+    scans that share one Gaussian set (one stream): two steps equal the scans'
+    own projections, bit for bit."""
+    torch, rg, ctx = env
+    sizes = [(2, 33), (9, 64), (1, 8), (5, 48), (3, 96), (7, 40)]
+    gds = [synth.geom_parallel(v, s, s, 2.0 / s, 2.0 / s, -4.0, 4.0) if kind == "parallel" else
+           synth.geom_cone(v, s, s, 4.0 / s, 4.0 / s, 4.0, 8.0) for v, s in sizes]
+    geoms = [rg.Geometry(ctx, gd) for gd in gds]
+    gs = [rg.Gaussians(ctx, *_dev(torch, synth.gaussians_uniform(300 + 700 * (i % 4), 60 + i, log_sigma=math.log(0.05))))
+          for i in range(1 if shared else len(sizes))]
+    gs = gs * len(sizes) if shared else gs
+    b = rg.Batch(ctx, gs, geoms)
+    outs = [torch.empty(g.n_rays, device="cuda") for g in geoms]
+    for _ in range(2):
+        b.forward(outs)
+        for g, geom, o in zip(gs, geoms, outs):
+            ref = rg.project_forward(ctx, g, geom, torch.empty(geom.n_rays, device="cuda"))
+            torch.cuda.synchronize()
+            assert torch.equal(o, ref)
