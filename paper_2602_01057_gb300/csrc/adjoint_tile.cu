@@ -10,9 +10,9 @@
 // list at a time (all lanes of a warp read the same ray: broadcasts), keeping
 // that Gaussian's view-space moments in registers -- no cross-thread
 // reduction -- and finishes with the parameter chain and one set of vector
-// atomics per (Gaussian, tile).  The tile list is ordered by footprint
-// position, so the 32 Gaussians of a warp sit close together: rows and
-// 8-column groups that none of their boxes touches are skipped.  Within a row
+// atomics per (Gaussian, tile).  On the cone beam the tile list is ordered by
+// footprint position, so the 32 Gaussians of a warp sit close together: rows and
+// 4-column groups that none of their boxes touches are skipped.  Within a row
 // the Q and A quadratics are evaluated in Horner form in du with the dv terms
 // hoisted.  For 3-D PET the LOR slope kappa varies from column to column:
 // the moments carry its powers (pet3d_chain).
@@ -229,9 +229,10 @@ __device__ __forceinline__ void adjoint_tile(const DevGeom &g, uint32_t tile, ui
             // and its rows, two at a time in packed binary32, need only five
             // kappa-free sums (h, h v~, h v~^2, p = h arg), folded into the 15
             // moments with the column's du and kappa powers afterwards.  (The
-            // list's order keeps the boxes of a warp alike; walking the union
-            // of them in step, row by row, took 76.7 ms instead of 59.4 on 3-D
-            // PET of 200,000 Gaussians and 33 million bins.)
+            // list's order by box size keeps the loops of a warp alike: 54.9 ms
+            // on 3-D PET of 200,000 Gaussians and 33 million bins, 59.4 ordered
+            // by position; walking the union of a warp's boxes in step, row by
+            // row, took 76.7.)
             const float4 c0 = r.c0, c1 = r.c1, c2 = r.c2;
             float s[15];
 #pragma unroll

@@ -128,8 +128,8 @@ cudaError_t launch_sort(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint
                         uint32_t n, int bits, uint32_t *tmp, cudaStream_t s, bool *in_alt = nullptr,
                         const unsigned long long *n_dev = nullptr, int shift = 0);
 // First key bit that the tile sort takes.  Cone-beam and 3-D PET tiles order
-// their lists by position code, then id (the tile adjoint skips rows and
-// columns that a warp's Gaussians leave empty); parallel rays, whose adjoint
+// their lists by the key's code, then id (position: the tile adjoint skips rows
+// and columns that a warp's Gaussians leave empty; box size on 3-D PET); parallel rays, whose adjoint
 // reads no lists, by id alone, which saves the pass over the code's 8 bits (PET
 // ring sort 1.85 -> 0.97 ms, its forward 5.7 ms either way).
 inline int sort_shift(const DevGeom &g) { return g.kind == GM_PARALLEL ? 8 : 0; }
