@@ -58,12 +58,13 @@ MUFU_LANES_PER_SM = 16
 # kernel sources hash to the recorded digest (otherwise the bench line
 # reports null)
 TRAFFIC = {
-    ("c2", "k_forward"): (261.9e6, "7259bc5991d372fe"),
-    ("c2", "k_adjoint"): (275.9e6, "7259bc5991d372fe"),
-    ("c3", "k_forward"): (472.0e6, "7259bc5991d372fe"),
-    ("c3", "k_adjoint"): (477.1e6, "7259bc5991d372fe"),
+    ("c2", "k_forward"): (262.0e6, "ebb4b6c5a81cbe24"),
+    ("c2", "k_adjoint"): (278.0e6, "ebb4b6c5a81cbe24"),
+    ("c3", "k_forward"): (525.0e6, "ebb4b6c5a81cbe24"),
+    ("c3", "k_adjoint"): (1837.0e6, "ebb4b6c5a81cbe24"),
 }
-KERNEL_SOURCES = ("paper_2602_01057_gb300/csrc/project.cu", "paper_2602_01057_gb300/csrc/pair.cuh")
+KERNEL_SOURCES = tuple("paper_2602_01057_gb300/csrc/" + f for f in (
+    "project.cu", "adjoint.cu", "adjoint_tile.cu", "pair.cuh", "packed.cuh", "view.cuh"))
 WORKLOADS = {
     "c2": "cone-beam CT fwd+bwd (L2 + Adam): 50,000 Gaussians fitted to a 12-ellipsoid phantom, "
           "180 views over 360 deg, 256x256 detector, source-origin 1000 mm, source-detector 1500 mm",
@@ -393,20 +394,21 @@ def sources_digest():
     return h.hexdigest()[:16]
 
 
-def sort_passes(tiles, n_views=1):
+def sort_passes(tiles, n_views=1, code_bits=8):
     """Radix passes of the tile sort: 8-bit digits over the tile within the
-    view plus an 8-bit position code (each view's keys are sorted on their
-    own while view << bits of the tile fits 24 bits; else over the tile id of
-    all the views)."""
+    view plus an 8-bit position code (code_bits = 0: without it, as the
+    parallel-ray geometries sort; each view's keys are sorted on their own
+    while view << bits of the tile fits 24 bits; else over the tile id of all
+    the views)."""
     tpv = max(1, tiles // max(1, n_views))
     lb = math.ceil(math.log2(tpv)) if tpv > 1 else 0
     if (n_views << lb) < (1 << 24):
-        return (lb + 8 + 7) // 8
-    bits = max(1, math.ceil(math.log2(max(tiles, 2)))) + 8
+        return (lb + code_bits + 7) // 8
+    bits = max(1, math.ceil(math.log2(max(tiles, 2)))) + code_bits
     return (bits + 7) // 8
 
 
-def binning_bytes(n_gauss, n_views, keys, tiles):
+def binning_bytes(n_gauss, n_views, keys, tiles, code_bits=8):
     """Algorithmic DRAM bytes of one binning (cull, scan, emit, sort, ranges):
     per (view, Gaussian) the 48-byte culling record read and its count and
     pixel box written (60 B), the scan's read and write (8 B), the emit's
@@ -414,12 +416,12 @@ def binning_bytes(n_gauss, n_views, keys, tiles):
     ranges' 4-byte read; 8 B per tile range."""
     e = float(n_gauss) * n_views
     parts = dict(k_cull=60.0 * e, scan=8.0 * e, k_emit=16.0 * e + 8.0 * keys,
-                 radix_sort=16.0 * sort_passes(tiles, n_views) * keys, k_ranges=4.0 * keys + 8.0 * tiles)
+                 radix_sort=16.0 * sort_passes(tiles, n_views, code_bits) * keys, k_ranges=4.0 * keys + 8.0 * tiles)
     return parts
 
 
 def roofline(kernels, pairs, keys, n_gauss, n_views, tiles, n_sm, sm_mhz, clock_note, peaks, workload,
-             traffic_table=None, n_tof=0):
+             traffic_table=None, n_tof=0, code_bits=8):
     """Roofline of the integration kernels (FP32 issue and MUFU against the
     SM count read from the device and the sampled clock) and of the binning
     kernels (HBM against the measured copy bandwidth).  The top-level
@@ -447,7 +449,7 @@ def roofline(kernels, pairs, keys, n_gauss, n_views, tiles, n_sm, sm_mhz, clock_
                          sfu=dict(achieved=sfu, peak=mufu_peak, unit="T MUFU op/s", frac=sfu / mufu_peak),
                          kernel_ms_per_step=step_ms, launches_per_step=kernels[name]["launches"] / max(STEPS_TIMED[0], 1),
                          ms_per_launch=kms, traffic=tr)
-    bb = binning_bytes(n_gauss, n_views, keys, tiles)
+    bb = binning_bytes(n_gauss, n_views, keys, tiles, code_bits)
     bin_ms = sum(kernels[k]["ms"] for k in bb) / max(STEPS_TIMED[0], 1)
     tot = sum(bb.values())
     gbs = tot / (bin_ms / 1e3) / 1e9 if bin_ms > 0 else 0.0
@@ -567,7 +569,8 @@ def measure_step(args, name, rgrt, ctx, dev, seed, world, rank, local, cpu=True,
     n_views = synth.num_rays(gd) // (int(gd["n_rows"]) * int(gd["n_cols"]) * max(1, int(gd.get("n_tof", 0))))
     tiles = n_views * geom.tiles_per_view
     roof = roofline(kernels, pairs, st["keys"], int(G["mu"].shape[0]), n_views, tiles, n_sm, sm_mhz, note,
-                    peaks, name, TRAFFIC, n_tof=int(gd.get("n_tof", 0)))
+                    peaks, name, TRAFFIC, n_tof=int(gd.get("n_tof", 0)),
+                    code_bits=0 if gd["kind"] in ("parallel", "pet") else 8)
     line = dict(metric=METRIC, value=value, unit=UNIT, n_gpus=world, steps=args.steps,
                 warmup=args.warmup, ms_per_step=ms_max / args.steps, higher_is_better=True,
                 scaling="weak", vs_baseline=None, dtype="f32", data="synthetic",

@@ -314,8 +314,9 @@ int rgrt_batch_forward(rgrt_batch *b, float *const *out_I, void *stream);
 
 /* One optimisation step of every scan, as loss_step does for one: forward,
  * loss against y[i] (device arrays), adjoint (the small scans: one persistent
- * forward and one persistent adjoint launch over all of them; a large scan:
- * binning, forward, loss and adjoint back to back, its lists still in L2),
+ * forward launch over all of them, and one persistent adjoint launch (cone
+ * beam) or one per scan; a large scan: binning, forward, loss and adjoint back
+ * to back, its lists still in L2),
  * then the parameter chains and Adam (step t) of every scan.  loss_out[n_scans] (host or
  * device, may be null) receives the losses.  Captured in a CUDA graph that is
  * replayed while y, loss and hp stay the same.  Synchronises with `stream`. */
