@@ -15,7 +15,7 @@
 // blocks, and every warp compacts the records that touch its own.
 //
 // Bound by issue.  Measured on a GB300, 50,000 Gaussians on 256^3: the kernel
-// 0.92 -> 0.58 ms (every warp used to read every record of its brick).
+// 0.92 -> 0.56 ms (every warp used to read every record of its brick).
 #include "packed.cuh"
 #include "rgrt_internal.h"
 
@@ -148,8 +148,8 @@ __global__ void __launch_bounds__(VB) k_voxelize(const float4 *__restrict__ rec,
     const int i = bx * 8 + (lane & 7);
     const int j = by * 8 + (w & 1) * 4 + (lane >> 3);
     const int k0 = bz * BZ + (w >> 1) * VZ;
-    const float x = v.ox + (float)i * v.sx, y = v.oy + (float)j * v.sy, z0 = v.oz + (float)k0 * v.sz;
-    const f2 zA = pk(z0, z0 + v.sz), zB = pk(z0 + 2.0f * v.sz, z0 + 3.0f * v.sz);
+    const float x = fmaf((float)i, v.sx, v.ox), y = fmaf((float)j, v.sy, v.oy), z0 = fmaf((float)k0, v.sz, v.oz);
+    const f2 zA = pk(z0, z0 + v.sz), zB = pk(fmaf(2.0f, v.sz, z0), fmaf(3.0f, v.sz, z0));
     // the brick's blocks of 8 x 4 x VZ voxels: first centre and half extents
     const float cx = v.ox + ((float)(bx * 8) + 3.5f) * v.sx, cy = v.oy + ((float)(by * 8) + 1.5f) * v.sy;
     const float cz = v.oz + ((float)(bz * BZ) + 0.5f * (float)(VZ - 1)) * v.sz;
@@ -200,9 +200,12 @@ __global__ void __launch_bounds__(VB) k_voxelize(const float4 *__restrict__ rec,
             const float4 g0 = s.g0[e], g1 = s.g1[e];
             const float2 g2 = s.g2[e];
             const float dx = x - g0.x, dy = y - g0.y;
-            // arg(dz) = a0 + dz (b0 + c0 dz): the xy terms once, then VZ voxels along z
-            const float a0 = dx * (g1.x * dx + g1.y * dy) + g1.z * dy * dy;
-            const float b0 = g1.w * dx + g2.x * dy;
+            // arg(dz) = a0 + dz (b0 + c0 dz): the xy terms once, then VZ voxels along
+            // z.  The order of the roundings is part of the result (an ulp of arg
+            // decides which side of the cut a voxel falls on, and the last bit of
+            // its value), so it is written out rather than left to contraction.
+            const float a0 = fmaf(dx, fmaf(g1.x, dx, __fmul_rn(g1.y, dy)), __fmul_rn(__fmul_rn(g1.z, dy), dy));
+            const float b0 = fmaf(g2.x, dy, __fmul_rn(g1.w, dx));
             const f2 A0 = pk(a0, a0), B0 = pk(b0, b0), C0 = pk(g2.y, g2.y), nz = pk(-g0.z, -g0.z);
             const f2 dA = add2(zA, nz), dB = add2(zB, nz);
             accA = add2(accA, vox_value<KER>(fma2(dA, fma2(C0, dA, B0), A0), g0.w));

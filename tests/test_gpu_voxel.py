@@ -3,6 +3,7 @@ voxeliser: every voxel of small ragged grids, sampled slabs of a 256^3 grid
 of the cone-beam workload's Gaussians, an empty set, Gaussians off the grid,
 host and device outputs, invalid grids."""
 import math
+import os
 
 import numpy as np
 import pytest
@@ -117,3 +118,21 @@ def test_invalid_grid_rejected(rg, ctx, torch, bad):
         vol["origin"] = (0.0, float("nan"), 0.0)
     with pytest.raises(rg.RgrtError):
         rg.gaussians_voxelize(ctx, gauss(rg, ctx, torch, G), vol, np.zeros(64, np.float32))
+
+
+def golden_scene():
+    """Gaussians and a ragged grid over several bricks of the kernel."""
+    G = synth.gaussians_uniform(40, 47, half_box=0.8, log_sigma=math.log(0.2))
+    return G, dict(origin=(-0.91, -0.87, -1.04), size=(0.17, 0.21, 0.113), dims=(11, 9, 18))
+
+
+@pytest.mark.parametrize("kernel", ["gaussian", "epanechnikov"])
+def test_volume_bits(rg, ctx, torch, kernel):
+    """The exponent's roundings are part of the result (they decide the voxels
+    at the cut): the volume equals the stored one bit for bit, which the scalar
+    form of the kernel (one voxel at a time, every record of the brick) gave."""
+    G, vol = golden_scene()
+    V = rg.gaussians_voxelize(ctx, gauss(rg, ctx, torch, G).set_kernel(kernel), vol)
+    gold = np.load(os.path.join(os.path.dirname(__file__), "golden", "voxels.npz"))[kernel]
+    assert np.count_nonzero(gold) > 1000
+    np.testing.assert_array_equal(V.view(np.uint32), gold.view(np.uint32))
