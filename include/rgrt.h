@@ -115,8 +115,8 @@ typedef struct rgrt_geom rgrt_geom;
 typedef struct {
     int32_t kind;        /* RGRT_GEOM_* */
     int32_t n_views;     /* CT projections / PET sinogram angles (PET_3D: per ring difference) */
-    int32_t n_rows;      /* CT detector rows / PET planes / PET_3D rings */
-    int32_t n_cols;      /* CT detector columns / PET radial bins */
+    int32_t n_rows;      /* CT detector rows / PET planes / PET_3D rings, <= 65536 */
+    int32_t n_cols;      /* CT detector columns / PET radial bins, <= 65536 */
     const double *angles;/* CT: n_views angles in radians (host memory); PET: null or n_views angles */
     double pitch_u, pitch_v;
     double t_a, t_b;     /* CT_PARALLEL segment */

@@ -576,8 +576,10 @@ int validate_desc(const rgrt_geom_desc *d)
     if ((tw != 8 && tw != 16 && tw != 32) || th % 4 || th > 32 || tw * th > 256 || tw * th < 32)
         return fail(RGRT_E_INVAL, "tile %dx%d: width 8, 16 or 32, height a multiple of 4 up to 32, "
                     "32..256 rays", tw, th);
-    if ((d->n_cols + tw - 1) / tw > 65535 || (d->n_rows + th - 1) / th > 65535)
-        return fail(RGRT_E_INVAL, "too many tiles per detector axis");
+    // a Gaussian's pixel box is kept as four 16-bit indices
+    if (d->n_cols > MAX_DETECTOR_SIDE || d->n_rows > MAX_DETECTOR_SIDE)
+        return fail(RGRT_E_INVAL, "detector of %d x %d pixels (%d a side at most)", d->n_rows, d->n_cols,
+                    MAX_DETECTOR_SIDE);
     const bool pet = d->kind == RGRT_GEOM_PET_RING || d->kind == RGRT_GEOM_PET_3D;
     if (d->kind == RGRT_GEOM_PET_3D && (d->max_ring_diff < 0 || d->max_ring_diff >= d->n_rows))
         return fail(RGRT_E_INVAL, "max_ring_diff %d outside 0..%d", d->max_ring_diff, d->n_rows - 1);

@@ -51,6 +51,9 @@ int64_t desc_rays(const rgrt_geom_desc *d);
 // pointers.
 void geom_tables(const rgrt_geom_desc *d, float *tab, DevGeom &dg);
 
+// most detector rows or columns: the pixel boxes of k_cull hold 16-bit indices
+constexpr int MAX_DETECTOR_SIDE = 65536;
+
 // Tile indices of pixels below 65,536 without divisions: tile widths are powers
 // of two, and ceil(2^32 / h) reproduces j / h for h <= 32.
 struct TileDiv {

@@ -83,3 +83,20 @@ def test_binding_structs_match_the_header(struct, cls, tmp_path):
     size, offs = _c_layout(struct, names, tmp_path)
     assert ctypes.sizeof(C) == size
     assert [getattr(C, n).offset for n in names] == offs
+
+
+@pytest.mark.parametrize("rows,cols,refused", [(65536, 1, False), (1, 65536, False), (65537, 1, True), (1, 65537, True),
+                                               (8, 600_000, True)])
+def test_detector_sides_beyond_the_boxes_indices_are_rejected(lib, rows, cols, refused):
+    """Pixel boxes hold 16-bit indices: a longer side has its boxes cut short
+    after their tiles were counted.  The call that needs no device to validate a
+    geometry takes smaller detectors still, so an admissible side ends at its
+    own limit (RGRT_E_CAPACITY) and an inadmissible one in validation."""
+    import numpy as np
+
+    from paper_2602_01057_gb300 import rgrt, synth
+    desc, angles = rgrt.make_desc(synth.geom_parallel(1, rows, cols, 1e-3, 1e-3, -1.0, 1.0))
+    out = np.zeros(1, np.float32)
+    rc = rgrt.lib().project_forward_noalloc(ctypes.byref(desc), 0, None, None, None, None, rgrt._ptr(out), None)
+    assert rc == (-1 if refused else -3), rc
+    del angles
