@@ -15,17 +15,21 @@
 //  * lane k chains Gaussian k's moments (view_chain) into the world-space
 //    gradient that it keeps over the CTA's views.
 // No tile lists, no per-tile atomics: one set of 16 sums per Gaussian and view
-// range, added to the accumulator at the end.
+// range, added to the accumulator at the end.  Footprints far larger than their
+// neighbours', and launches of few Gaussians, are walked in place instead
+// (k_adjoint_direct).
 //
 // Bound by instruction issue (the pixels of the chords, their set-up, and the
 // lanes that wait for a longer chord of the same round).  Against one Gaussian
 // per thread and tile (record gathers, box searches, a chain and 16 atomics
 // for each of the 1.9 tiles of a PET footprint), measured on a GB300: PET ring
-// of 288 x 329 x 63, 200,000 Gaussians 9.6 -> 6.85 ms; 8 raw angles, 100,000
-// 0.73 -> 0.14 ms; 24 angles x 13 time-of-flight bins 4.96 -> 2.87 ms; parallel
-// beam, 1,000 Gaussians on 16 x 64^2 0.34 -> 0.09 ms (that one had 256 CTAs of
+// of 288 x 329 x 63, 200,000 Gaussians 9.6 -> 6.9 ms; 8 raw angles, 100,000
+// 0.73 -> 0.14 ms; 24 angles x 13 time-of-flight bins 4.96 -> 2.83 ms; parallel
+// beam, 1,000 Gaussians on 16 x 64^2 0.34 -> 0.07 ms (that one had 256 CTAs of
 // serial pixels).  Sorting a warp's Gaussians by box area per view took the
 // ring from 8.0 to 6.9 ms: a round's lanes then have chords of like length.
+// Only the Gaussians that meet a band are walked in it (a ring with 13
+// time-of-flight bins, 288 angles: 35.7 -> 33.9 ms).
 #include <type_traits>
 
 #include "packed.cuh"
@@ -82,6 +86,48 @@ struct Band {
     int cb, rb, w, h, st;
 };
 
+// where a walk reads: a staged band, coordinates relative to it ...
+struct Staged {
+    static constexpr int UNROLL = 1, STEP = 2;
+    const float *sg, *su, *sv;
+    Band bd;
+    __device__ __forceinline__ int cb() const { return bd.cb; }
+    __device__ __forceinline__ int rb() const { return bd.rb; }
+    __device__ __forceinline__ int w() const { return bd.w; }
+    __device__ __forceinline__ int h() const { return bd.h; }
+    __device__ __forceinline__ int col0() const { return 0; }
+    __device__ __forceinline__ int plane() const { return bd.h * bd.st; }
+    __device__ __forceinline__ float2 u2(int i) const { return *reinterpret_cast<const float2 *>(su + i); }
+    __device__ __forceinline__ float v(int j) const { return sv[j]; }
+    __device__ __forceinline__ const float *row(int j) const { return sg + j * bd.st; }
+    __device__ __forceinline__ float2 g2(const float *p, int i) const { return *reinterpret_cast<const float2 *>(p + i); }
+};
+
+// ... or the view itself, 2^DIRECT_LG lanes side by side in a row
+constexpr int DIRECT_LG = 2;
+struct Direct {
+    static constexpr int UNROLL = 2, STEP = 2 << DIRECT_LG;
+    const DevGeom &g;
+    const float *I;
+    int lc;
+    __device__ __forceinline__ int cb() const { return 0; }
+    __device__ __forceinline__ int rb() const { return 0; }
+    __device__ __forceinline__ int w() const { return g.n_cols; }
+    __device__ __forceinline__ int h() const { return g.n_rows; }
+    __device__ __forceinline__ int col0() const { return 2 * lc; }
+    __device__ __forceinline__ long long plane() const { return g.stride_tof; }
+    __device__ __forceinline__ float2 u2(int i) const
+    {
+        return make_float2(__ldg(g.utab + i), __ldg(g.utab + min(i + 1, g.n_cols - 1)));
+    }
+    __device__ __forceinline__ float v(int j) const { return __ldg(g.vtab + j); }
+    __device__ __forceinline__ const float *row(int j) const { return I + j * g.stride_row; }
+    __device__ __forceinline__ float2 g2(const float *p, int i) const
+    {
+        return make_float2(__ldg(p + i), i + 1 < g.n_cols ? __ldg(p + i + 1) : 0.0f);
+    }
+};
+
 // cut of the chords: a little outside the pairs' own, so that rounding in the
 // roots loses no pixel (the chord is widened by 0.05 columns as well)
 template <int KER>
@@ -107,31 +153,30 @@ __device__ __forceinline__ void chord(float al, float be, float ga, float xc, fl
 // profile and p = h arg,
 //   m[0..5] = sum h {1, du, dv, du^2, du dv, dv^2},  m[6] = sum p;
 // A is constant along parallel rays, its powers are left to finish().
-template <int KER>
+template <int KER, class Src>
 __device__ __forceinline__ void rows(const DevGeom &g, const float4 &c0, const float4 &c1, const Box &bx, int r0,
-                                     int dr, const Band &bd, const float *sg, const float *su, const float *sv,
-                                     float *m)
+                                     int dr, const Src &src, float *m)
 {
     const float u0 = c0.x, v0 = c0.y, kMuv2 = c0.w, kMvv = c1.x, thr = chord_cut<KER>();
-    const int ilo = max(bx.ilo - bd.cb, 0), ihi = min(bx.ihi - bd.cb, bd.w - 1);
-    const float xc = (u0 - g.u0) * g.uinv - (float)bd.cb;
-    int j = bx.jlo - bd.rb + r0;
+    const int ilo = max(bx.ilo - src.cb(), 0), ihi = min(bx.ihi - src.cb(), src.w() - 1);
+    const float xc = (u0 - g.u0) * g.uinv - (float)src.cb();
+    int j = bx.jlo - src.rb() + r0;
     if (j < 0) j += (-j + dr - 1) / dr * dr;
-    const int je = min(bx.jhi - bd.rb, bd.h - 1);
+    const int je = min(bx.jhi - src.rb(), src.h() - 1);
     const f2 nu0 = pk(-u0, -u0), Muu = pk(c0.z, c0.z);
 #pragma unroll
     for (int q = 0; q < 7; q++) m[q] = 0.0f;
     for (; j <= je; j += dr) {
-        const float dv = sv[j] - v0, dv2 = dv * dv;
+        const float dv = src.v(j) - v0, dv2 = dv * dv;
         const float a1 = kMuv2 * dv, a0 = kMvv * dv2;
         const f2 A1 = pk(a1, a1), A0 = pk(a0, a0);
         int ia = ilo, ie = ihi;
         if (g.uinv != 0.0f && c0.z < 0.0f) chord(c0.z, a1, a0 - thr, xc, g.uinv, ia, ie);
-        const float *gr = sg + j * bd.st;
+        const float *gr = src.row(j);
         f2 h0 = 0, h1 = 0, h2 = 0, q0 = 0;
-#pragma unroll 1
-        for (int i = ia & ~1; i <= ie; i += 2) {
-            const float2 uu = *reinterpret_cast<const float2 *>(su + i), gg = *reinterpret_cast<const float2 *>(gr + i);
+#pragma unroll Src::UNROLL
+        for (int i = (ia & ~1) + src.col0(); i <= ie; i += Src::STEP) {
+            const float2 uu = src.u2(i), gg = src.g2(gr, i);
             const f2 du = add2(pk(uu.x, uu.y), nu0);
             const f2 q = fma2(fma2(Muu, du, A1), du, A0);
             float qx, qy;
@@ -159,19 +204,19 @@ __device__ __forceinline__ void rows(const DevGeom &g, const float4 &c0, const f
 // sigma_T^2.  h carries G = sum_k g_k W_k in place of dL/dI, and four more
 // sums the weights' own gradients: m[7..10] = val dW/dt* (1, du, dv) and
 // val dW/ds^2.
+template <class Src>
 __device__ __forceinline__ void rows_tof(const DevGeom &g, const float4 &c0, const float4 &c1, const float4 &t4,
-                                         const Box &bx, int r0, int dr, const Band &bd, const float *sg,
-                                         const float *su, const float *sv, float *m)
+                                         const Box &bx, int r0, int dr, const Src &src, float *m)
 {
     const float u0 = c0.x, v0 = c0.y;
-    const int ilo = max(bx.ilo - bd.cb, 0), ihi = min(bx.ihi - bd.cb, bd.w - 1);
-    const float xc = (u0 - g.u0) * g.uinv - (float)bd.cb;
-    int j = bx.jlo - bd.rb + r0;
+    const int ilo = max(bx.ilo - src.cb(), 0), ihi = min(bx.ihi - src.cb(), src.w() - 1);
+    const float xc = (u0 - g.u0) * g.uinv - (float)src.cb();
+    int j = bx.jlo - src.rb() + r0;
     if (j < 0) j += (-j + dr - 1) / dr * dr;
-    const int je = min(bx.jhi - bd.rb, bd.h - 1);
+    const int je = min(bx.jhi - src.rb(), src.h() - 1);
     const float s2 = t4.w + g.tof_s2, is2 = 1.0f / s2, ns = Kern<0>::QSCALE * is2;
     const float nrm = rsqrtf(2.0f * 3.14159265358979324f / is2);
-    const int plane = bd.h * bd.st;
+    const auto plane = src.plane();
 #pragma unroll
     for (int q = 0; q < 11; q++) m[q] = 0.0f;
     const f2 NS = pk(ns, ns), TH = pk(g.tof_h, g.tof_h), MINUS1 = pk(-1.0f, -1.0f);
@@ -186,33 +231,33 @@ __device__ __forceinline__ void rows_tof(const DevGeom &g, const float4 &c0, con
         if (i > ie) {
             j += dr;
             if (j > je) break;
-            dv = sv[j] - v0;
+            dv = src.v(j) - v0;
             const float dv2 = dv * dv;
             a1 = c0.w * dv;
             a0 = c1.x * dv2;
             i = ilo;
             ie = ihi;
             if (g.uinv != 0.0f && c0.z < 0.0f) chord(c0.z, a1, a0 - chord_cut<0>(), xc, g.uinv, i, ie);
-            i &= ~1;
+            i = (i & ~1) + src.col0();
         }
         if (i <= ie) {
-            const float2 uu = *reinterpret_cast<const float2 *>(su + i);
+            const float2 uu = src.u2(i);
             const int at = i;
-            i += 2;
+            i += Src::STEP;
             const float du0 = uu.x - u0, du1 = uu.y - u0;
             const float q0 = fmaf(fmaf(c0.z, du0, a1), du0, a0), q1 = fmaf(fmaf(c0.z, du1, a1), du1, a0);
             const float e0 = profile<0>(q0), e1 = profile<0>(q1);
             const float tb = t4.x + t4.z * dv - g.tof_t0;
             const f2 ts = pk(tb + t4.y * du0, tb + t4.y * du1);
             f2 Ge = 0, D1 = 0, D2 = 0, nb = 0;      // nb: minus the bin
-            const float *gp = sg + j * bd.st + at;
+            const float *gp = src.row(j);
 #pragma unroll 2
             for (int b = 0; b < g.n_tof; b++, gp += plane) {
                 const f2 x = fma2(nb, TH, ts), x2 = mul2(x, x);
                 nb = add2(nb, MINUS1);
                 float y0, y1;
                 up(mul2(NS, x2), y0, y1);
-                const float2 gg = *reinterpret_cast<const float2 *>(gp);
+                const float2 gg = src.g2(gp, at);
                 const f2 gw = mul2(pk(gg.x, gg.y), pk(ex2_approx(y0), ex2_approx(y1)));
                 Ge = add2(Ge, gw);
                 D1 = fma2(gw, x, D1);
@@ -295,11 +340,9 @@ __device__ __noinline__ void general_box(const DevGeom &g, int view, const float
     r.g0 = __ldg(rec + REC_F4 * (size_t)gid);
     r.g1 = __ldg(rec + REC_F4 * (size_t)gid + 1);
     r.g2 = __ldg(rec + REC_F4 * (size_t)gid + 2);
-    const int w = ihi - ilo + 1;
-    const long long np = (long long)w * (jhi - jlo + 1);
+    const int w = ihi - ilo + 1, di = 32 % w, dj = 32 / w;     // 32 pixels on, row by row
     for (int q = 0; q < NG; q++) val[q] = 0.0f;
-    for (long long p = lane; p < np; p += 32) {
-        const int i = ilo + (int)(p % w), j = jlo + (int)(p / w);
+    for (int i = ilo + lane % w, j = jlo + lane / w; j <= jhi; i += di, j += dj, j += i > ihi, i -= i > ihi ? w : 0) {
         const Ray ray = make_ray<GM_PARALLEL>(g, F, __ldg(g.utab + i), __ldg(g.vtab + j));
         PairGeo q;
         pair_geo(ray, r, q);
@@ -327,12 +370,13 @@ template <bool TOF> struct Shared {
     int4 sbox[2][NW];
     float4 c0[BS], c1[BS], t4[TOF ? BS : 1];
     int2 box[BS];                // the Gaussian's rectangle (packed as k_cull's)
+    uint8_t list[NW][32];        // a warp's Gaussians that meet the band
     float mom[BS * NM];
     float acc[16][BS];
 };
 
 template <int KER, bool TOF, int LG>
-__global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, int64_t n, int gw, int vper,
+__global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, int64_t n, int gw, int vper, int max_px,
                                                    const uint32_t *__restrict__ order,
                                                    const float4 *__restrict__ rec,
                                                    const float4 *__restrict__ crec,
@@ -357,7 +401,8 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
         if (vl + 1 < vb && active) rc_next = __ldg(rect + (int64_t)(vl + 1) * n + gid);
         Box me;
         me.ilo = rc.x & 0xffff; me.ihi = rc.x >> 16; me.jlo = rc.y & 0xffff; me.jhi = rc.y >> 16;
-        const bool vis = active && me.ilo <= me.ihi;
+        const int area = (me.ihi - me.ilo + 1) * (me.jhi - me.jlo + 1);
+        const bool vis = active && me.ilo <= me.ihi && area <= max_px;   // (the others: k_adjoint_direct)
         // the rectangle that holds the CTA's boxes
         {
             int4 b;
@@ -382,9 +427,8 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
         uint32_t bigs;
         int turn;
         {
-            const int area = vis ? (me.ihi - me.ilo + 1) * (me.jhi - me.jlo + 1) : 0;
-            const int mean = (int)(__reduce_add_sync(0xffffffffu, (unsigned)min(area, 1 << 26)) >> 5);
-            const bool big = LG < 5 && area > 64 * S && area > 4 * mean;
+            const int mean = (int)(__reduce_add_sync(0xffffffffu, vis ? (unsigned)min(area, 1 << 26) : 0u) >> 5);
+            const bool big = vis && area > 64 * S && area > 4 * mean;
             bool sat = false;
             if (vis) {
                 float F[9];
@@ -416,15 +460,28 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
             for (int q = 0; q < NM; q++) sh.mom[threadIdx.x * NM + q] = 0.0f;
         }
         const int n_vs = __popc(__ballot_sync(0xffffffffu, vis && !gen));
-        bool first = true;
         Band bd;
+        bd.st = min(BW, (ub.y - ub.x + 2) & ~1);
+        const bool many = ub.y - ub.x >= BW || ub.w - ub.z >= min(BH, Cap<TOF>::v / (bd.st * nb));
         for (bd.cb = ub.x; bd.cb <= ub.y; bd.cb += BW) {
             bd.w = min(BW, ub.y - bd.cb + 1);
             bd.st = (bd.w + 1) & ~1;
             const int hmax = min(BH, Cap<TOF>::v / (bd.st * nb));
             for (bd.rb = ub.z; bd.rb <= ub.w; bd.rb += hmax) {
                 bd.h = min(hmax, ub.w - bd.rb + 1);
-                if (!first) __syncthreads();
+                int now = turn, n_now = n_vs;
+                if (many) {
+                    // several bands: the Gaussians that meet this one, and no
+                    // staging where there is none
+                    const int2 b = sh.box[wb + turn];
+                    const bool on = lane < n_vs && (b.x & 0xffff) < bd.cb + bd.w && (int)((unsigned)b.x >> 16) >= bd.cb &&
+                                    (b.y & 0xffff) < bd.rb + bd.h && (int)((unsigned)b.y >> 16) >= bd.rb;
+                    const uint32_t bal = __ballot_sync(0xffffffffu, on);
+                    if (on) sh.list[w][__popc(bal & ((1u << lane) - 1u))] = (uint8_t)turn;
+                    n_now = __popc(bal);
+                    if (!__syncthreads_or(n_now)) continue;     // (also: every warp is done with the band before)
+                    now = lane < n_now ? sh.list[w][lane] : 0;
+                }
                 // stage dL/dI of the band, a warp taking 1, 2 or 4 rows at a time
                 for (int i = threadIdx.x; i < bd.st; i += BS)
                     sh.su[i] = __ldg(g.utab + min(bd.cb + i, g.n_cols - 1));
@@ -452,7 +509,6 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
                     }
                 }
                 __syncthreads();
-                first = false;
                 // the sub-warps take the warp's Gaussians in turn ...
                 auto take = [&](int k, int l, auto lgc, bool on) {
                     constexpr int L = decltype(lgc)::value;
@@ -463,22 +519,20 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
                     if (!on) { bx.jlo = 1; bx.jhi = 0; bx.ilo = 1; bx.ihi = 0; }
                     const float4 c0 = sh.c0[wb + k], c1 = sh.c1[wb + k];
                     float m[NM];
-                    if (TOF) {
-                        rows_tof(g, c0, c1, sh.t4[wb + k], bx, l, 1 << L, bd, sh.sg, sh.su, sh.sv, m);
-                    } else {
-                        rows<KER>(g, c0, c1, bx, l, 1 << L, bd, sh.sg, sh.su, sh.sv, m);
-                    }
+                    const Staged src = { sh.sg, sh.su, sh.sv, bd };
+                    if constexpr (TOF) rows_tof(g, c0, c1, sh.t4[wb + k], bx, l, 1 << L, src, m);
+                    else rows<KER>(g, c0, c1, bx, l, 1 << L, src, m);
                     __syncwarp();
                     reduce_add<NM, L>(m, l, sh.mom + (wb + k) * NM);
                 };
                 __syncwarp();
                 {
-                    for (int t = 0; t < n_vs; t += 32 / S) {
-                        const int k = __shfl_sync(0xffffffffu, turn, t + sw);
-                        take(k, sl, std::integral_constant<int, LG>{}, !((bigs >> k) & 1u));
+                    for (int t = 0; t < n_now; t += 32 / S) {
+                        const int k = __shfl_sync(0xffffffffu, now, t + sw);
+                        take(k, sl, std::integral_constant<int, LG>{}, t + sw < n_now && !((bigs >> k) & 1u));
                     }
                     // ... and the whole warp the big ones
-                    for (uint32_t bm = LG < 5 ? bigs : 0u; bm; bm &= bm - 1u)
+                    for (uint32_t bm = bigs; bm; bm &= bm - 1u)
                         take(__ffs(bm) - 1, lane, std::integral_constant<int, 5>{}, true);
                 }
             }
@@ -539,6 +593,167 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
             for (int q = 0; q < 4; q++)
                 atomicAdd(gp + q, make_float4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]));
         }
+    }
+}
+
+// The Gaussians whose boxes exceed min_px pixels, dL/dI read in place (no band
+// to stage, nothing shared with the neighbours).  A CTA takes 128 Gaussians of a
+// view and cuts the boxes into strips of whole rows of about strip_px pixels;
+// its warps, and those of the gridDim.z CTAs with the same Gaussians, take the
+// strips in equal shares, 32 at a time: lane k prepares strip k's record and
+// chains its moments, the whole warp walks each, 8 rows by 8 columns at a step (4
+// or 16 rows: 20,000 Gaussians of 150 x 150 px on 8 x 512^2 4.5 and 6.1 ms against
+// 4.2).  Bound by issue for large footprints and by latency for few.  Against
+// the staged walk, and (last) one Gaussian per thread and tile: 64 of 10^5 px on
+// one view 8.1, 0.16, 0.18 ms; 8 of 960 px 0.12, 0.015, 0.014; 1,000 of 23,000
+// px on 8 views 0.82, 0.23, 0.26.
+template <int KER, bool TOF>
+__global__ void __launch_bounds__(BS, TOF ? 3 : 6) k_adjoint_direct(DevGeom g, int nv, int64_t n, int min_px, int strip_px,
+                                                                    const float4 *__restrict__ rec,
+                                                                    const float4 *__restrict__ crec,
+                                                                    const uint2 *__restrict__ rect,
+                                                                    const float *__restrict__ dLdI,
+                                                                    float4 *__restrict__ grad)
+{
+    constexpr int NM = TOF ? 11 : 7, ROWS = 32 >> DIRECT_LG;
+    __shared__ uint32_t ids[BS], first[BS];      // the view's Gaussians, and the first of their strips
+    __shared__ uint2 box[BS], wsum[NW];
+    __shared__ float4 sc0[BS], sc1[BS], st4[TOF ? BS : 1];
+    __shared__ uint2 strip[BS];
+    __shared__ float mom[BS * NM];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, wb = 32 * w;
+    const int64_t k = (int64_t)blockIdx.x * BS + threadIdx.x;
+    // rows of a strip
+    auto rows_of = [&](int wd) { return (max(strip_px / wd, 1) + ROWS - 1) / ROWS * ROWS; };
+    for (int vl = blockIdx.y; vl < nv; vl += gridDim.y) {
+        const uint2 rc = k < n ? __ldg(rect + (int64_t)vl * n + k) : make_uint2(1u, 1u);
+        const int bw = (int)(rc.x >> 16) - (int)(rc.x & 0xffff) + 1, bh = (int)(rc.y >> 16) - (int)(rc.y & 0xffff) + 1;
+        const bool on = bw > 0 && bw * bh > min_px;
+        if (!__syncthreads_or(on)) continue;
+        const uint32_t mine = on ? (uint32_t)((bh - 1) / rows_of(bw) + 1) : 0u;
+        uint32_t inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const uint32_t bal = __ballot_sync(0xffffffffu, on);
+        if (lane == 31) wsum[w] = make_uint2(__popc(bal), inc);
+        __syncthreads();
+        uint32_t at = __popc(bal & ((1u << lane) - 1u)), num = 0, strips = 0;
+        inc -= mine;
+#pragma unroll
+        for (int q = 0; q < NW; q++) {
+            if (q < w) {
+                at += wsum[q].x;
+                inc += wsum[q].y;
+            }
+            num += wsum[q].x;
+            strips += wsum[q].y;
+        }
+        if (on) {
+            ids[at] = (uint32_t)k;
+            box[at] = rc;
+            first[at] = inc;
+        }
+        __syncthreads();
+        const int view = g.v0 + vl;
+        const float *I = dLdI + (long long)view * g.stride_view;
+        float F[9];
+#pragma unroll
+        for (int q = 0; q < 9; q++) F[q] = __ldg(g.frames + 9 * (size_t)view + q);
+        const uint32_t share = blockIdx.z * NW + w, shares = gridDim.z * NW;
+        const uint32_t sa = (uint32_t)((uint64_t)strips * share / shares), sb = (uint32_t)((uint64_t)strips * (share + 1) / shares);
+        for (uint32_t s0 = sa; s0 < sb; s0 += 32) {
+            // lane k: strip s0 + k
+            const uint32_t st = s0 + lane;
+            const bool vis = st < sb;
+            uint32_t gid = 0;
+            Box bx = { 1, 0, 1, 0 };
+            bool gen = false;
+            if (vis) {
+                uint32_t e = 0;
+                for (uint32_t hi = num - 1; e < hi;) {
+                    const uint32_t mid = (e + hi + 1) >> 1;
+                    if (first[mid] <= st) e = mid; else hi = mid - 1;
+                }
+                gid = ids[e];
+                const uint2 b = box[e];
+                bx.ilo = b.x & 0xffff; bx.ihi = b.x >> 16; bx.jlo = b.y & 0xffff; bx.jhi = b.y >> 16;
+                const int per = rows_of(bx.ihi - bx.ilo + 1);
+                bx.jlo += (int)(st - first[e]) * per;
+                bx.jhi = min(bx.jhi, bx.jlo + per - 1);
+                VRec r;
+                prep_record<GM_PARALLEL, KER>(g, F, gid, rec, crec, r);
+                gen = r.g2.w == 0.0f;
+                sc0[threadIdx.x] = r.c0;
+                sc1[threadIdx.x] = r.c1;
+                if (TOF) st4[threadIdx.x] = r.t4;
+            }
+            strip[threadIdx.x] = make_uint2((uint32_t)bx.ilo | ((uint32_t)bx.ihi << 16),
+                                            (uint32_t)bx.jlo | ((uint32_t)bx.jhi << 16));
+#pragma unroll
+            for (int q = 0; q < NM; q++) mom[threadIdx.x * NM + q] = 0.0f;
+            __syncwarp();
+            for (uint32_t m32 = __ballot_sync(0xffffffffu, vis && !gen); m32; m32 &= m32 - 1u) {
+                const int t = wb + __ffs(m32) - 1;
+                const uint2 b = strip[t];
+                Box s;
+                s.ilo = b.x & 0xffff; s.ihi = b.x >> 16; s.jlo = b.y & 0xffff; s.jhi = b.y >> 16;
+                const Direct src = { g, I, lane & ((1 << DIRECT_LG) - 1) };
+                float v[NM];
+                if constexpr (TOF) rows_tof(g, sc0[t], sc1[t], st4[t], s, lane >> DIRECT_LG, ROWS, src, v);
+                else rows<KER>(g, sc0[t], sc1[t], s, lane >> DIRECT_LG, ROWS, src, v);
+                __syncwarp();
+                reduce_add<NM, 5>(v, lane, mom + t * NM);
+            }
+            __syncwarp();
+            float o[16];
+            bool any = false;
+#pragma unroll
+            for (int q = 0; q < 16; q++) o[q] = 0.0f;
+            if (vis && !gen) {
+                float m[NM], sm[12], tof4[4];
+#pragma unroll
+                for (int q = 0; q < NM; q++) {
+                    m[q] = mom[threadIdx.x * NM + q];
+                    any |= m[q] != 0.0f;
+                }
+                const float4 c1 = sc1[threadIdx.x];
+                if (any) {
+                    finish<KER>(m, c1.y, c1.z, sm);
+                    if (TOF) {
+#pragma unroll
+                        for (int q = 0; q < 4; q++) tof4[q] = c1.z * m[TOF ? 7 + q : 0];
+                    }
+                    view_chain<GM_PARALLEL, KER>(g, F, rec, gid, sm, o, TOF ? tof4 : nullptr);
+                }
+            }
+            // Gaussians near a segment end
+            for (uint32_t gm = __ballot_sync(0xffffffffu, vis && gen); gm; gm &= gm - 1u) {
+                const int owner = __ffs(gm) - 1;
+                const uint2 b = strip[wb + owner];
+                float val[NG];
+                general_box<KER, TOF>(g, view, rec, __shfl_sync(0xffffffffu, gid, owner), b.x & 0xffff, b.x >> 16,
+                                      b.y & 0xffff, b.y >> 16, dLdI, val);
+                if (lane == owner) {
+                    const int slot_of[NG] = { 0, 1, 2, 4, 5, 6, 7, 8, 9, 3 };
+#pragma unroll
+                    for (int q = 0; q < NG; q++) {
+                        o[slot_of[q]] = val[q];
+                        any |= val[q] != 0.0f;
+                    }
+                }
+            }
+            if (any) {
+                float4 *gp = grad + GRAD_F4 * (size_t)gid;
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    atomicAdd(gp + q, make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]));
+            }
+            __syncwarp();   // the strips' records are done with
+        }
+        __syncthreads();   // the list is done before another view's
     }
 }
 
@@ -763,13 +978,21 @@ cudaError_t launch_order(const float4 *crec, int64_t n, void *tmp, uint32_t *ord
 
 namespace {
 
-template <int KER, bool TOF>
-void adjoint_lg(int lg, const DevGeom &g, int nv, int64_t n, const uint32_t *order, const float4 *rec,
-                const float4 *crec, const uint2 *rect, const float *dLdI, float4 *grad, cudaStream_t s)
+// average footprint of a launch in pixels, from its tile entries per (view,
+// Gaussian): a w x w box lands on about (1 + w / tile)^2 tiles
+double footprint_px(const DevGeom &g, int nv, int64_t n, int64_t entries)
 {
-    // Gaussians per warp: fewer where 32 would leave the GPU short of CTAs (10
-    // per SM; 1,000 Gaussians on 16 x 64^2 pixels: 0.117 ms at 8 and 5 CTAs per
-    // SM, 0.088 at 2)
+    const double per = (double)entries / ((double)nv * (double)n);
+    const double side = per > 1.0 ? sqrt(per) - 1.0 : 0.0;
+    return side * side * g.tile_w * g.tile_h;
+}
+
+template <int KER, bool TOF>
+void adjoint_staged_launch(double px, int max_px, const DevGeom &g, int nv, int64_t n, const uint32_t *order,
+                           const float4 *rec, const float4 *crec, const uint2 *rect, const float *dLdI, float4 *grad,
+                           cudaStream_t s)
+{
+    // Gaussians per warp: fewer where 32 would leave the GPU short of CTAs
     int gw = 32;
     while (gw > 2 && (n / (gw * NW)) * nv < 152 * 10) gw >>= 1;
     const int64_t bx = (n + NW * gw - 1) / (NW * gw);
@@ -778,36 +1001,77 @@ void adjoint_lg(int lg, const DevGeom &g, int nv, int64_t n, const uint32_t *ord
     if (chunks > 65535) chunks = 65535;
     const int vper = (int)((nv + chunks - 1) / chunks);
     const dim3 grid((unsigned)bx, (unsigned)((nv + vper - 1) / vper));
-#define RGRT_ADJ(L) k_adjoint<KER, TOF, L><<<grid, BS, 0, s>>>(g, nv, n, gw, vper, order, rec, crec, rect, dLdI, grad)
-    if (lg <= 1) RGRT_ADJ(1);
-    else if (lg == 2) RGRT_ADJ(2);
-    else if (lg == 3) RGRT_ADJ(3);
-    else RGRT_ADJ(4);
+    // lanes per Gaussian: measured 2 / 4 / 8 lanes at 36 px (PET ring) 6.9 / 7.2 /
+    // 8.4 ms, at 65 px (raw PET) 0.143 / 0.143 / 0.163, at 180 px (20,000 on 90 x
+    // 256^2) 4 / 8 lanes 0.706 / 0.744, at 5,900 px 10.9 / 10.65
+    const int lg = px > 80.0 ? 2 : 1;
+#define RGRT_ADJ(L) k_adjoint<KER, TOF, L><<<grid, BS, 0, s>>>(g, nv, n, gw, vper, max_px, order, rec, crec, rect, dLdI, grad)
+    if (lg == 1) RGRT_ADJ(1);
+    else RGRT_ADJ(2);
 #undef RGRT_ADJ
+    count_launches(1);
+}
+
+template <int KER, bool TOF>
+void adjoint_direct_launch(double px, int min_px, const DevGeom &g, int nv, int64_t n, const float4 *rec,
+                           const float4 *crec, const uint2 *rect, const float *dLdI, float4 *grad, cudaStream_t s)
+{
+    // CTAs for a few waves, each looking through the boxes of several views; where
+    // the Gaussians are too few for that, several share a set's strips
+    const int64_t bx = (n + BS - 1) / BS;
+    int64_t by = (152 * 48 + bx - 1) / bx;
+    if (by > nv) by = nv;
+    if (by > 65535) by = 65535;
+    // strips for about 64 warps per SM
+    const double pairs = (double)n * (double)nv, strip = px * pairs / (152 * 64.0);
+    const int strip_px = strip < 256.0 ? 256 : strip > 4096.0 ? 4096 : (int)strip;
+    const double most = pairs * (1.0 + px / strip_px) / (double)(bx * by * NW * 4);   // four strips a warp
+    int64_t z = 152 * 40 / (bx * by);
+    if (z > (int64_t)most) z = (int64_t)most;
+    z = z < 1 ? 1 : z;
+    const dim3 grid((unsigned)bx, (unsigned)by, (unsigned)z);
+    k_adjoint_direct<KER, TOF><<<grid, BS, 0, s>>>(g, nv, n, min_px, strip_px, rec, crec, rect, dLdI, grad);
+    count_launches(1);
 }
 
 }  // namespace
 
-cudaError_t launch_adjoint(const DevGeom &g, int nv, int64_t n, int64_t entries, const uint32_t *order,
+// k_adjoint needs enough (view, Gaussian) pairs that neighbours share bands and
+// the CTAs that hold far-apart Gaussians are a small part; below that every pair
+// goes to k_adjoint_direct, whose cost is its own pixels.  Measured staged /
+// direct: 64 Gaussians on one view of 512^2 0.15 / 0.01 ms, 16,000 pairs of 470
+// px 0.088 / 0.068, 90,000 of 180 px 0.16 / 0.095, 160,000 of 960 px 0.38 / 0.29;
+// 200,000 of 75 px 2.5 / 3.7 (a batch's step), 800,000 of 65 px 0.14 / 0.73.
+bool adjoint_staged(const DevGeom &g, int nv, int64_t n, int64_t entries)
+{
+    const int64_t pairs = n * nv;
+    return pairs > 262144 || (pairs > 32768 && footprint_px(g, nv, n, entries) <= 200.0);
+}
+
+cudaError_t launch_adjoint(const DevGeom &g, int nv, int64_t n, int64_t entries, bool large, const uint32_t *order,
                            const float4 *rec, const float4 *crec, const uint2 *rect, const float *dLdI,
                            float4 *grad, int ker, cudaStream_t s)
 {
     if (nv <= 0 || n <= 0) return cudaSuccess;
-    // average footprint in pixels, from the tile entries per (view, Gaussian):
-    // a w x w box lands on about (1 + w / tile)^2 tiles
-    const double per = (double)entries / ((double)nv * (double)n);
-    const double side = per > 1.0 ? sqrt(per) - 1.0 : 0.0;
-    const double px = side * side * g.tile_w * g.tile_h;
-    // lanes per Gaussian: measured 2 / 4 / 8 lanes at 36 px (PET ring) 6.9 / 7.2 /
-    // 8.4 ms, at 65 px (raw PET) 0.143 / 0.143 / 0.163, at 470 px (parallel beam)
-    // 0.17 / 0.11 / 0.12; beyond that a lane would walk more rows than the
-    // warps in flight can hide
-    const int lg = px > 20000.0 ? 4 : px > 4000.0 ? 3 : px > 80.0 ? 2 : 1;
+    const double px = footprint_px(g, nv, n, entries);
+    const bool staged = adjoint_staged(g, nv, n, entries);
+    // Footprints beyond max_px are walked in place: staged, each would take band
+    // after band of its CTA's union.  2,048 px: 50,000 Gaussians of 50 px and 100
+    // of 10^4 px on 90 x 256^2 11.5 -> 4.4 ms, log-sizes with a deviation of 1.0
+    // 4.9 -> 3.0 (1,024 px 2.9, 4,096 3.0), a PET ring with 0.7 15.3 -> 14.5;
+    // where the average is itself larger, four times that (20,000 of 5,900 px:
+    // 12.8 ms at 2,048 px, 10.6 at 8,192).
+    const int max_px = !staged ? 0 : px > ADJOINT_LARGE_PX ? 4 * ADJOINT_LARGE_PX : ADJOINT_LARGE_PX;
+#define RGRT_ADJ(K, T)                                                                                          \
+    {                                                                                                           \
+        if (staged) adjoint_staged_launch<K, T>(px, max_px, g, nv, n, order, rec, crec, rect, dLdI, grad, s);   \
+        if (!staged || large) adjoint_direct_launch<K, T>(px, max_px, g, nv, n, rec, crec, rect, dLdI, grad, s); \
+    }
     // time of flight: PET ring, Gaussian kernel (checked by the caller)
-    if (g.n_tof > 0) adjoint_lg<0, true>(lg, g, nv, n, order, rec, crec, rect, dLdI, grad, s);
-    else if (ker == 1) adjoint_lg<1, false>(lg, g, nv, n, order, rec, crec, rect, dLdI, grad, s);
-    else adjoint_lg<0, false>(lg, g, nv, n, order, rec, crec, rect, dLdI, grad, s);
-    count_launches(1);
+    if (g.n_tof > 0) RGRT_ADJ(0, true)
+    else if (ker == 1) RGRT_ADJ(1, false)
+    else RGRT_ADJ(0, false)
+#undef RGRT_ADJ
     return cudaGetLastError();
 }
 

@@ -182,8 +182,9 @@ void prof_harvest(rgrt_ctx *c)
 
 // ---- pipeline pieces ------------------------------------------------------
 
-// records of the current parameters; total[1] collects the non-finite flag,
-// which the next host read-back of the binning totals checks
+// records of the current parameters; total[1] collects two flags for the next
+// host read-back of the binning totals: non-finite parameters (low word) and
+// boxes of more than ADJOINT_LARGE_PX pixels (high word, k_cull)
 int build_records(rgrt_ctx *ctx, const rgrt_gauss *g, cudaStream_t s)
 {
     if (g->n == 0) return RGRT_OK;
@@ -195,14 +196,15 @@ int build_records(rgrt_ctx *ctx, const rgrt_gauss *g, cudaStream_t s)
     return RGRT_OK;
 }
 
-// the binning totals (K) and the non-finite flag, read back together
-int read_totals(rgrt_ctx *ctx, cudaStream_t s, unsigned long long *K)
+// the binning totals (K) and the flags, read back together
+int read_totals(rgrt_ctx *ctx, cudaStream_t s, unsigned long long *K, bool *large = nullptr)
 {
     CK(cudaMemcpyAsync(ctx->h_total, ctx->total.p, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
-    if (ctx->h_total[1])
+    if ((uint32_t)ctx->h_total[1])
         return fail(RGRT_E_INVAL, "non-finite Gaussian parameters (mu, log-scale, quaternion or rho)");
     if (K) *K = ctx->h_total[0];
+    if (large) *large = (ctx->h_total[1] >> 32) != 0;
     return RGRT_OK;
 }
 
@@ -234,7 +236,8 @@ int bin_views(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, int v0,
     TRY(ensure(ctx, ctx->ranges, sizeof(uint2) * (size_t)T));
     {
         PROF("k_cull");
-        CK(launch_cull(dg, nv, g->crec, N, (uint32_t *)ctx->cnt.p, (uint2 *)ctx->rect.p, s));
+        CK(launch_cull(dg, nv, g->crec, N, (uint32_t *)ctx->cnt.p, (uint2 *)ctx->rect.p, s,
+                       (uint32_t *)ctx->total.p + 3));
     }
     {
         PROF("scan");
@@ -242,7 +245,7 @@ int bin_views(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, int v0,
                        (unsigned long long *)ctx->total.p, (unsigned long long *)ctx->scan_tmp.p, s));
     }
     unsigned long long K = 0;
-    TRY(read_totals(ctx, s, &K));
+    TRY(read_totals(ctx, s, &K, &ctx->bin_large));
     if (K >= 0xffffffffull)
         return fail(RGRT_E_CAPACITY, "views %d..%d produce %llu tile entries (more than 2^32)", v0,
                     v0 + nv, K);
@@ -502,10 +505,9 @@ int run_forward(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, float
     });
 }
 
-// the Gaussians' spatial order, for the adjoint
-int build_order(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, cudaStream_t s)
+// the Gaussians' spatial order, for the adjoint of parallel rays
+int build_order(rgrt_ctx *ctx, const rgrt_gauss *g, cudaStream_t s)
 {
-    if (geom->dg.kind != GM_PARALLEL) return RGRT_OK;   // adjoint tile by tile
     TRY(ensure(ctx, ctx->order, sizeof(uint32_t) * (size_t)g->n));
     TRY(ensure(ctx, ctx->order_tmp, order_tmp_bytes(g->n)));
     PROF("k_order");
@@ -519,12 +521,14 @@ int adjoint_views(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, int
 {
     DevGeom dg = geom->dg;
     dg.v0 = v0;
+    if (dg.kind == GM_PARALLEL && adjoint_staged(dg, nv, g->n, K)) TRY(build_order(ctx, g, s));
     PROF("k_adjoint");
     if (dg.kind != GM_PARALLEL)
         CK(launch_adjoint_tiles(dg, nv, K, g->rec, g->crec, (const uint32_t *)ctx->vals.p, (const uint2 *)ctx->ranges.p,
                                 dLdI, (float4 *)ctx->grad.p, g->kernel, s));
-    else CK(launch_adjoint(dg, nv, g->n, K, (const uint32_t *)ctx->order.p, g->rec, g->crec, (const uint2 *)ctx->rect.p,
-                      dLdI, (float4 *)ctx->grad.p, g->kernel, s));
+    else
+        CK(launch_adjoint(dg, nv, g->n, K, ctx->bin_large, (const uint32_t *)ctx->order.p, g->rec, g->crec,
+                          (const uint2 *)ctx->rect.p, dLdI, (float4 *)ctx->grad.p, g->kernel, s));
     return RGRT_OK;
 }
 
@@ -556,7 +560,6 @@ int run_backward(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, cons
     }
     if (geom->dg.n_tof && g->kernel != RGRT_KERNEL_GAUSSIAN)
         return fail(RGRT_E_INVAL, "time of flight takes the Gaussian kernel");
-    TRY(build_order(ctx, g, geom, s));
     TRY(for_chunks(ctx, g, geom, s, reuse, [&](int v0, int nv, uint32_t K) -> int {
         return adjoint_views(ctx, g, geom, v0, nv, K, dLdI, s);
     }));
@@ -1131,7 +1134,6 @@ static int run_loss_grad(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *ge
         const int64_t HW = (int64_t)geom->dg.n_rows * geom->dg.n_cols;
         float *I = (float *)ctx->I.p, *dLdI = (float *)ctx->dLdI.p;
         const float *y = (const float *)dy;
-        TRY(build_order(ctx, g, geom, s));
         TRY(for_chunks(ctx, g, geom, s, false, [&](int v0, int nv, uint32_t K) -> int {
             DevGeom dg = geom->dg;
             dg.v0 = v0;

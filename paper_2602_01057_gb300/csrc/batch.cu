@@ -416,8 +416,9 @@ int enqueue_adjoint(rgrt_batch *b, int i, cudaStream_t s)
                                 RGRT_KERNEL_GAUSSIAN, s));
         return RGRT_OK;
     }
-    BK(launch_order(x.g->crec, x.N, b->lane[x.lane].order_tmp, x.order, s));
-    BK(launch_adjoint(dg, dg.n_views, x.N, x.keys, x.order, x.g->rec, x.g->crec, x.rect, x.dLdI, x.grad,
+    if (adjoint_staged(dg, dg.n_views, x.N, x.keys))
+        BK(launch_order(x.g->crec, x.N, b->lane[x.lane].order_tmp, x.order, s));
+    BK(launch_adjoint(dg, dg.n_views, x.N, x.keys, true, x.order, x.g->rec, x.g->crec, x.rect, x.dLdI, x.grad,
                       RGRT_KERNEL_GAUSSIAN, s));
     return RGRT_OK;
 }

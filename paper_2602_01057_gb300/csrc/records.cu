@@ -241,7 +241,7 @@ __device__ __forceinline__ void cull_write(const DevGeom &g, int i0, int i1, int
 // turn (they share the frame and the columns)
 template <int GM>
 __global__ void k_cull(DevGeom g, int nv, const float4 *__restrict__ crec, int64_t n,
-                       uint32_t *__restrict__ cnt, uint2 *__restrict__ rect)
+                       uint32_t *__restrict__ cnt, uint2 *__restrict__ rect, uint32_t *large)
 {
     constexpr bool CONE = GM == GM_CONE, P3 = GM == GM_PET3D;
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -273,6 +273,9 @@ __global__ void k_cull(DevGeom g, int nv, const float4 *__restrict__ crec, int64
             const int j0 = lower_idx_g(g.vtab, g.n_rows, vlo, g.v0f, g.vinv);
             const int j1 = upper_idx_g(g.vtab, g.n_rows, vhi, g.v0f, g.vinv);
             cull_write(g, i0, i1, j0, j1, cnt + (int64_t)vf * n + k, rect + (int64_t)vf * n + k);
+            if (GM == GM_PARALLEL && large && i0 <= i1 && j0 <= j1 &&
+                (int64_t)(i1 - i0 + 1) * (j1 - j0 + 1) > ADJOINT_LARGE_PX)
+                *large = 1u;
             continue;
         }
         // 3-D PET: the LOR of radial position s and mid-height z has
@@ -333,14 +336,14 @@ cudaError_t launch_records(const float *mu, const float *ls, const float *q, con
 }
 
 cudaError_t launch_cull(const DevGeom &g, int nv, const float4 *crec, int64_t n, uint32_t *cnt,
-                        uint2 *rect, cudaStream_t s)
+                        uint2 *rect, cudaStream_t s, uint32_t *large)
 {
     if (nv <= 0 || n <= 0) return cudaSuccess;
     const int nf = g.kind == GM_PET3D && nv > g.n_ang ? g.n_ang : nv;
     const dim3 grid((unsigned)((n + 255) / 256), (unsigned)(nf < 65535 ? nf : 65535));
-    if (g.kind == GM_CONE) k_cull<GM_CONE><<<grid, 256, 0, s>>>(g, nv, crec, n, cnt, rect);
-    else if (g.kind == GM_PET3D) k_cull<GM_PET3D><<<grid, 256, 0, s>>>(g, nv, crec, n, cnt, rect);
-    else k_cull<GM_PARALLEL><<<grid, 256, 0, s>>>(g, nv, crec, n, cnt, rect);
+    if (g.kind == GM_CONE) k_cull<GM_CONE><<<grid, 256, 0, s>>>(g, nv, crec, n, cnt, rect, nullptr);
+    else if (g.kind == GM_PET3D) k_cull<GM_PET3D><<<grid, 256, 0, s>>>(g, nv, crec, n, cnt, rect, nullptr);
+    else k_cull<GM_PARALLEL><<<grid, 256, 0, s>>>(g, nv, crec, n, cnt, rect, large);
     count_launches(1);
     return cudaGetLastError();
 }

@@ -98,8 +98,10 @@ int report_error(int code, const char *msg);
 // bad (nullable): set to nonzero when a parameter is not finite
 cudaError_t launch_records(const float *mu, const float *ls, const float *q, const float *rho,
                            int64_t n, float4 *rec, float4 *crec, uint32_t *bad, cudaStream_t s);
+// large (nullable; parallel rays): set to nonzero when a box exceeds
+// ADJOINT_LARGE_PX pixels
 cudaError_t launch_cull(const DevGeom &g, int nv, const float4 *crec, int64_t n, uint32_t *cnt,
-                        uint2 *rect, cudaStream_t s);
+                        uint2 *rect, cudaStream_t s, uint32_t *large = nullptr);
 // key = tile field << 8 | position code; lbits >= 0: the tile field is
 // (view << lbits) | tile within the view, for launch_sort_views; lbits < 0:
 // the tile id view * tiles per view + tile
@@ -158,8 +160,12 @@ cudaError_t launch_forward(const DevGeom &g, int nv, int64_t entries, const floa
 size_t order_tmp_bytes(int64_t n);
 cudaError_t launch_order(const float4 *crec, int64_t n, void *tmp, uint32_t *order, cudaStream_t s);
 // adjoint of parallel-ray views v0 .. v0 + nv - 1: rect = k_cull's pixel boxes
-// of those views, entries = their (tile, Gaussian) entries (the footprints' size)
-cudaError_t launch_adjoint(const DevGeom &g, int nv, int64_t n, int64_t entries, const uint32_t *order,
+// of those views, entries = their (tile, Gaussian) entries (the footprints' size),
+// large = some box may exceed ADJOINT_LARGE_PX pixels.  adjoint_staged: the
+// launch reads the order.
+constexpr int ADJOINT_LARGE_PX = 2048;
+bool adjoint_staged(const DevGeom &g, int nv, int64_t n, int64_t entries);
+cudaError_t launch_adjoint(const DevGeom &g, int nv, int64_t n, int64_t entries, bool large, const uint32_t *order,
                            const float4 *rec, const float4 *crec, const uint2 *rect, const float *dLdI,
                            float4 *grad, int ker, cudaStream_t s);
 // the same for cone-beam and 3-D PET views, from the tile lists

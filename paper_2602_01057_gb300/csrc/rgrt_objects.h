@@ -38,6 +38,7 @@ struct rgrt_ctx {
     unsigned long long bin_version = 0;
     int bin_v0 = -1, bin_nv = 0;
     uint32_t bin_keys = 0;
+    bool bin_large = false;    // some box may exceed ADJOINT_LARGE_PX pixels (parallel rays)
     bool bin_valid = false;
     // profiling
     bool prof = false;

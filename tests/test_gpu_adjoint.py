@@ -119,3 +119,100 @@ def test_non_finite_weight_outside_the_cut_adds_nothing(env, name, bad):
         rg.project_backward(ctx, gs, geom, torch.where(empty, torch.full_like(w, fill), w), *outs)
         res.append(torch.cat([o.reshape(-1) for o in outs]).double().cpu())
     assert torch.linalg.norm(res[1] - res[0]) <= 1e-5 * torch.linalg.norm(res[0])
+
+
+def _sizes(n, seed, ls, box=0.9, large=()):
+    """n Gaussians, the first of them of other log-sizes: (count, log-size), ..."""
+    G = synth.gaussians_uniform(n, seed, half_box=box, log_sigma=ls)
+    at = 0
+    for count, x in large:
+        G["ls"][at:at + count] = x
+        at += count
+    p = np.random.default_rng(seed).permutation(n)
+    return {k: v[p] for k, v in G.items()}
+
+
+def _ring(V, W, H, bins=0, arc_mode=0):
+    gd = synth.geom_pet(V, W, H, 400.0, 576, 9.0, arc_mode=arc_mode)
+    return synth.with_tof_bins(gd, bins, 40.0, 30.0) if bins else gd
+
+
+L = math.log
+# sets large enough to be staged; in parts of 8,000 (view, Gaussian) pairs they are not
+STAGED = {
+    "rows_banded": lambda: (_sizes(40_000, 51, L(0.01)), _parallel(1, 300, 130, 0.008)),
+    "columns_banded": lambda: (_sizes(40_000, 52, L(0.01)), _parallel(1, 9, 700, 0.004)),
+    "one_column": lambda: (_sizes(40_000, 53, L(0.01)), _parallel(1, 300, 1, 0.008)),
+    "views": lambda: (_sizes(12_000, 54, L(0.02)), _parallel(4, 61, 47, 0.03)),
+    "outliers": lambda: (_sizes(40_000, 55, L(0.01), large=((20, L(0.08)), (5, L(0.3)))), _parallel(1, 200, 211, 0.01)),
+    "ends": lambda: (_sizes(40_000, 56, L(0.01), large=((20, L(0.08)), (5, L(0.3)))),
+                     synth.geom_parallel(1, 200, 211, 0.01, 0.01, -0.3, 0.2)),
+    "ring": lambda: (_sizes(20_000, 57, L(4.0), 120.0, ((9, L(30.0)),)), _ring(2, 281, 21)),
+    "ring_raw": lambda: (_sizes(20_000, 58, L(4.0), 120.0, ((9, L(30.0)),)), _ring(2, 281, 21, arc_mode=1)),
+    "ring_5_bins": lambda: (_sizes(20_000, 59, L(4.0), 120.0, ((9, L(30.0)),)), _ring(2, 281, 21, 5)),
+    "ring_16_bins": lambda: (_sizes(20_000, 60, L(4.0), 120.0, ((9, L(60.0)),)), _ring(2, 281, 21, 16)),
+}
+
+
+@pytest.mark.parametrize("kernel", ["gaussian", "epanechnikov"])
+@pytest.mark.parametrize("name", list(STAGED))
+def test_staged_and_direct_walks_agree(env, name, kernel):
+    """A Gaussian's gradient takes nothing from the others, so a set's equals its
+    parts' -- the set staged (with its large footprints in place), the small
+    parts all in place.  Both decide every pair by the same roundings, only the
+    sums' order differs: within 2e-6 of the norm (a few ulp of the terms)."""
+    torch, rg, ctx = env
+    G, gd = STAGED[name]()
+    if kernel == "epanechnikov" and gd.get("n_tof"):
+        pytest.skip("time of flight takes the Gaussian kernel")
+    geom = rg.Geometry(ctx, gd)
+    w = torch.from_numpy(synth.random_weights(geom.n_rays, 7)).cuda()
+
+    def grads(G):
+        gs = rg.Gaussians(ctx, *[torch.from_numpy(np.ascontiguousarray(G[k])).cuda() for k in ("mu", "ls", "q", "rho")])
+        gs.set_kernel(kernel)
+        outs = [torch.empty(s, device="cuda") for s in ((gs.n, 3), (gs.n, 3), (gs.n, 4), (gs.n, 1))]
+        ctx.prof_reset()
+        ctx.prof_enable(True)
+        rg.project_backward(ctx, gs, geom, w, *outs)
+        staged = ctx.prof_get("k_order")[0] > 0
+        ctx.prof_enable(False)
+        return [o.double() for o in outs], staged
+
+    whole, staged = grads(G)
+    assert staged
+    n, step = G["rho"].size, 8000 // int(gd["n_views"])
+    parts = []
+    for a in range(0, n, step):
+        part, staged = grads({k: v[a:a + step] for k, v in G.items()})
+        assert not staged
+        parts.append(part)
+    for key, a, b in zip(("mu", "ls", "q", "rho"), whole, [torch.cat(x) for x in zip(*parts)]):
+        e = float(torch.linalg.norm(a - b) / torch.linalg.norm(b))
+        assert e < 2e-6, f"{key}: {e:.2e}"
+
+
+def test_few_large_footprints_are_shared_out(env):
+    """64 Gaussians over most of a 512 x 512 view (their boxes, walked by one warp
+    each, took 50 times the forward): the gradient takes no more than five
+    forward projections, best of five each."""
+    torch, rg, ctx = env
+    geom = rg.Geometry(ctx, _parallel(1, 512, 512, 2.0 / 512))
+    G = synth.gaussians_uniform(64, 61, half_box=0.7, log_sigma=math.log(0.2))
+    gs = rg.Gaussians(ctx, *[torch.from_numpy(np.ascontiguousarray(G[k])).cuda() for k in ("mu", "ls", "q", "rho")])
+    img, w = torch.empty(geom.n_rays, device="cuda"), torch.rand(geom.n_rays, device="cuda")
+    outs = [torch.empty(s, device="cuda") for s in ((64, 3), (64, 3), (64, 4), (64,))]
+
+    def best(call):
+        ms = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            call()
+            b.record()
+            torch.cuda.synchronize()
+            ms.append(a.elapsed_time(b))
+        return min(ms[2:])
+
+    fwd = best(lambda: rg.project_forward(ctx, gs, geom, img))
+    assert best(lambda: rg.project_backward(ctx, gs, geom, w, *outs)) < 5.0 * fwd
