@@ -81,6 +81,12 @@ struct Box {
     int ilo, ihi, jlo, jhi;
 };
 
+// pixels of a box, at most 2^26 (a detector of 65,536 x 65,536 has 2^32)
+__device__ __forceinline__ int box_px(int w, int h)
+{
+    return (int)min((long long)w * h, 1ll << 26);
+}
+
 // a staged band: columns [cb, cb + w), rows [rb, rb + h), row stride st
 struct Band {
     int cb, rb, w, h, st;
@@ -401,7 +407,7 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
         if (vl + 1 < vb && active) rc_next = __ldg(rect + (int64_t)(vl + 1) * n + gid);
         Box me;
         me.ilo = rc.x & 0xffff; me.ihi = rc.x >> 16; me.jlo = rc.y & 0xffff; me.jhi = rc.y >> 16;
-        const int area = (me.ihi - me.ilo + 1) * (me.jhi - me.jlo + 1);
+        const int area = box_px(me.ihi - me.ilo + 1, me.jhi - me.jlo + 1);
         const bool vis = active && me.ilo <= me.ihi && area <= max_px;   // (the others: k_adjoint_direct)
         // the rectangle that holds the CTA's boxes
         {
@@ -427,7 +433,7 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
         uint32_t bigs;
         int turn;
         {
-            const int mean = (int)(__reduce_add_sync(0xffffffffu, vis ? (unsigned)min(area, 1 << 26) : 0u) >> 5);
+            const int mean = (int)(__reduce_add_sync(0xffffffffu, vis ? (unsigned)area : 0u) >> 5);
             const bool big = vis && area > 64 * S && area > 4 * mean;
             bool sat = false;
             if (vis) {
@@ -445,7 +451,7 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
             bigs = __ballot_sync(0xffffffffu, big && sat);
             // the warp's Gaussians by the size of their boxes, largest first:
             // sub-warps walk side by side, so those of a round should be alike
-            uint32_t key = ((vis && sat ? (uint32_t)min(area, 1 << 26) : 0u) << 5) | (uint32_t)lane;
+            uint32_t key = ((vis && sat ? (uint32_t)area : 0u) << 5) | (uint32_t)lane;
 #pragma unroll
             for (int k = 2; k <= 32; k <<= 1)
 #pragma unroll
@@ -628,7 +634,7 @@ __global__ void __launch_bounds__(BS, TOF ? 3 : 6) k_adjoint_direct(DevGeom g, i
     for (int vl = blockIdx.y; vl < nv; vl += gridDim.y) {
         const uint2 rc = k < n ? __ldg(rect + (int64_t)vl * n + k) : make_uint2(1u, 1u);
         const int bw = (int)(rc.x >> 16) - (int)(rc.x & 0xffff) + 1, bh = (int)(rc.y >> 16) - (int)(rc.y & 0xffff) + 1;
-        const bool on = bw > 0 && bw * bh > min_px;
+        const bool on = bw > 0 && box_px(bw, bh) > min_px;
         if (!__syncthreads_or(on)) continue;
         const uint32_t mine = on ? (uint32_t)((bh - 1) / rows_of(bw) + 1) : 0u;
         uint32_t inc = mine;

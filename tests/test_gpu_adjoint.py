@@ -216,3 +216,25 @@ def test_few_large_footprints_are_shared_out(env):
 
     fwd = best(lambda: rg.project_forward(ctx, gs, geom, img))
     assert best(lambda: rg.project_backward(ctx, gs, geom, w, *outs)) < 5.0 * fwd
+
+
+def test_footprint_of_more_than_2_31_pixels(env):
+    """One isotropic Gaussian over a detector whose pixels an int does not count:
+    dL/drho is the weighted sum of the closed form at the few weighted pixels."""
+    torch, rg, ctx = env
+    side, sigma, pitch = 46_400, 1.0, 1e-4
+    geom = rg.Geometry(ctx, synth.geom_parallel(1, side, side, pitch, pitch, -40.0, 40.0))
+    f = dict(dtype=torch.float32, device="cuda")
+    gs = rg.Gaussians(ctx, torch.zeros((1, 3), **f), torch.zeros((1, 3), **f),
+                      torch.tensor([[1.0, 0.0, 0.0, 0.0]], **f), torch.ones(1, **f))
+    rng = np.random.default_rng(62)
+    row, col = rng.integers(0, side, (2, 500))
+    wt = rng.uniform(0.5, 1.5, 500)
+    w = torch.zeros(side * side, **f)
+    w[torch.from_numpy(row * side + col).cuda()] = torch.from_numpy(wt).float().cuda()
+    out = torch.empty(1, **f)
+    rg.project_backward(ctx, gs, geom, w, None, None, None, out)
+    u, v = (col - 0.5 * (side - 1)) * pitch, (row - 0.5 * (side - 1)) * pitch
+    m = u * u + v * v          # a pair counts within 3 sigma of the line
+    ref = float((wt * math.sqrt(2.0 * math.pi) * sigma * np.exp(-0.5 * m))[m <= 9.0].sum())
+    assert abs(float(out) - ref) < 1e-4 * ref
