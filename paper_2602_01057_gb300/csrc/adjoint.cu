@@ -69,12 +69,12 @@ __device__ __forceinline__ float profile(float arg)
     return ex2_approx(arg);
 }
 
-// the Gaussian's cut acts on x (dL/dI or what is made of it), so that an
-// infinite or NaN dL/dI outside the cut adds nothing
+// the cut (the end of the support) acts on x -- dL/dI or what is made of it --,
+// so that an infinite or NaN dL/dI outside it adds nothing
 template <int KER>
 __device__ __forceinline__ float cut(float arg, float x)
 {
-    return KER == 1 || arg >= CUT_ARG ? x : 0.0f;
+    return (KER == 1 ? arg > -1.0f : arg >= CUT_ARG) ? x : 0.0f;
 }
 
 struct Box {

@@ -182,7 +182,7 @@ __device__ __forceinline__ void adjoint_tile(const DevGeom &g, uint32_t tile, ui
                         // 1.5 w rA iA sqrt(c) / kappa^2, dL/dA / alpha = w rA iA sqrt(c) (1.5 - 2c)
                         const float c = 1.0f + arg;
                         const float sc = c > 0.0f ? sqrt_approx(c) : 0.0f;
-                        const float t = gl_row[i] * rA * sc;
+                        const float t = (c > 0.0f ? gl_row[i] : 0.0f) * rA * sc;
                         wv = t * c;
                         h = (1.5f / Kern<1>::KAPPA2) * t * iA;
                         gA = t * iA * (1.5f - 2.0f * c);
@@ -262,12 +262,14 @@ __device__ __forceinline__ void adjoint_tile(const DevGeom &g, uint32_t tile, ui
                     const f2 q = mul2(fma2(fma2(Cvv, vt, LQ), vt, KQ), IA);
                     float q0, q1, e0, e1;
                     up(q, q0, q1);
+                    // the cut acts on g: an infinite or NaN g outside it adds nothing
                     if (KER == 1) {
                         const float x0 = 1.0f + q0, x1 = 1.0f + q1;
+                        g0 = x0 > 0.0f ? g0 : 0.0f;
+                        g1 = x1 > 0.0f ? g1 : 0.0f;
                         e0 = x0 > 0.0f ? sqrt_approx(x0) : 0.0f;
                         e1 = x1 > 0.0f ? sqrt_approx(x1) : 0.0f;
                     } else {
-                        // the cut acts on g: an infinite or NaN g outside it adds nothing
                         g0 = q0 >= CUT_ARG ? g0 : 0.0f;
                         g1 = q1 >= CUT_ARG ? g1 : 0.0f;
                         e0 = ex2_approx(q0);

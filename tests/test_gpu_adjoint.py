@@ -238,3 +238,36 @@ def test_footprint_of_more_than_2_31_pixels(env):
     m = u * u + v * v          # a pair counts within 3 sigma of the line
     ref = float((wt * math.sqrt(2.0 * math.pi) * sigma * np.exp(-0.5 * m))[m <= 9.0].sum())
     assert abs(float(out) - ref) < 1e-4 * ref
+
+
+@pytest.mark.parametrize("bad", [math.nan, math.inf])
+@pytest.mark.parametrize("walk", ["direct", "staged"])
+@pytest.mark.parametrize("name", [n for n in MASKED if n != "ring_tof"])
+def test_non_finite_weight_outside_the_support_adds_nothing(env, name, walk, bad):
+    """The same for the Epanechnikov kernel, a NaN or infinite dL/dI where no
+    support reaches: one Gaussian, and (staged) one among 40,000 far smaller.
+    The sums are of the same terms; 1e-5 as above."""
+    torch, rg, ctx = env
+    s, gd = MASKED[name]()
+    n = 1
+    G = {"mu": np.array([[0.4 * s, -0.3 * s, 0.2 * s]]), "ls": np.log([[s, 0.5 * s, 0.7 * s]]),
+         "q": np.array([[0.9, 0.1, -0.3, 0.2]]), "rho": np.ones(1)}
+    if walk == "staged":
+        n, rng = 40_000, np.random.default_rng(63)
+        G["mu"] = np.concatenate([G["mu"], rng.uniform(-s, s, (n - 1, 3))])
+        G["ls"] = np.concatenate([G["ls"], np.full((n - 1, 3), math.log(0.02 * s))])
+        G["q"] = np.concatenate([G["q"], rng.normal(size=(n - 1, 4))])
+        G["rho"] = np.ones(n)
+    geom = rg.Geometry(ctx, gd)
+    gs = rg.Gaussians(ctx, *[torch.from_numpy(G[k]).float().cuda() for k in ("mu", "ls", "q", "rho")])
+    gs.set_kernel("epanechnikov")
+    img = rg.project_forward(ctx, gs, geom, torch.empty(geom.n_rays, device="cuda"))
+    empty = img.reshape(-1) == 0.0
+    assert 0 < int(empty.sum()) < empty.numel()
+    w = torch.from_numpy(synth.random_weights(geom.n_rays, 6)).cuda().reshape(-1)
+    res = []
+    for fill in (0.0, bad):
+        outs = [torch.empty(sh, device="cuda") for sh in ((n, 3), (n, 3), (n, 4), (n,))]
+        rg.project_backward(ctx, gs, geom, torch.where(empty, torch.full_like(w, fill), w), *outs)
+        res.append(torch.cat([o.reshape(-1) for o in outs]).double().cpu())
+    assert torch.linalg.norm(res[1] - res[0]) <= 1e-5 * torch.linalg.norm(res[0])
