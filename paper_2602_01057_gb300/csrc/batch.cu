@@ -68,6 +68,7 @@ struct BatchScan {
     uint2 *rect = nullptr;      // pixel boxes [E] (a large scan: the shared scratch)
     uint32_t *order = nullptr;  // spatial order [N]
     int64_t keys = 0;           // planned tile entries
+    unsigned long long *total = nullptr;   // the step's tile entries, on the device
     float *I = nullptr, *dLdI = nullptr;
     float4 *grad = nullptr;
     float *gflat = nullptr;
@@ -91,7 +92,7 @@ struct Lane {
              *vals_alt = nullptr, *sort_tmp = nullptr;
     uint2 *rect = nullptr;
     void *order_tmp = nullptr;
-    unsigned long long *stmp = nullptr, *total = nullptr;
+    unsigned long long *stmp = nullptr;
 };
 
 // Small scans are binned on LANES streams of the captured graph: one scan's
@@ -157,7 +158,7 @@ void free_plan(rgrt_batch *b)
         l.cnt = l.off = l.keys = l.keys_alt = l.vals_alt = l.sort_tmp = nullptr;
         l.rect = nullptr;
         l.order_tmp = nullptr;
-        l.stmp = l.total = nullptr;
+        l.stmp = nullptr;
     }
     b->n_lanes = 1;
     b->d_desc = nullptr;
@@ -180,7 +181,7 @@ size_t lane_bytes(const Need &n)
 {
     return sizeof(uint32_t) * (2 * (size_t)n.E + 3 * (size_t)n.cap + sort_tmp_elems(n.cap, n.views)) +
            sizeof(uint2) * (size_t)n.E + (n.order ? order_tmp_bytes(n.N) : 0) +
-           sizeof(unsigned long long) * (scan_tmp_elems(n.E) + 2);
+           sizeof(unsigned long long) * scan_tmp_elems(n.E);
 }
 
 int alloc_count(rgrt_batch *b, Lane &l, const Need &n)
@@ -190,7 +191,6 @@ int alloc_count(rgrt_batch *b, Lane &l, const Need &n)
     BTRY(balloc(b, (void **)&l.rect, sizeof(uint2) * n.E));
     if (n.order) BTRY(balloc(b, &l.order_tmp, order_tmp_bytes(n.N)));
     BTRY(balloc(b, (void **)&l.stmp, sizeof(unsigned long long) * scan_tmp_elems(n.E)));
-    BTRY(balloc(b, (void **)&l.total, sizeof(unsigned long long) * 2));
     return RGRT_OK;
 }
 
@@ -216,6 +216,9 @@ int plan(rgrt_batch *b)
         all.N = std::max<int64_t>(all.N, x.N);
     }
     BTRY(alloc_count(b, l0, all));
+    unsigned long long *totals = nullptr;
+    BTRY(balloc(b, (void **)&totals, sizeof(unsigned long long) * b->n));
+    for (int i = 0; i < b->n; i++) b->sc[i].total = totals + i;
     b->grid_f = persistent_grid(b->cone, b->tile_w * b->tile_h);
     int n_small = 0;
     b->keys_capacity = 0;
@@ -225,15 +228,16 @@ int plan(rgrt_batch *b)
         dg.v0 = 0;
         BK(launch_records(x.g->mu, x.g->ls, x.g->q, x.g->rho, x.N, x.g->rec, x.g->crec, nullptr, s));
         BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, l0.cnt, l0.rect, s));
-        BK(launch_scan(l0.cnt, l0.off, x.E, l0.total, l0.stmp, s));
+        BK(launch_scan(l0.cnt, l0.off, x.E, x.total, l0.stmp, s));
         unsigned long long K = 0;
-        BK(cudaMemcpyAsync(&K, l0.total, sizeof(K), cudaMemcpyDeviceToHost, s));
+        BK(cudaMemcpyAsync(&K, x.total, sizeof(K), cudaMemcpyDeviceToHost, s));
         BK(cudaStreamSynchronize(s));
         unsigned long long cap = K + K / 4 + 4096;
         if (cap >= 0xffffffffull) return report_error(RGRT_E_CAPACITY, "a scan of the batch has more than 2^32 tile entries");
         x.cap = (uint32_t)cap;
         x.keys = (int64_t)K;
-        x.large = (int64_t)x.T >= 16 * (int64_t)b->grid_f;
+        // (large scans' launches are fixed: with that many tiles a list has one part)
+        x.large = (int64_t)x.T >= std::max(16 * (int64_t)b->grid_f, FORWARD_SPLIT_CTAS);
         if (!b->cone) {
             if (!x.large) BTRY(balloc(b, (void **)&x.rect, sizeof(uint2) * (size_t)std::max<int64_t>(x.E, 1)));
             BTRY(balloc(b, (void **)&x.order, sizeof(uint32_t) * (size_t)std::max<int64_t>(x.N, 1)));
@@ -306,7 +310,7 @@ int plan(rgrt_batch *b)
         d.grad = x.grad;
         d.item_begin = (uint32_t)items;
         d.n_items = x.T;
-        d.parts = forward_parts(x.T, x.keys);   // as a projection of its own would
+        d.entries = x.total;
         items += x.T;
     }
     if (items >= 0xffffffffull) return report_error(RGRT_E_CAPACITY, "too many tiles in the batch");
@@ -347,7 +351,7 @@ int enqueue_bin_scan(rgrt_batch *b, int i)
         dg.v0 = 0;
         BK(launch_records(x.g->mu, x.g->ls, x.g->q, x.g->rho, x.N, x.g->rec, x.g->crec, nullptr, s));
         BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, l.cnt, x.rect, s));
-        BK(launch_scan(l.cnt, l.off, x.E, l.total, l.stmp, s));
+        BK(launch_scan(l.cnt, l.off, x.E, x.total, l.stmp, s));
         // the scan's total (on the device) is the number of keys this step
         // emits: the sort and the ranges take only those (at most the planned
         // capacity; an item past it writes padding keys, which sort last and
@@ -356,12 +360,12 @@ int enqueue_bin_scan(rgrt_batch *b, int i)
                        b->d_overflow, s, x.lbits));
         if (x.lbits >= 0)
             BK(launch_sort_views(l.keys, x.vals, l.keys_alt, l.vals_alt, x.cap, x.bits, l.off, x.N,
-                                 dg.n_views, l.sort_tmp, s, nullptr, l.total, sort_shift(dg)));
+                                 dg.n_views, l.sort_tmp, s, nullptr, x.total, sort_shift(dg)));
         else
             BK(launch_sort(l.keys, x.vals, l.keys_alt, l.vals_alt, x.cap, x.bits, l.sort_tmp, s, nullptr,
-                           l.total, sort_shift(dg)));
+                           x.total, sort_shift(dg)));
         BK(cudaMemsetAsync(x.ranges, 0, sizeof(uint2) * (size_t)x.T, s));
-        BK(launch_ranges(l.keys, x.cap, x.ranges, x.T, s, l.total, (uint32_t)x.geom->tiles_per_view,
+        BK(launch_ranges(l.keys, x.cap, x.ranges, x.T, s, x.total, (uint32_t)x.geom->tiles_per_view,
                          x.lbits));
     }
     return RGRT_OK;

@@ -20,7 +20,7 @@
 // beam 50,000 Gaussians, 180 x 256^2 8.5 -> 6.3 ms; PET ring 200,000, 288 x
 // 329 x 63 8.2 -> 5.7 ms; fully 3-D PET (the pair shares its column's slope
 // terms) 79 -> 62 ms; time of flight 4.05 -> 3.3 ms before the lists were
-// shared (SPLIT_CTAS).
+// shared (forward_parts).
 //
 // The closed form (Eqs. 7-11) for a ray and one Gaussian is
 //   rho sqrt(2 pi / A) exp(-m/2),  A = d^T P d,  m = C - B^2/A,
@@ -66,14 +66,13 @@ constexpr int FBS = 128;            // most threads of a CTA (two rays each)
 // memory so that two buffers fit 6 to 8 CTAs per SM.
 constexpr int NBUF = 2;
 // A tile's list is shared by 2, 4 or 8 CTAs of a cluster while the launch has
-// fewer CTAs than SPLIT_CTAS (about 9 waves: tile lists are uneven, and a few
+// fewer CTAs than FORWARD_SPLIT_CTAS (about 9 waves: tile lists are uneven, and a few
 // waves leave most of the SMs waiting for the longest) and a CTA's share of an
-// average list stays above SPLIT_LIST records.  Measured without and with it:
+// average list stays above FORWARD_SPLIT_LIST records.  Measured without and with it:
 // 672 tiles of 2,700 records (8 raw PET angles) 0.46 -> 0.165 ms, 2,016 tiles
 // (time of flight, 24 angles) 3.4 -> 2.0, 2,048 of 1,270 (8 cone-beam views)
 // 0.55 -> 0.37, 256 of 350 (parallel beam) 0.080 -> 0.036; at 24,000 tiles
 // (PET ring) 5.7 either way, so those keep one CTA.
-constexpr int64_t SPLIT_CTAS = 8192, SPLIT_LIST = 128;
 
 // A lane's two rays: neighbouring columns of one row, or (3-D PET, whose ray
 // slope is a column's) neighbouring rows of one column.  The lanes of a group
@@ -627,8 +626,10 @@ __global__ void __launch_bounds__(FBS, CONE ? 6 : 7) k_forward_persistent(const 
     int scan;
     while (next_item(d, nscan, total, queue, item, scan)) {
         const ScanDesc &sd = d[scan];
-        forward_tile<CONE ? GM_CONE : GM_PARALLEL, false, 0, false, true>(sd.g, item - sd.item_begin, 0, sd.parts, sd.rec, sd.crec, sd.gids, sd.ranges,
-                                  sd.out, nullptr);
+        // the parts that a projection of the scan's own would take now
+        forward_tile<CONE ? GM_CONE : GM_PARALLEL, false, 0, false, true>(
+            sd.g, item - sd.item_begin, 0, forward_parts(sd.n_items, (int64_t)*sd.entries), sd.rec, sd.crec, sd.gids,
+            sd.ranges, sd.out, nullptr);
     }
 }
 
@@ -654,13 +655,6 @@ int persistent_grid(bool cone, int tile_rays)
 {
     const int bs = forward_threads(tile_rays);
     return cone ? grid_for(k_forward_persistent<true>, bs) : grid_for(k_forward_persistent<false>, bs);
-}
-
-uint32_t forward_parts(int64_t tiles, int64_t entries)
-{
-    uint32_t parts = 1;
-    while (parts < 8 && tiles * parts < SPLIT_CTAS && entries / (tiles * parts) >= SPLIT_LIST) parts *= 2;
-    return parts;
 }
 
 cudaError_t launch_forward(const DevGeom &g, int nv, int64_t entries, const float4 *rec, const float4 *crec,

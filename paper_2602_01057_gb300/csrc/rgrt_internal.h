@@ -149,8 +149,16 @@ cudaError_t launch_sort_views(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt
                               const unsigned long long *n_dev = nullptr, int shift = 0);
 
 // ker: kernel of the primitives (RGRT_KERNEL_GAUSSIAN / RGRT_KERNEL_EPANECHNIKOV)
-// parts that a tile's list of a launch is cut into, from its tiles and entries
-uint32_t forward_parts(int64_t tiles, int64_t entries);
+// Parts that a tile's list of a launch is cut into, from its tiles and entries:
+// 2, 4 or 8 while the launch has fewer CTAs than FORWARD_SPLIT_CTAS and a
+// part of an average list stays above FORWARD_SPLIT_LIST records (project.cu).
+constexpr int64_t FORWARD_SPLIT_CTAS = 8192, FORWARD_SPLIT_LIST = 128;
+__host__ __device__ inline uint32_t forward_parts(int64_t tiles, int64_t entries)
+{
+    uint32_t parts = 1;
+    while (parts < 8 && tiles * parts < FORWARD_SPLIT_CTAS && entries >= FORWARD_SPLIT_LIST * tiles * parts) parts *= 2;
+    return parts;
+}
 // entries: (tile, Gaussian) entries of the views
 cudaError_t launch_forward(const DevGeom &g, int nv, int64_t entries, const float4 *rec, const float4 *crec,
                            const uint32_t *gids, const uint2 *ranges, float *out, Stats *stats,
@@ -183,7 +191,7 @@ struct ScanDesc {
     float4 *grad;           // adjoint accumulator
     uint32_t item_begin;    // first (scan, tile) work item of the scan
     uint32_t n_items;       // tiles of the scan
-    uint32_t parts;         // of every tile's list (forward_parts)
+    const unsigned long long *entries;   // tile entries of the scan's present lists
 };
 // persistent integration (adjoint: cone beam) over every tile of a batch of
 // scans; the queue counter must be zero at launch.  tile_rays = tile_w * tile_h of every scan.

@@ -241,3 +241,26 @@ def test_batch_bins_scans_side_by_side(env, kind, shared):
             ref = rg.project_forward(ctx, g, geom, torch.empty(geom.n_rays, device="cuda"))
             torch.cuda.synchronize()
             assert torch.equal(o, ref)
+
+
+def test_batch_projection_follows_moved_gaussians(env):
+    """A scan's lists are cut into as many parts as a projection of its own cuts
+    them, also after its Gaussians have shrunk or grown across the rule's
+    thresholds since the batch was planned: bit for bit at every size."""
+    torch, rg, ctx = env
+    gd = synth.geom_parallel(6, 64, 64, 2.0 / 64, 2.0 / 64, -4.0, 4.0)
+    G = synth.gaussians_uniform(2500, 71, log_sigma=math.log(0.09))
+    g, geom = rg.Gaussians(ctx, *_dev(torch, G)), rg.Geometry(ctx, gd)
+    small = rg.Gaussians(ctx, *_dev(torch, synth.gaussians_uniform(50, 72)))
+    b = rg.Batch(ctx, [g, small], [geom, geom])
+    outs = [torch.empty(geom.n_rays, device="cuda") for _ in range(2)]
+    lists = set()
+    for shrink in (0.0, 0.7, 1.4, 2.1, 0.3):
+        g.set(ls=torch.from_numpy(G["ls"] - np.float32(shrink)).cuda())
+        b.forward(outs)
+        ref = rg.project_forward(ctx, g, geom, torch.empty(geom.n_rays, device="cuda"))
+        start, _ = b.debug_tile_lists(0)
+        lists.add(int(math.log2(start[-1] / (start.size - 1))))
+        torch.cuda.synchronize()
+        assert torch.equal(outs[0], ref), shrink
+    assert lists == {7, 8, 9}     # 2, 4 and 8 parts: average lists from 128, 256 and 512 entries
