@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
     const int sl = lane & (S - 1), sw = lane >> LG;
     const int64_t slot = ((int64_t)blockIdx.x * NW + w) * gw + lane;
     const bool active = lane < gw && slot < n;
-    const uint32_t gid = active ? __ldg(order + slot) : 0u;
+    const uint32_t gid = !active ? 0u : order ? __ldg(order + slot) : (uint32_t)slot;
     const int va = blockIdx.y * vper, vb = min(nv, va + vper);
     const int nb = TOF ? g.n_tof : 1;
 #pragma unroll

@@ -8,7 +8,8 @@
 // taken from an atomic counter (uneven scans fill the GPU together instead of
 // leaving it under-filled one by one), then their losses and the adjoint: ONE
 // persistent launch (cone beam, from the tile lists), or one per scan (parallel
-// rays, from the boxes).  The parameter chains and the Adam updates of every scan
+// rays, from the boxes, which are taken again: kept from the binning they would
+// hold 8 bytes per view and Gaussian of every scan).  The parameter chains and the Adam updates of every scan
 // come last.  The whole step is captured once in a CUDA graph and replayed,
 // so a step costs one graph launch and one small read-back (losses and the
 // key-capacity overflow flag) instead of a host round trip per scan.
@@ -19,8 +20,8 @@
 // entries no longer fit, the emit kernel raises the overflow flag, every Adam
 // update of that step is skipped on the device, and the host re-plans,
 // re-captures and repeats the step.  Only the sorted Gaussian ids and tile ranges of a scan
-// are kept per scan (parallel rays: the boxes as well); counts, keys and sort
-// buffers are scratch of a stream, sized for the largest of its scans.
+// are kept per scan; counts, boxes, keys and sort buffers are scratch of a
+// stream, sized for the largest of its scans.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -65,8 +66,6 @@ struct BatchScan {
     int lane = 0;               // the stream and scratch it is binned with
     uint32_t *vals = nullptr;   // sorted Gaussian ids [cap]
     uint2 *ranges = nullptr;    // [T]
-    uint2 *rect = nullptr;      // pixel boxes [E] (a large scan: the shared scratch)
-    uint32_t *order = nullptr;  // spatial order [N]
     int64_t keys = 0;           // planned tile entries
     unsigned long long *total = nullptr;   // the step's tile entries, on the device
     float *I = nullptr, *dLdI = nullptr;
@@ -91,7 +90,7 @@ struct Lane {
     uint32_t *cnt = nullptr, *off = nullptr, *keys = nullptr, *keys_alt = nullptr,
              *vals_alt = nullptr, *sort_tmp = nullptr;
     uint2 *rect = nullptr;
-    void *order_tmp = nullptr;
+    size_t key_bytes = 0;       // of keys
     unsigned long long *stmp = nullptr;
 };
 
@@ -151,13 +150,12 @@ void free_plan(rgrt_batch *b)
     for (auto &a : b->allocs) ctx_free(b->ctx, a.first, a.second);
     b->allocs.clear();
     for (auto &s : b->sc) {
-        s.vals = nullptr; s.ranges = nullptr; s.rect = nullptr; s.order = nullptr; s.I = s.dLdI = nullptr;
+        s.vals = nullptr; s.ranges = nullptr; s.I = s.dLdI = nullptr;
         s.grad = nullptr; s.gflat = nullptr; s.partial = nullptr;
     }
     for (Lane &l : b->lane) {
         l.cnt = l.off = l.keys = l.keys_alt = l.vals_alt = l.sort_tmp = nullptr;
         l.rect = nullptr;
-        l.order_tmp = nullptr;
         l.stmp = nullptr;
     }
     b->n_lanes = 1;
@@ -171,17 +169,15 @@ void free_plan(rgrt_batch *b)
 
 // A lane's scratch: E (view, Gaussian) pairs and cap keys of one scan at a time.
 struct Need {
-    int64_t E = 1, N = 1;
+    int64_t E = 1;
     uint32_t cap = 1;
     int views = 0;
-    bool order = false;
 };
 
 size_t lane_bytes(const Need &n)
 {
     return sizeof(uint32_t) * (2 * (size_t)n.E + 3 * (size_t)n.cap + sort_tmp_elems(n.cap, n.views)) +
-           sizeof(uint2) * (size_t)n.E + (n.order ? order_tmp_bytes(n.N) : 0) +
-           sizeof(unsigned long long) * scan_tmp_elems(n.E);
+           sizeof(uint2) * (size_t)n.E + sizeof(unsigned long long) * scan_tmp_elems(n.E);
 }
 
 int alloc_count(rgrt_batch *b, Lane &l, const Need &n)
@@ -189,14 +185,14 @@ int alloc_count(rgrt_batch *b, Lane &l, const Need &n)
     BTRY(balloc(b, (void **)&l.cnt, sizeof(uint32_t) * n.E));
     BTRY(balloc(b, (void **)&l.off, sizeof(uint32_t) * n.E));
     BTRY(balloc(b, (void **)&l.rect, sizeof(uint2) * n.E));
-    if (n.order) BTRY(balloc(b, &l.order_tmp, order_tmp_bytes(n.N)));
     BTRY(balloc(b, (void **)&l.stmp, sizeof(unsigned long long) * scan_tmp_elems(n.E)));
     return RGRT_OK;
 }
 
 int alloc_keys(rgrt_batch *b, Lane &l, const Need &n)
 {
-    BTRY(balloc(b, (void **)&l.keys, sizeof(uint32_t) * n.cap));
+    l.key_bytes = sizeof(uint32_t) * n.cap;
+    BTRY(balloc(b, (void **)&l.keys, l.key_bytes));
     BTRY(balloc(b, (void **)&l.keys_alt, sizeof(uint32_t) * n.cap));
     BTRY(balloc(b, (void **)&l.vals_alt, sizeof(uint32_t) * n.cap));
     BTRY(balloc(b, (void **)&l.sort_tmp, sizeof(uint32_t) * sort_tmp_elems(n.cap, n.views)));
@@ -210,11 +206,7 @@ int plan(rgrt_batch *b)
     cudaStream_t s = b->stream;
     Lane &l0 = b->lane[0];
     Need all, small;   // of every scan, of the small ones
-    all.order = small.order = !b->cone;
-    for (auto &x : b->sc) {
-        all.E = std::max<int64_t>(all.E, x.E);
-        all.N = std::max<int64_t>(all.N, x.N);
-    }
+    for (auto &x : b->sc) all.E = std::max<int64_t>(all.E, x.E);
     BTRY(alloc_count(b, l0, all));
     unsigned long long *totals = nullptr;
     BTRY(balloc(b, (void **)&totals, sizeof(unsigned long long) * b->n));
@@ -238,15 +230,10 @@ int plan(rgrt_batch *b)
         x.keys = (int64_t)K;
         // (large scans' launches are fixed: with that many tiles a list has one part)
         x.large = (int64_t)x.T >= std::max(16 * (int64_t)b->grid_f, FORWARD_SPLIT_CTAS);
-        if (!b->cone) {
-            if (!x.large) BTRY(balloc(b, (void **)&x.rect, sizeof(uint2) * (size_t)std::max<int64_t>(x.E, 1)));
-            BTRY(balloc(b, (void **)&x.order, sizeof(uint32_t) * (size_t)std::max<int64_t>(x.N, 1)));
-        }
         if (!x.large) n_small++;
         for (Need *n : { &all, &small }) {
             if (n == &small && x.large) continue;
             n->E = std::max<int64_t>(n->E, x.E);
-            n->N = std::max<int64_t>(n->N, x.N);
             n->cap = std::max(n->cap, x.cap);
             if (x.lbits >= 0) n->views = std::max(n->views, x.geom->dg.n_views);
         }
@@ -267,7 +254,10 @@ int plan(rgrt_batch *b)
     BTRY(balloc(b, (void **)&b->d_loss, sizeof(float) * b->n));
     BTRY(balloc(b, (void **)&b->d_bc, sizeof(float) * 2));
     // the other lanes are a convenience: as many as the bound and the memory allow
-    const size_t each = lane_bytes(small), left = b->ctx->budget - std::min(b->ctx->budget, b->ctx->used);
+    // (what the sets' Adam moments are still to take is not theirs)
+    size_t taken = b->ctx->used;
+    for (auto &x : b->sc) taken += x.g->adam_m ? 0 : sizeof(float) * 22 * (size_t)x.N;
+    const size_t each = lane_bytes(small), left = b->ctx->budget - std::min(b->ctx->budget, taken);
     const size_t most = std::min(LANE_BYTES, left / 16);
     while (b->distinct && b->n_lanes < LANES && b->n_lanes < n_small && each * b->n_lanes <= most) {
         Lane &l = b->lane[b->n_lanes];
@@ -281,10 +271,7 @@ int plan(rgrt_batch *b)
         b->n_lanes++;
     }
     int turn = 0;
-    for (auto &x : b->sc) {
-        x.lane = x.large ? 0 : turn++ % b->n_lanes;
-        if (!x.rect) x.rect = b->lane[x.lane].rect;
-    }
+    for (auto &x : b->sc) x.lane = x.large ? 0 : turn++ % b->n_lanes;
     // A scan whose tiles fill the GPU for 16 waves or more gains nothing from
     // sharing the persistent launches: it is binned, projected, and its loss
     // and adjoint taken back to back with launches of its own, while its
@@ -350,13 +337,13 @@ int enqueue_bin_scan(rgrt_batch *b, int i)
         DevGeom dg = x.geom->dg;
         dg.v0 = 0;
         BK(launch_records(x.g->mu, x.g->ls, x.g->q, x.g->rho, x.N, x.g->rec, x.g->crec, nullptr, s));
-        BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, l.cnt, x.rect, s));
+        BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, l.cnt, l.rect, s));
         BK(launch_scan(l.cnt, l.off, x.E, x.total, l.stmp, s));
         // the scan's total (on the device) is the number of keys this step
         // emits: the sort and the ranges take only those (at most the planned
         // capacity; an item past it writes padding keys, which sort last and
         // map to no tile, and raises the overflow flag)
-        BK(launch_emit(dg, dg.n_views, x.N, l.cnt, l.off, x.rect, l.keys, x.vals, x.cap,
+        BK(launch_emit(dg, dg.n_views, x.N, l.cnt, l.off, l.rect, l.keys, x.vals, x.cap,
                        b->d_overflow, s, x.lbits));
         if (x.lbits >= 0)
             BK(launch_sort_views(l.keys, x.vals, l.keys_alt, l.vals_alt, x.cap, x.bits, l.off, x.N,
@@ -409,7 +396,10 @@ int enqueue_loss(rgrt_batch *b, int i, const float *const *y, int loss, const rg
 }
 
 // adjoint of scan i by launches of its own: parallel rays (from its boxes) and
-// large cone-beam scans (from its tile lists)
+// large cone-beam scans (from its tile lists).  The lane's binning scratch is
+// free by then: a small scan's boxes are taken again (a large one's are still
+// there), the order goes to the offsets and its scratch to the keys (none is
+// taken where they are too small for it).
 int enqueue_adjoint(rgrt_batch *b, int i, cudaStream_t s)
 {
     BatchScan &x = b->sc[i];
@@ -420,9 +410,14 @@ int enqueue_adjoint(rgrt_batch *b, int i, cudaStream_t s)
                                 RGRT_KERNEL_GAUSSIAN, s));
         return RGRT_OK;
     }
-    if (adjoint_staged(dg, dg.n_views, x.N, x.keys))
-        BK(launch_order(x.g->crec, x.N, b->lane[x.lane].order_tmp, x.order, s));
-    BK(launch_adjoint(dg, dg.n_views, x.N, x.keys, true, x.order, x.g->rec, x.g->crec, x.rect, x.dLdI, x.grad,
+    Lane &l = b->lane[x.lane];
+    if (!x.large) BK(launch_cull(dg, dg.n_views, x.g->crec, x.N, l.cnt, l.rect, s));
+    uint32_t *order = nullptr;
+    if (adjoint_staged(dg, dg.n_views, x.N, x.keys) && order_tmp_bytes(x.N) <= l.key_bytes) {
+        order = l.off;
+        BK(launch_order(x.g->crec, x.N, l.keys, order, s));
+    }
+    BK(launch_adjoint(dg, dg.n_views, x.N, x.keys, true, order, x.g->rec, x.g->crec, l.rect, x.dLdI, x.grad,
                       RGRT_KERNEL_GAUSSIAN, s));
     return RGRT_OK;
 }

@@ -170,7 +170,8 @@ cudaError_t launch_order(const float4 *crec, int64_t n, void *tmp, uint32_t *ord
 // adjoint of parallel-ray views v0 .. v0 + nv - 1: rect = k_cull's pixel boxes
 // of those views, entries = their (tile, Gaussian) entries (the footprints' size),
 // large = some box may exceed ADJOINT_LARGE_PX pixels.  adjoint_staged: the
-// launch reads the order.
+// launch reads the order (null: Gaussians as they are numbered, which costs time
+// only).
 constexpr int ADJOINT_LARGE_PX = 2048;
 bool adjoint_staged(const DevGeom &g, int nv, int64_t n, int64_t entries);
 cudaError_t launch_adjoint(const DevGeom &g, int nv, int64_t n, int64_t entries, bool large, const uint32_t *order,

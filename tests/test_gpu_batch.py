@@ -264,3 +264,39 @@ def test_batch_projection_follows_moved_gaussians(env):
         torch.cuda.synchronize()
         assert torch.equal(outs[0], ref), shrink
     assert lists == {7, 8, 9}     # 2, 4 and 8 parts: average lists from 128, 256 and 512 entries
+
+
+def test_parallel_batch_needs_no_scratch_per_scan(env):
+    """A batch of parallel-beam scans keeps a scan's ids, ranges, images and
+    gradients, and binning scratch for one scan at a time: a budget for these
+    admits it, and its steps are those of a batch with room to spare (the terms
+    of a sum in another order: within 1e-4 of a step's size)."""
+    torch, rg, ctx = env
+    n, N, V, side = 6, 40_000, 30, 64
+    gd = synth.geom_parallel(V, side, side, 2.0 / side, 2.0 / side, -4.0, 4.0)
+    sets = [synth.gaussians_uniform(N, 80 + i, log_sigma=math.log(0.012)) for i in range(n)]
+    y = [torch.rand(V * side * side, device="cuda") for _ in range(n)]
+
+    def steps(budget):
+        c = rg.Context(0, budget)
+        gs = [rg.Gaussians(c, *_dev(torch, G)) for G in sets]
+        geom = rg.Geometry(c, gd)
+        b = rg.Batch(c, gs, [geom] * n)
+        cap = b.info()["key_capacity"]
+        loss = [b.loss_step(y, t=t) for t in (1, 2)]
+        out = [g.numpy() for g in gs]
+        b.close()
+        c.close()
+        return cap, loss, out
+
+    cap, loss, out = steps(0)
+    E, T, R = N * V, V * (side // 16) ** 2, V * side * side
+    per_scan = 4 * cap / n + 8 * T + 8 * R + (64 + 44) * N            # ids, ranges, image and dL/dI, gradients
+    sets_bytes = (44 + 80 + 48 + 88) * N                               # parameters, records, Adam moments
+    shared = 16 * E + 13 * 1.1 * cap / n                               # one scan's binning
+    _, loss2, out2 = steps(int(1.03 * (n * (per_scan + sets_bytes) + shared)) + (1 << 20))
+    for a, b in zip(loss, loss2):
+        np.testing.assert_allclose(a, b, rtol=1e-5)
+    for a, b, g in zip(out, out2, sets):
+        for k in a:
+            assert np.linalg.norm(a[k] - b[k]) <= 1e-4 * np.linalg.norm(a[k] - g[k]), k
