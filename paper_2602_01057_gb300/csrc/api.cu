@@ -59,13 +59,38 @@ int fail(int code, const char *fmt, ...)
 
 namespace {
 
+void release(rgrt_ctx *c, Buf &b)
+{
+    if (b.p) {
+        cudaFree(b.p);
+        c->used -= b.bytes;
+    }
+    b.p = nullptr;
+    b.bytes = 0;
+}
+
+// The adjoint's spatial order only saves time: its scratch gives way where the
+// budget is short (cudaFree waits for the kernels that read it).
+bool drop_order(rgrt_ctx *c)
+{
+    const bool held = c->order.p || c->order_tmp.p;
+    release(c, c->order);
+    release(c, c->order_tmp);
+    return held;
+}
+
 int dev_alloc(rgrt_ctx *c, void **p, size_t bytes)
 {
     if (bytes == 0) bytes = 16;
+    if (c->used + bytes > c->budget) drop_order(c);
     if (c->used + bytes > c->budget)
         return fail(RGRT_E_NOMEM, "allocation of %zu bytes exceeds the HBM budget (%zu of %zu used)",
                     bytes, c->used, c->budget);
     cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess && drop_order(c)) {
+        cudaGetLastError();
+        e = cudaMalloc(p, bytes);
+    }
     if (e != cudaSuccess) return fail(RGRT_E_NOMEM, "cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
     c->used += bytes;
     return RGRT_OK;
@@ -92,16 +117,6 @@ int ensure(rgrt_ctx *c, Buf &b, size_t bytes)
     TRY(dev_alloc(c, &b.p, want));
     b.bytes = want;
     return RGRT_OK;
-}
-
-void release(rgrt_ctx *c, Buf &b)
-{
-    if (b.p) {
-        cudaFree(b.p);
-        c->used -= b.bytes;
-    }
-    b.p = nullptr;
-    b.bytes = 0;
 }
 
 bool is_device_ptr(const void *p)
@@ -259,7 +274,9 @@ int bin_views(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, int v0,
     size_t need = 4 * sizeof(uint32_t) * (size_t)K + sizeof(uint32_t) * sort_tmp_elems((uint32_t)K, nseg);
     size_t have = ctx->keys.bytes + ctx->vals.bytes + ctx->keys_alt.bytes + ctx->vals_alt.bytes +
                   ctx->sort_tmp.bytes;
-    if (need > have && ctx->used - have + need + need / 8 > ctx->budget)
+    auto over = [&]() { return need > have && ctx->used - have + need + need / 8 > ctx->budget; };
+    if (over()) drop_order(ctx);
+    if (over())
         return fail(RGRT_E_CAPACITY, "views %d..%d produce %llu tile entries, over the budget", v0,
                     v0 + nv, K);
     TRY(ensure(ctx, ctx->keys, sizeof(uint32_t) * (size_t)K));
@@ -397,9 +414,10 @@ int for_ray_ranges(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, cu
     ctx->h_cnt.resize(TL);
     CK(cudaMemcpyAsync(ctx->h_cnt.data(), ctx->cnt.p, sizeof(uint32_t) * TL, cudaMemcpyDeviceToHost, s));
     TRY(read_totals(ctx, s, nullptr));
-    // list capacity: what the budget leaves (the current list buffer included)
+    // list capacity: what the budget leaves (the current list buffer and what
+    // gives way included)
     size_t avail = ctx->budget > ctx->used ? ctx->budget - ctx->used : 0;
-    avail += ctx->vals.bytes;
+    avail += ctx->vals.bytes + ctx->order.bytes + ctx->order_tmp.bytes;
     avail = avail > ((size_t)1 << 20) ? avail - ((size_t)1 << 20) : 0;
     uint64_t cap = avail / sizeof(uint32_t);
     if (cap > 0x7fffffffull) cap = 0x7fffffffull;
@@ -505,11 +523,18 @@ int run_forward(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, float
     });
 }
 
-// the Gaussians' spatial order, for the adjoint of parallel rays
+// the Gaussians' spatial order, for the adjoint of parallel rays; none (order
+// released) where memory is short
 int build_order(rgrt_ctx *ctx, const rgrt_gauss *g, cudaStream_t s)
 {
-    TRY(ensure(ctx, ctx->order, sizeof(uint32_t) * (size_t)g->n));
-    TRY(ensure(ctx, ctx->order_tmp, order_tmp_bytes(g->n)));
+    const size_t a = sizeof(uint32_t) * (size_t)g->n, b = order_tmp_bytes(g->n);
+    const size_t others = ctx->used - ctx->order.bytes - ctx->order_tmp.bytes;
+    if (others + a + b + (a + b) / 8 + 512 > ctx->budget || ensure(ctx, ctx->order, a) != RGRT_OK ||
+        ensure(ctx, ctx->order_tmp, b) != RGRT_OK || !ctx->order.p) {
+        cudaGetLastError();
+        drop_order(ctx);
+        return RGRT_OK;
+    }
     PROF("k_order");
     CK(launch_order(g->crec, g->n, ctx->order_tmp.p, (uint32_t *)ctx->order.p, s));
     return RGRT_OK;

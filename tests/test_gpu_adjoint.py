@@ -271,3 +271,37 @@ def test_non_finite_weight_outside_the_support_adds_nothing(env, name, walk, bad
         rg.project_backward(ctx, gs, geom, torch.where(empty, torch.full_like(w, fill), w), *outs)
         res.append(torch.cat([o.reshape(-1) for o in outs]).double().cpu())
     assert torch.linalg.norm(res[1] - res[0]) <= 1e-5 * torch.linalg.norm(res[0])
+
+
+def test_order_gives_way_to_the_budget(env):
+    """The staged walk's spatial order is left out where the memory budget has no
+    room for it: a budget for the set, one view's binning and the gradient
+    accumulator admits the call, and the gradient is the same (sums in another
+    order, 2e-6 as above).  Scratch is taken an eighth larger than asked."""
+    torch, rg, ctx = env
+    N, side = 400_000, 128
+    gd = _parallel(1, side, side, 0.015)
+    G = _sizes(N, 64, L(0.01))
+    w = torch.rand(side * side, device="cuda")
+
+    def grads(budget, keys=False):
+        c = rg.Context(0, budget)
+        gs = rg.Gaussians(c, *[torch.from_numpy(np.ascontiguousarray(G[k])).cuda() for k in ("mu", "ls", "q", "rho")])
+        geom = rg.Geometry(c, gd)
+        outs = [torch.empty(s, device="cuda") for s in ((N, 3), (N, 3), (N, 4), (N, 1))]
+        c.prof_enable(True)
+        rg.project_backward(c, gs, geom, w, *outs)
+        ordered = c.prof_get("k_order")[0]
+        K = rg.debug_tile_lists(c, gs, geom)[1].size if keys else 0
+        gs.close()
+        geom.close()
+        c.close()
+        return [o.double() for o in outs], ordered, K
+
+    ref, ordered, K = grads(0, True)
+    assert ordered == 1
+    own = (44 + 80 + 48) * N + 1.125 * (16 * N + 64 * N + 17 * K)     # set; counts, boxes, accumulator, keys
+    got, ordered, _ = grads(int(1.01 * own) + (1 << 20))
+    assert ordered == 0
+    for a, b in zip(got, ref):
+        assert float(torch.linalg.norm(a - b) / torch.linalg.norm(b)) < 2e-6
