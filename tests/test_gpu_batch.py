@@ -300,3 +300,73 @@ def test_parallel_batch_needs_no_scratch_per_scan(env):
     for a, b, g in zip(out, out2, sets):
         for k in a:
             assert np.linalg.norm(a[k] - b[k]) <= 1e-4 * np.linalg.norm(a[k] - g[k]), k
+
+
+def _parallel(v, side):
+    return synth.geom_parallel(v, side, side, 2.0 / side, 2.0 / side, -4.0, 4.0)
+
+
+def test_parallel_batch_steps_match_single_scans(env):
+    """Optimisation steps of parallel-ray scans: more small ones than streams, of
+    uneven sizes, both walks of the adjoint (few pairs in place; 17,001 Gaussians
+    staged, with the order's scratch), a large scan among them and a ring.
+    Losses and parameters follow the scans' own steps as far as the cone beam's
+    do above: 1e-5 of a loss, 1e-3 of a parameter's way."""
+    torch, rg, ctx = env
+    scans = [(synth.gaussians_uniform(n, 90 + i, log_sigma=math.log(s)), gd) for i, (n, s, gd) in enumerate([
+        (300, 0.06, _parallel(5, 33)), (17_001, 0.02, _parallel(4, 64)), (1, 0.2, _parallel(2, 16)),
+        (2_500, 0.03, _parallel(90, 256)), (900, 0.05, _parallel(9, 48)), (40_000, 0.015, _parallel(9, 64)),
+        (33, 0.1, _parallel(1, 80))])]
+    ring = synth.gaussians_uniform(5_000, 98, half_box=120.0, log_sigma=math.log(5.0))
+    scans.append((ring, synth.geom_pet(12, 129, 21, 400.0, 288, 9.0)))
+    hp = rg.adam_params()
+    geoms = [rg.Geometry(ctx, gd) for _, gd in scans]
+    ys = []
+    for (G, gd), geom in zip(scans, geoms):
+        gt = rg.Gaussians(ctx, *_dev(torch, synth.perturbed(G, 7, pos_std=0.01)))
+        ys.append(rg.project_forward(ctx, gt, geom, torch.empty(geom.n_rays, device="cuda")))
+    gb = [rg.Gaussians(ctx, *_dev(torch, G)) for G, _ in scans]
+    own = [rg.Gaussians(ctx, *_dev(torch, G)) for G, _ in scans]
+    b = rg.Batch(ctx, gb, geoms)
+    assert b.info()["work_items"] > 16_000          # the large scan's tiles among them
+    for t in (1, 2, 3):
+        lb = b.loss_step(ys, rg.RGRT_LOSS_L2, hp, t)
+        for i, (g, geom, y) in enumerate(zip(own, geoms, ys)):
+            ls = np.zeros(1, np.float32)
+            rg.loss_step(ctx, g, geom, y, rg.RGRT_LOSS_L2, hp, t, ls)
+            assert lb[i] == pytest.approx(float(ls[0]), rel=1e-5, abs=1e-12), (t, i)
+    for i, (G, _) in enumerate(scans):
+        a, c = gb[i].numpy(), own[i].numpy()
+        for k in a:
+            d = np.linalg.norm((a[k].astype(np.float64) - c[k]).ravel())
+            assert d <= 1e-3 * np.linalg.norm((c[k].astype(np.float64) - G[k]).ravel()), (i, k)
+
+
+@pytest.mark.parametrize("kind", ["parallel", "cone"])
+def test_step_of_scans_that_share_a_set(env, kind):
+    """Two scans of one set in a batch: both gradients are taken at the step's
+    start, then Adam is applied for one scan after the other (the two updates
+    recomputed in binary64 from the scans' own gradients; 1e-3 of the way)."""
+    torch, rg, ctx = env
+    gds = [_parallel(5, 48), _parallel(3, 64)] if kind == "parallel" else \
+        [synth.geom_cone(v, s, s, 4.0 / s, 4.0 / s, 4.0, 8.0) for v, s in ((5, 48), (3, 64))]
+    G = synth.gaussians_uniform(700, 99, log_sigma=math.log(0.06))
+    geoms = [rg.Geometry(ctx, gd) for gd in gds]
+    gt = rg.Gaussians(ctx, *_dev(torch, synth.perturbed(G, 8, pos_std=0.01)))
+    ys = [rg.project_forward(ctx, gt, q, torch.empty(q.n_rays, device="cuda")) for q in geoms]
+    hp = rg.adam_params()
+    g = rg.Gaussians(ctx, *_dev(torch, G))
+    grads = []
+    for geom, y in zip(geoms, ys):
+        o = {k: torch.empty(G[k].shape, device="cuda") for k in G}
+        rg.loss_grad(ctx, g, geom, y, rg.RGRT_LOSS_L2, hp, None, o["mu"], o["ls"], o["q"], o["rho"])
+        grads.append({k: v.double().cpu().numpy() for k, v in o.items()})
+    rg.Batch(ctx, [g, g], geoms).loss_step(ys, rg.RGRT_LOSS_L2, hp, 1)
+    got = g.numpy()
+    for k, lr in (("mu", hp.lr_mu), ("ls", hp.lr_logscale), ("q", hp.lr_quat), ("rho", hp.lr_rho)):
+        p, m, v = G[k].astype(np.float64), 0.0, 0.0
+        for d in grads:
+            m = hp.beta1 * m + (1.0 - hp.beta1) * d[k]
+            v = hp.beta2 * v + (1.0 - hp.beta2) * d[k] ** 2
+            p = p - lr / (1.0 - hp.beta1) * m / (np.sqrt(v / (1.0 - hp.beta2)) + hp.eps)
+        assert np.linalg.norm(got[k] - p) <= 1e-3 * np.linalg.norm(p - G[k]), k
