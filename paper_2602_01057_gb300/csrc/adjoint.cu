@@ -23,7 +23,7 @@
 // lanes that wait for a longer chord of the same round).  Against one Gaussian
 // per thread and tile (record gathers, box searches, a chain and 16 atomics
 // for each of the 1.9 tiles of a PET footprint), measured on a GB300: PET ring
-// of 288 x 329 x 63, 200,000 Gaussians 9.6 -> 6.9 ms; 8 raw angles, 100,000
+// of 288 x 329 x 63, 200,000 Gaussians 9.6 -> 6.8 ms; 8 raw angles, 100,000
 // 0.73 -> 0.14 ms; 24 angles x 13 time-of-flight bins 4.96 -> 2.83 ms; parallel
 // beam, 1,000 Gaussians on 16 x 64^2 0.34 -> 0.07 ms (that one had 256 CTAs of
 // serial pixels).  Sorting a warp's Gaussians by box area per view took the
@@ -57,34 +57,37 @@ template <> struct Fac<1> {
     static constexpr float FQ = 1.5f / 7.0f, FP = -2.0f;
 };
 
-// the kernel's profile of a pair: e^{-m/2} (Gaussian), sqrt(c) inside the
-// support (Epanechnikov, c = 1 + arg)
-template <int KER>
-__device__ __forceinline__ float profile(float arg)
-{
-    if (KER == 1) {
-        const float c = 1.0f + arg;
-        return c > 0.0f ? sqrt_approx(c) : 0.0f;
-    }
-    return ex2_approx(arg);
-}
-
-// the cut (the end of the support) acts on x -- dL/dI or what is made of it --,
-// so that an infinite or NaN dL/dI outside it adds nothing
-template <int KER>
+// the Gaussian's cut acts on x (dL/dI or what is made of it), so that an
+// infinite or NaN dL/dI outside the cut adds nothing
 __device__ __forceinline__ float cut(float arg, float x)
 {
-    return (KER == 1 ? arg > -1.0f : arg >= CUT_ARG) ? x : 0.0f;
+    return arg >= CUT_ARG ? x : 0.0f;
+}
+
+// dL/dI times the kernel's profile, of two pixels: g e^{-m/2} (Gaussian), g sqrt(c)
+// inside the support (Epanechnikov, c = 1 + arg); 0 outside the cut or support,
+// whatever g is
+template <int KER>
+__device__ __forceinline__ f2 weighted(float a0, float a1, float2 g)
+{
+    if (KER == 1) {
+        float x, y;
+        up(mul2(pk(g.x, g.y), pk(sqrt_approx(1.0f + a0), sqrt_approx(1.0f + a1))), x, y);
+        return pk(a0 > -1.0f ? x : 0.0f, a1 > -1.0f ? y : 0.0f);
+    }
+    return mul2(pk(cut(a0, g.x), cut(a1, g.y)), pk(ex2_approx(a0), ex2_approx(a1)));
 }
 
 struct Box {
     int ilo, ihi, jlo, jhi;
 };
 
-// pixels of a box, at most 2^26 (a detector of 65,536 x 65,536 has 2^32)
+// Pixels of a box, its sides taken as 16,384 at most (a detector of 65,536 x 65,536
+// has 2^32): exact where it is compared with the limits of the two walks, and
+// it only orders the larger ones.
 __device__ __forceinline__ int box_px(int w, int h)
 {
-    return (int)min((long long)w * h, 1ll << 26);
+    return min(w, 16384) * min(h, 16384);
 }
 
 // a staged band: columns [cb, cb + w), rows [rb, rb + h), row stride st
@@ -187,7 +190,7 @@ __device__ __forceinline__ void rows(const DevGeom &g, const float4 &c0, const f
             const f2 q = fma2(fma2(Muu, du, A1), du, A0);
             float qx, qy;
             up(q, qx, qy);
-            const f2 h = mul2(pk(cut<KER>(qx, gg.x), cut<KER>(qy, gg.y)), pk(profile<KER>(qx), profile<KER>(qy)));
+            const f2 h = weighted<KER>(qx, qy, gg);
             const f2 hd = mul2(h, du);
             h0 = add2(h0, h);
             h1 = add2(h1, hd);
@@ -252,7 +255,7 @@ __device__ __forceinline__ void rows_tof(const DevGeom &g, const float4 &c0, con
             i += Src::STEP;
             const float du0 = uu.x - u0, du1 = uu.y - u0;
             const float q0 = fmaf(fmaf(c0.z, du0, a1), du0, a0), q1 = fmaf(fmaf(c0.z, du1, a1), du1, a0);
-            const float e0 = profile<0>(q0), e1 = profile<0>(q1);
+            const float e0 = ex2_approx(q0), e1 = ex2_approx(q1);
             const float tb = t4.x + t4.z * dv - g.tof_t0;
             const f2 ts = pk(tb + t4.y * du0, tb + t4.y * du1);
             f2 Ge = 0, D1 = 0, D2 = 0, nb = 0;      // nb: minus the bin
@@ -276,9 +279,9 @@ __device__ __forceinline__ void rows_tof(const DevGeom &g, const float4 &c0, con
                 up(D1, d10, d11);
                 up(D2, d20, d21);
                 const float du = k ? du1 : du0, e = k ? e1 : e0, q = k ? q1 : q0;
-                const float ge = cut<0>(q, k ? G1 : G0) * nrm;
-                const float v1 = e * (cut<0>(q, k ? d11 : d10) * (-nrm * is2));     // val sum g_k dW_k/dt*
-                const float v2 = e * (0.5f * is2 * (nrm * is2 * cut<0>(q, k ? d21 : d20) - ge));   // val sum g_k dW_k/ds^2
+                const float ge = cut(q, k ? G1 : G0) * nrm;
+                const float v1 = e * (cut(q, k ? d11 : d10) * (-nrm * is2));     // val sum g_k dW_k/dt*
+                const float v2 = e * (0.5f * is2 * (nrm * is2 * cut(q, k ? d21 : d20) - ge));   // val sum g_k dW_k/ds^2
                 const float h = ge * e, hd = h * du;
                 m[0] += h;
                 m[1] += hd;
@@ -365,6 +368,29 @@ __device__ __noinline__ void general_box(const DevGeom &g, int view, const float
     }
     for (int q = 0; q < NG; q++)
         for (int o = 16; o > 0; o >>= 1) val[q] += __shfl_xor_sync(0xffffffffu, val[q], o);
+}
+
+// The warp's Gaussians that meet a band, of the n first that lane k's turn names:
+// their number << 8 | the one of this lane (0 past them).
+__device__ __forceinline__ uint32_t band_list(const int2 *box, uint8_t *list, int turn, int n, Band bd)
+{
+    const int lane = threadIdx.x & 31;
+    const int2 b = box[turn];
+    const bool on = lane < n && (b.x & 0xffff) < bd.cb + bd.w && (int)((unsigned)b.x >> 16) >= bd.cb &&
+                    (b.y & 0xffff) < bd.rb + bd.h && (int)((unsigned)b.y >> 16) >= bd.rb;
+    const uint32_t bal = __ballot_sync(0xffffffffu, on);
+    if (on) list[__popc(bal & ((1u << lane) - 1u))] = (uint8_t)turn;
+    const uint32_t num = (uint32_t)__popc(bal);
+    __syncwarp();
+    return num << 8 | (lane < (int)num ? list[lane] : 0u);
+}
+
+// Without time of flight a view is mostly one band, and the list out of line
+// leaves the walk its registers (PET ring 6.99 -> 6.77 ms; 13 bins, several bands
+// a view, 2.83 -> 3.03).
+__device__ __noinline__ uint32_t band_list_call(const int2 *box, uint8_t *list, int turn, int n, Band bd)
+{
+    return band_list(box, list, turn, n, bd);
 }
 
 // views staged by the CTA and its warps' records and moments
@@ -467,8 +493,8 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
         }
         const int n_vs = __popc(__ballot_sync(0xffffffffu, vis && !gen));
         Band bd;
-        bd.st = min(BW, (ub.y - ub.x + 2) & ~1);
-        const bool many = ub.y - ub.x >= BW || ub.w - ub.z >= min(BH, Cap<TOF>::v / (bd.st * nb));
+        const int uw = ub.y - ub.x + 1, uh = ub.w - ub.z + 1;
+        const bool many = uw > BW || uh > BH || uh * ((uw + 1) & ~1) * nb > Cap<TOF>::v;
         for (bd.cb = ub.x; bd.cb <= ub.y; bd.cb += BW) {
             bd.w = min(BW, ub.y - bd.cb + 1);
             bd.st = (bd.w + 1) & ~1;
@@ -479,14 +505,11 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
                 if (many) {
                     // several bands: the Gaussians that meet this one, and no
                     // staging where there is none
-                    const int2 b = sh.box[wb + turn];
-                    const bool on = lane < n_vs && (b.x & 0xffff) < bd.cb + bd.w && (int)((unsigned)b.x >> 16) >= bd.cb &&
-                                    (b.y & 0xffff) < bd.rb + bd.h && (int)((unsigned)b.y >> 16) >= bd.rb;
-                    const uint32_t bal = __ballot_sync(0xffffffffu, on);
-                    if (on) sh.list[w][__popc(bal & ((1u << lane) - 1u))] = (uint8_t)turn;
-                    n_now = __popc(bal);
+                    const uint32_t r = TOF ? band_list(sh.box + wb, sh.list[w], turn, n_vs, bd)
+                                           : band_list_call(sh.box + wb, sh.list[w], turn, n_vs, bd);
+                    n_now = (int)(r >> 8);
                     if (!__syncthreads_or(n_now)) continue;     // (also: every warp is done with the band before)
-                    now = lane < n_now ? sh.list[w][lane] : 0;
+                    now = (int)(r & 255u);
                 }
                 // stage dL/dI of the band, a warp taking 1, 2 or 4 rows at a time
                 for (int i = threadIdx.x; i < bd.st; i += BS)
@@ -974,7 +997,8 @@ cudaError_t launch_order(const float4 *crec, int64_t n, void *tmp, uint32_t *ord
     cudaError_t e = cudaMemsetAsync(cells, 0, sizeof(uint32_t) * (CELLS + 6), s);
     if (e != cudaSuccess) return e;
     const unsigned nb = (unsigned)((n + 255) / 256);
-    k_order_box<<<nb < 152u ? nb : 152u, 256, 0, s>>>(crec, n, box);
+    const unsigned sms = (unsigned)sm_count();
+    k_order_box<<<nb < sms ? nb : sms, 256, 0, s>>>(crec, n, box);
     k_order_cells<<<nb, 256, 0, s>>>(crec, n, bits, box, cells, where);
     k_order_scan<<<1, SMALL_BS, 0, s>>>(cells);
     k_order_scatter<<<nb, 256, 0, s>>>(n, cells, where, order);
@@ -998,11 +1022,12 @@ void adjoint_staged_launch(double px, int max_px, const DevGeom &g, int nv, int6
                            const float4 *rec, const float4 *crec, const uint2 *rect, const float *dLdI, float4 *grad,
                            cudaStream_t s)
 {
-    // Gaussians per warp: fewer where 32 would leave the GPU short of CTAs
+    // Gaussians per warp: fewer where 32 would leave the GPU short of CTAs (10 per SM)
+    const int64_t sms = sm_count();
     int gw = 32;
-    while (gw > 2 && (n / (gw * NW)) * nv < 152 * 10) gw >>= 1;
+    while (gw > 2 && (n / (gw * NW)) * nv < sms * 10) gw >>= 1;
     const int64_t bx = (n + NW * gw - 1) / (NW * gw);
-    int64_t chunks = (152 * 5 * 12 + bx - 1) / bx;
+    int64_t chunks = (sms * 5 * 12 + bx - 1) / bx;
     if (chunks > nv) chunks = nv;
     if (chunks > 65535) chunks = 65535;
     const int vper = (int)((nv + chunks - 1) / chunks);
@@ -1024,15 +1049,15 @@ void adjoint_direct_launch(double px, int min_px, const DevGeom &g, int nv, int6
 {
     // CTAs for a few waves, each looking through the boxes of several views; where
     // the Gaussians are too few for that, several share a set's strips
-    const int64_t bx = (n + BS - 1) / BS;
-    int64_t by = (152 * 48 + bx - 1) / bx;
+    const int64_t sms = sm_count(), bx = (n + BS - 1) / BS;
+    int64_t by = (sms * 48 + bx - 1) / bx;
     if (by > nv) by = nv;
     if (by > 65535) by = 65535;
     // strips for about 64 warps per SM
-    const double pairs = (double)n * (double)nv, strip = px * pairs / (152 * 64.0);
+    const double pairs = (double)n * (double)nv, strip = px * pairs / (64.0 * (double)sms);
     const int strip_px = strip < 256.0 ? 256 : strip > 4096.0 ? 4096 : (int)strip;
     const double most = pairs * (1.0 + px / strip_px) / (double)(bx * by * NW * 4);   // four strips a warp
-    int64_t z = 152 * 40 / (bx * by);
+    int64_t z = sms * 40 / (bx * by);
     if (z > (int64_t)most) z = (int64_t)most;
     z = z < 1 ? 1 : z;
     const dim3 grid((unsigned)bx, (unsigned)by, (unsigned)z);
@@ -1065,9 +1090,11 @@ cudaError_t launch_adjoint(const DevGeom &g, int nv, int64_t n, int64_t entries,
     // after band of its CTA's union.  2,048 px: 50,000 Gaussians of 50 px and 100
     // of 10^4 px on 90 x 256^2 11.5 -> 4.4 ms, log-sizes with a deviation of 1.0
     // 4.9 -> 3.0 (1,024 px 2.9, 4,096 3.0), a PET ring with 0.7 15.3 -> 14.5;
-    // where the average is itself larger, four times that (20,000 of 5,900 px:
-    // 12.8 ms at 2,048 px, 10.6 at 8,192).
-    const int max_px = !staged ? 0 : px > ADJOINT_LARGE_PX ? 4 * ADJOINT_LARGE_PX : ADJOINT_LARGE_PX;
+    // where the average is itself larger, up to four times that, eight times
+    // (20,000 of 5,900 px: 12.8 ms at 2,048 px, 10.0 at 8,192, 8.9 at 16,384; of
+    // 23,000 px 4.3, 4.3 and 4.7).
+    const bool alike = px > ADJOINT_LARGE_PX && px <= 4 * ADJOINT_LARGE_PX;
+    const int max_px = !staged ? 0 : alike ? 8 * ADJOINT_LARGE_PX : ADJOINT_LARGE_PX;
 #define RGRT_ADJ(K, T)                                                                                          \
     {                                                                                                           \
         if (staged) adjoint_staged_launch<K, T>(px, max_px, g, nv, n, order, rec, crec, rect, dLdI, grad, s);   \

@@ -273,9 +273,10 @@ __global__ void k_cull(DevGeom g, int nv, const float4 *__restrict__ crec, int64
             const int j0 = lower_idx_g(g.vtab, g.n_rows, vlo, g.v0f, g.vinv);
             const int j1 = upper_idx_g(g.vtab, g.n_rows, vhi, g.v0f, g.vinv);
             cull_write(g, i0, i1, j0, j1, cnt + (int64_t)vf * n + k, rect + (int64_t)vf * n + k);
-            if (GM == GM_PARALLEL && large && i0 <= i1 && j0 <= j1 &&
-                (int64_t)(i1 - i0 + 1) * (j1 - j0 + 1) > ADJOINT_LARGE_PX)
-                *large = 1u;
+            if (GM == GM_PARALLEL) {
+                const unsigned a = i1 - i0, b = j1 - j0;   // (a + 1) (b + 1) pixels
+                if (i0 <= i1 && j0 <= j1 && a * b + a + b >= (unsigned)ADJOINT_LARGE_PX && large) *large = 1u;
+            }
             continue;
         }
         // 3-D PET: the LOR of radial position s and mid-height z has

@@ -517,15 +517,21 @@ __device__ __forceinline__ bool next_item(const ScanDesc *d, int nscan, uint32_t
     return item < total;
 }
 
+int sm_count()
+{
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n < 1 ? 1 : n;
+}
+
 // CTAs of a persistent launch: SMs x resident CTAs per SM
 template <class K>
 int grid_for(K kernel, int threads)
 {
-    int dev = 0, nsm = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    int per = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0);
-    return nsm * (per < 1 ? 1 : per);
+    return sm_count() * (per < 1 ? 1 : per);
 }
 
 }  // namespace
