@@ -316,9 +316,10 @@ __device__ __forceinline__ void finish(const float *m, float iA, float rA, float
 
 // Sum the N moments over sub-warps of 2^LG lanes, transposed (each halving of
 // the sub-warp also halves the values a lane keeps), and add this lane's sums
-// to out[0..N).
+// to out[0..N) (on, the same over a sub-warp: not where it has no Gaussian of its
+// own, whose out may be another sub-warp's).
 template <int N, int LG>
-__device__ __forceinline__ void reduce_add(float *v, int sl, float *out)
+__device__ __forceinline__ void reduce_add(float *v, int sl, float *out, bool on = true)
 {
     constexpr int H1 = (N + 1) / 2, H2 = (H1 + 1) / 2, H3 = (H2 + 1) / 2, H4 = (H3 + 1) / 2, H5 = (H4 + 1) / 2;
     constexpr int HN[6] = { N, H1, H2, H3, H4, H5 };
@@ -331,7 +332,7 @@ __device__ __forceinline__ void reduce_add(float *v, int sl, float *out)
     constexpr int LAST = HN[LG];
 #pragma unroll
     for (int q = 0; q < LAST; q++)
-        if (q < len) out[p + q] += v[q];
+        if (on && q < len) out[p + q] += v[q];
 }
 
 // A Gaussian near a segment end, in world coordinates: the warp shares the
@@ -552,7 +553,7 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
                     if constexpr (TOF) rows_tof(g, c0, c1, sh.t4[wb + k], bx, l, 1 << L, src, m);
                     else rows<KER>(g, c0, c1, bx, l, 1 << L, src, m);
                     __syncwarp();
-                    reduce_add<NM, L>(m, l, sh.mom + (wb + k) * NM);
+                    reduce_add<NM, L>(m, l, sh.mom + (wb + k) * NM, on);
                 };
                 __syncwarp();
                 {
