@@ -241,7 +241,11 @@ int geometry_set_corrections(rgrt_geom *g, const float *mult, const float *add);
 /* ---- projector (Eqs. 4, 11, 12) ------------------------------------- */
 
 /* out_I[geometry_num_rays] = sum over Gaussians of rho sqrt(2 pi/A)
- * exp(-m/2) Phi, Phi the erf factor of the finite segment.  Overwrites. */
+ * exp(-m/2) Phi, Phi the erf factor of the finite segment.  Overwrites.
+ * Repeated calls give the same bits.  A ray's sum is grouped by the parts that
+ * its tile's list is cut into, and these follow the tiles and list entries of
+ * the launch: the same views projected with others, or in other chunks (a smaller
+ * memory budget), may differ in the last bits. */
 int project_forward(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, float *out_I,
                     void *stream);
 
@@ -309,13 +313,15 @@ int rgrt_batch_destroy(rgrt_batch *b);
  * GPU for 16 waves; a larger scan is projected right after its binning by a
  * launch of its own.  Captured once in a CUDA graph and replayed).  out_I[i] receives scan i's projection (host or device; null
  * skips it).  Re-plans and repeats when the parameters have moved so far that
- * a scan's tile entries no longer fit.  Synchronises with `stream`. */
+ * a scan's tile entries no longer fit.  A scan's projection equals
+ * project_forward's bit for bit where that takes the scan's views in one chunk.
+ * Synchronises with `stream`. */
 int rgrt_batch_forward(rgrt_batch *b, float *const *out_I, void *stream);
 
 /* One optimisation step of every scan, as loss_step does for one: forward,
  * loss against y[i] (device arrays), adjoint (the small scans: one persistent
  * forward launch over all of them, and one persistent adjoint launch (cone
- * beam) or one per scan; a large scan: binning, forward, loss and adjoint back
+ * beam) or the boxes and launches of each scan; a large scan: binning, forward, loss and adjoint back
  * to back, its lists still in L2),
  * then the parameter chains and Adam (step t) of every scan.  loss_out[n_scans] (host or
  * device, may be null) receives the losses.  Captured in a CUDA graph that is

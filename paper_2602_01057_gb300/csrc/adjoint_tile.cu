@@ -1,8 +1,7 @@
 // Adjoint of the cone-beam and fully 3-D PET geometries, tile by tile (a5).
 // (Parallel rays walk Gaussian by Gaussian instead, adjoint.cu.  Measured that
 // way too, the cone beam gained little -- its footprints span several tiles,
-// so its cost is the pixels -- and 3-D PET keeps adding its thousands of views
-// to the accumulator one by one, in view order.)
+// so its cost is the pixels -- and 3-D PET nothing.)
 //
 // Adjoint, one Gaussian per thread.  A CTA takes a tile: it stages the
 // tile's dL/dI (times |d~| for cone beam) and pixel coordinates in shared

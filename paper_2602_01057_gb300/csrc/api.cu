@@ -240,7 +240,7 @@ int bin_views(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, int v0,
     DevGeom dg = geom->dg;
     dg.v0 = v0;
     const uint32_t T = (uint32_t)nv * (uint32_t)geom->tiles_per_view;
-    if (T >= (1u << 24))  // tile ids share the key with an 8-bit position code
+    if (T >= (1u << 24))  // tile ids share the key with an 8-bit order code
         return fail(RGRT_E_CAPACITY, "views %d..%d hold %u tiles (2^24 at most)", v0, v0 + nv, T);
     ctx->bin_valid = false;   // until the new lists and boxes are complete
     TRY(ensure(ctx, ctx->cnt, sizeof(uint32_t) * (size_t)E));
@@ -265,7 +265,7 @@ int bin_views(rgrt_ctx *ctx, const rgrt_gauss *g, const rgrt_geom *geom, int v0,
         return fail(RGRT_E_CAPACITY, "views %d..%d produce %llu tile entries (more than 2^32)", v0,
                     v0 + nv, K);
     // the views' keys are sorted view by view (on the tile within the view and
-    // the position code) when the padded tile field (view << lbits | tile)
+    // the order code) when the padded tile field (view << lbits | tile)
     // fits the key's 24 bits
     const uint32_t tpv = (uint32_t)geom->tiles_per_view;
     const int lbits = ceil_log2(tpv);

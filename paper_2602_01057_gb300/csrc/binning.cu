@@ -1,9 +1,10 @@
 // Binning (a2, second half): exclusive scan of per-(view, Gaussian) tile
-// counts, emission of (tile, position, Gaussian) keys, a stable LSD radix
+// counts, emission of (tile, order code, Gaussian) keys, a stable LSD radix
 // sort on the key bits, and per-tile ranges.  Keys are emitted in (view,
-// Gaussian) order and the sort is stable, so each tile's list is ordered by
-// footprint position and then by Gaussian id: the lists are canonical and the
-// per-ray sums deterministic.  Being emitted view by view, the keys are
+// Gaussian) order and the sort is stable, so each tile's list is ordered by the
+// code -- footprint position on the cone beam, box size on 3-D PET, nothing on
+// parallel rays, whose sort skips it -- and then by Gaussian id: the lists are
+// canonical.  Being emitted view by view, the keys are
 // already grouped by view: the sort then orders each view's keys on their
 // own (on the tile within the view and the order code), which takes
 // fewer 8-bit passes than sorting on the view's bits too.
@@ -205,10 +206,11 @@ __global__ void __launch_bounds__(SCAN_SMALL_BS) k_scan_small(const uint32_t *__
 }
 
 // one thread per (view of the chunk, Gaussian): write its tiles' keys.
-// key = tile id << 8 | position code, the code being the 4-bit row and
+// key = tile id << 8 | order code, the code being the 4-bit row and
 // column buckets of the centre of the Gaussian's pixel box within the tile:
-// sorting by it orders each tile's list by footprint position (Gaussians of
-// the same position keep ascending ids, the sort being stable).  3-D PET, whose
+// sorting by it orders a cone-beam tile's list by footprint position (Gaussians
+// of the same position keep ascending ids, the sort being stable; parallel rays
+// carry the code, but their sort starts above it).  3-D PET, whose
 // adjoint's lanes walk a box each, columns outer, takes the buckets of the box's
 // row and column counts within the tile instead, so that the lanes of a warp
 // have loops of one length (200,000 Gaussians, 33 million bins: adjoint 59.3 ->

@@ -3,7 +3,8 @@
 // One CTA per detector tile of tile_w x tile_h rays (or a cluster of up to 8
 // that share the tile's list), two rays per thread, a half- or quarter-warp
 // per block of 8 x 4 or 4 x 4 rays.  The tile's Gaussian list (ordered by
-// footprint position, then id) is walked in chunks: the CTA gathers each
+// footprint position on the cone beam, by box size on 3-D PET, by id alone on
+// parallel rays) is walked in chunks: the CTA gathers each
 // chunk's records, turning every Gaussian into its view-space form for this
 // view (see below) together with its detector bounding box, into one of two
 // shared-memory buffers.  A block skips a Gaussian whose box misses it, or
@@ -413,9 +414,9 @@ __device__ __forceinline__ void forward_tile(const DevGeom &g, uint32_t tile, ui
 #pragma unroll
     for (int q = 0; q < (TOF ? TOF_MAX : 1); q++) acc_t[q] = 0;
     unsigned n_eval = 0, n_kept0 = 0, n_kept1 = 0;
-    // chunk c takes list entries c, c + nch, c + 2 nch, ...: the lists are
-    // ordered by footprint position, and interleaving spreads every chunk
-    // over the whole tile, which keeps the groups' shares of it even
+    // chunk c takes list entries c, c + nch, c + 2 nch, ...: a list ordered by
+    // footprint position or size is spread over every chunk, which keeps the
+    // groups' shares of it even
     const uint32_t nlist = rg.y - rg.x;
     const uint32_t nch = ((nlist + CH - 1) / CH + parts - 1) / parts * parts;
     f2 sum = 0, gsum = 0;      // SEQ: the parts before

@@ -102,7 +102,7 @@ cudaError_t launch_records(const float *mu, const float *ls, const float *q, con
 // ADJOINT_LARGE_PX pixels
 cudaError_t launch_cull(const DevGeom &g, int nv, const float4 *crec, int64_t n, uint32_t *cnt,
                         uint2 *rect, cudaStream_t s, uint32_t *large = nullptr);
-// key = tile field << 8 | position code; lbits >= 0: the tile field is
+// key = tile field << 8 | order code; lbits >= 0: the tile field is
 // (view << lbits) | tile within the view, for launch_sort_views; lbits < 0:
 // the tile id view * tiles per view + tile
 cudaError_t launch_emit(const DevGeom &g, int nv, int64_t n, const uint32_t *cnt,
@@ -141,7 +141,7 @@ inline int sort_shift(const DevGeom &g) { return g.kind == GM_PARALLEL ? 8 : 0; 
 // The same sort, view by view: the emitted keys are grouped by view (view v's
 // keys start at off[v stride], the scan of the per-(view, Gaussian) counts),
 // and each view's keys are sorted on their own by their low `bits` bits --
-// the tile within the view and the position code, with keys emitted with
+// the tile within the view and the order code, with keys emitted with
 // lbits = bits - 8 -- which takes fewer passes than sorting on the view too.
 cudaError_t launch_sort_views(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt,
                               uint32_t n, int bits, const uint32_t *off, int64_t stride, int nv,

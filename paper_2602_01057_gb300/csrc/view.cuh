@@ -333,7 +333,7 @@ __device__ __forceinline__ void cross_acc(const float *a, const float *b, float 
 //   dL/drho = sqrt(2 pi) Sw
 // out16 = (dmu[3], drho, G_P[6], G_S[6]) in world coordinates.
 // tof4 (nullable; parallel rays with time of flight): the moments of the
-// TOF weight's derivatives (see adjoint_tile), added to dL/dmu' and dL/dP'.
+// TOF weight's derivatives (rows_tof in adjoint.cu), added to dL/dmu' and dL/dP'.
 template <int GM, int KER>
 __device__ __forceinline__ void view_chain(const DevGeom &g, const float *F, const float4 *rec,
                                            uint32_t gid, const float *s, float *out16,
