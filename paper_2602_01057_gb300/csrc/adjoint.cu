@@ -71,9 +71,8 @@ template <int KER>
 __device__ __forceinline__ f2 weighted(float a0, float a1, float2 g)
 {
     if (KER == 1) {
-        float x, y;
-        up(mul2(pk(g.x, g.y), pk(sqrt_approx(1.0f + a0), sqrt_approx(1.0f + a1))), x, y);
-        return pk(a0 > -1.0f ? x : 0.0f, a1 > -1.0f ? y : 0.0f);
+        const float x = 1.0f + a0, y = 1.0f + a1;
+        return mul2(pk(x > 0.0f ? g.x : 0.0f, y > 0.0f ? g.y : 0.0f), pk(sqrt_approx(fabsf(x)), sqrt_approx(fabsf(y))));
     }
     return mul2(pk(cut(a0, g.x), cut(a1, g.y)), pk(ex2_approx(a0), ex2_approx(a1)));
 }
@@ -387,8 +386,9 @@ __device__ __forceinline__ uint32_t band_list(const int2 *box, uint8_t *list, in
 }
 
 // Without time of flight a view is mostly one band, and the list out of line
-// leaves the walk its registers (PET ring 6.99 -> 6.77 ms; 13 bins, several bands
-// a view, 2.83 -> 3.03).
+// leaves the walk its registers (PET ring 6.99 -> 6.77 ms; but 13 bins, several
+// bands a view, 2.83 -> 3.03, and Epanechnikov, 20,000 on 90 x 256^2, 1.39 -> 1.42:
+// those keep it in line).
 __device__ __noinline__ uint32_t band_list_call(const int2 *box, uint8_t *list, int turn, int n, Band bd)
 {
     return band_list(box, list, turn, n, bd);
@@ -506,8 +506,8 @@ __global__ void __launch_bounds__(BS, TOF ? 5 : 6) k_adjoint(DevGeom g, int nv, 
                 if (many) {
                     // several bands: the Gaussians that meet this one, and no
                     // staging where there is none
-                    const uint32_t r = TOF ? band_list(sh.box + wb, sh.list[w], turn, n_vs, bd)
-                                           : band_list_call(sh.box + wb, sh.list[w], turn, n_vs, bd);
+                    const uint32_t r = TOF || KER == 1 ? band_list(sh.box + wb, sh.list[w], turn, n_vs, bd)
+                                                       : band_list_call(sh.box + wb, sh.list[w], turn, n_vs, bd);
                     n_now = (int)(r >> 8);
                     if (!__syncthreads_or(n_now)) continue;     // (also: every warp is done with the band before)
                     now = (int)(r & 255u);
